@@ -175,17 +175,98 @@ __global__ void k_synth_latent(const double* blobs, int nblobs, int c, int h, in
 // Multi-level security (Section 3): the private stream at a lower clearance
 // level, its least significant bits removed.  code = rint(x (2^bits - 1))
 // clamped to [0, 2^bits - 1], the `drop` low bits cleared, value
-// code / (2^bits - 1); in double precision whatever the element type.
-template <typename T>
-__global__ void k_truncate_lsb(const T* in, int64_t count, int bits, int drop, T* out) {
-  const double top = (double)((1ll << bits) - 1);
-  const long long mask = ~((1ll << drop) - 1);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const double c = fmin(fmax(rint((double)in[i] * top), 0.0), top);
-    const long long code = (long long)c & mask;
-    out[i] = (T)((double)code / top);
+// code / (2^bits - 1), as double-precision arithmetic gives it whatever the
+// element type.  In double arithmetic throughout (a product, a rounding, two
+// clamps, two conversions and a division) the kernel was bound by the double
+// units, which issue one warp instruction in ~64 cycles: 3.01 ms for 102 M
+// floats (0.27 TB/s).  The two forms below give the same bits from
+// single-precision and integer instructions; the float one is bound by memory
+// (0.138 ms for the same floats, 5.9 TB/s).
+//
+// Floats with codes of at most kTruncBitsF bits: x top = p + e exactly (FMA),
+// so rint(p) is the code unless p itself was rounded onto a half, where the
+// sign of e decides; the quotient by one multiplication and one FMA correction
+// is the correctly rounded one for every code of up to 22 bits (checked over
+// all of them), and a correctly rounded double quotient rounds to the same
+// float: it would have to lie within 2^-53 of the middle of two floats, and
+// code / (2^bits - 1) keeps 2^-(25 + bits) away from it.  Products of 2^23 and
+// above are integers beyond every code: they clamp.
+constexpr int kTruncBitsF = 22;
+constexpr int kTruncThreads = 256;
+constexpr int kTruncVec = 4;         // 16-byte groups in flight per thread
+
+struct TruncF {
+  float top, inv;
+  int mask;
+  __device__ __forceinline__ float operator()(float x) const {
+    const float p = x * top, e = fmaf(x, top, -p);
+    float r = rintf(p);
+    const float d = p - r;
+    if (d == 0.5f && e > 0.f) r += 1.f;
+    if (d == -0.5f && e < 0.f) r -= 1.f;
+    const float c = (float)((int)fminf(fmaxf(r, 0.f), top) & mask);   // NaN: code 0
+    const float q = c * inv;
+    return fmaf(fmaf(-q, top, c), inv, q);
   }
+};
+
+// Doubles, and floats with longer codes: one double product, clamped by
+// integer comparisons, rounded to an integer by adding 2^52; the quotient
+// c / (2^bits - 1) is the binary fraction 0.ccc... of the repeated code, so its
+// double is read off the repeated bit pattern (rounded by the first dropped
+// bit: the dropped tail is never exactly one half).  Two double instructions
+// an element.
+struct TruncW {
+  double top;
+  uint32_t topi, mask;
+  int bits;
+  __device__ __forceinline__ double operator()(double x) const {
+    long long v = __double_as_longlong(x * top);
+    if (v < 0 || v > 0x7ff0000000000000ll) v = 0;                      // negative or NaN: code 0
+    const long long vt = __double_as_longlong(top);
+    if (v > vt) v = vt;
+    const uint32_t c =
+        (uint32_t)__double_as_longlong(__longlong_as_double(v) + 0x1p52) & mask;
+    if (c == 0u) return 0.0;
+    if (c == topi) return 1.0;
+    const int lz = __clz(c) - (32 - bits);
+    const uint32_t cr = ((c << lz) | (lz ? c >> (bits - lz) : 0u)) & topi;   // leading bit first
+    uint64_t w = (uint64_t)cr << (64 - bits);
+    for (int s = bits; s < 64; s <<= 1) w |= w >> s;
+    const uint64_t m = ((w >> 10) + 1) >> 1;                           // 53 bits, rounded
+    return __longlong_as_double(((long long)(1022 - lz) << 52) + (long long)(m & 0xfffffffffffffull));
+  }
+};
+
+// A grid-stride pass; 16-byte groups when both buffers allow it.
+template <typename T, class Op>
+__global__ void __launch_bounds__(kTruncThreads) k_truncate_lsb(const T* in, int64_t count, Op op, T* out,
+                                                               int vec) {
+  constexpr int E = 16 / (int)sizeof(T);
+  struct alignas(16) V { T v[E]; };
+  const int64_t stride = (int64_t)gridDim.x * kTruncThreads;
+  const int64_t t0 = blockIdx.x * (int64_t)kTruncThreads + threadIdx.x;
+  int64_t done = 0;
+  if (vec) {
+    const int64_t groups = count / E;
+    const V* vi = (const V*)in;
+    V* vo = (V*)out;
+    for (int64_t g = t0; g < groups; g += kTruncVec * stride) {
+      V x[kTruncVec];
+#pragma unroll
+      for (int k = 0; k < kTruncVec; ++k)
+        if (g + k * stride < groups) x[k] = vi[g + k * stride];
+#pragma unroll
+      for (int k = 0; k < kTruncVec; ++k) {
+        if (g + k * stride >= groups) break;
+#pragma unroll
+        for (int e = 0; e < E; ++e) x[k].v[e] = (T)op(x[k].v[e]);
+        vo[g + k * stride] = x[k];
+      }
+    }
+    done = groups * E;
+  }
+  for (int64_t i = done + t0; i < count; i += stride) out[i] = (T)op(in[i]);
 }
 
 // Camera side (Section 3, "Blur Kernel Selection": new random kernels for
@@ -224,10 +305,22 @@ void launch_draw_kernels(int n, int t, int kind, int frame0, uint64_t seed, cons
 
 void launch_truncate_lsb(const void* in, int f64, int64_t count, int bits, int drop, void* out,
                          cudaStream_t st) {
-  const int64_t blocks64 = (count + 255) / 256;
-  const int blocks = (int)(blocks64 < 152 * 32 ? (blocks64 > 0 ? blocks64 : 1) : 152 * 32);
-  if (f64) k_truncate_lsb<double><<<blocks, 256, 0, st>>>((const double*)in, count, bits, drop, (double*)out);
-  else k_truncate_lsb<float><<<blocks, 256, 0, st>>>((const float*)in, count, bits, drop, (float*)out);
+  const int es = f64 ? 8 : 4;
+  const int vec = (((uintptr_t)in | (uintptr_t)out) & 15) == 0 ? 1 : 0;
+  const int64_t per = (int64_t)kTruncThreads * (vec ? 16 / es * kTruncVec : 1);
+  const int64_t want = (count + per - 1) / per;
+  const int blocks = (int)(want < 152 * 8 ? (want > 0 ? want : 1) : 152 * 8);
+  const uint32_t topi = (uint32_t)((1ull << bits) - 1), mask = topi & ~((1u << drop) - 1);
+  if (!f64 && bits <= kTruncBitsF) {
+    const TruncF op{(float)topi, 1.0f / (float)topi, (int)mask};
+    k_truncate_lsb<float><<<blocks, kTruncThreads, 0, st>>>((const float*)in, count, op, (float*)out, vec);
+    return;
+  }
+  const TruncW op{(double)topi, topi, mask, bits};
+  if (f64)
+    k_truncate_lsb<double><<<blocks, kTruncThreads, 0, st>>>((const double*)in, count, op, (double*)out, vec);
+  else
+    k_truncate_lsb<float><<<blocks, kTruncThreads, 0, st>>>((const float*)in, count, op, (float*)out, vec);
 }
 
 void launch_forward_blur(const void* latent, int n, int c, int h, int w, int f64,
