@@ -42,6 +42,7 @@ struct FoldDftArgs {
   int pz_all;              // float-float kernel: double copies of every sample, not only the real ones
   const int* accepted;     // learned path: pairs whose proposal passed the gate (skipped), or null
   int C;
+  Roots w;
 };
 
 // 8-byte bin m of a position: (hi, lo) floats (F32) or a double.
@@ -63,7 +64,10 @@ __global__ void __launch_bounds__(kDftThreads) k_fold_dft(FoldDftArgs a) {
   if (a.accepted && a.accepted[blockIdx.y / a.C]) return;   // the proposal stands (whole block)
   if (!CBP_CHECK(a.M <= kMaxM && a.ns <= a.M, 0)) return;    // the root tables' size (whole block)
   __shared__ double cs[kMaxM], sn[kMaxM];
-  for (int k = threadIdx.x; k < a.M; k += blockDim.x) sincospi(2.0 * (double)k / (double)a.M, &sn[k], &cs[k]);
+  for (int k = threadIdx.x; k < a.M; k += blockDim.x) {
+    cs[k] = a.w.c[k];
+    sn[k] = a.w.s[k];
+  }
   __syncthreads();
   const int z = blockIdx.z, fc = blockIdx.y, M = a.M, len = a.len[z];
   const int pos = blockIdx.x * blockDim.x + threadIdx.x;
@@ -134,8 +138,7 @@ __global__ void __launch_bounds__(kDftThreads, 4) k_fold_dft_ff(FoldDftArgs a) {
   if (!CBP_CHECK(a.M <= kMaxM && a.ns <= a.M, 0)) return;    // the root tables' size (whole block)
   __shared__ F2 cs[kMaxM], sn[kMaxM];
   for (int k = threadIdx.x; k < a.M; k += blockDim.x) {
-    double s, c;
-    sincospi(2.0 * (double)k / (double)a.M, &s, &c);
+    const double s = a.w.s[k], c = a.w.c[k];
     const float ch = (float)c, sh = (float)s;
     cs[k] = {ch, (float)(c - (double)ch)};
     sn[k] = {sh, (float)(s - (double)sh)};
@@ -205,6 +208,7 @@ void launch_fold_dft(const Plan& p, char* ws, cudaStream_t st) {
   a.pz_all = p.pz_all;
   a.accepted = p.learned ? (const int*)(ws + p.off_acc) : nullptr;
   a.C = p.C;
+  a.w = make_roots(p.M);
   dim3 g((maxlen + kDftThreads - 1) / kDftThreads, p.n * p.C, 4);
   // bins of float32 frames are (hi, lo) pairs; the mixed path of float32
   // frames takes the float-float kernel

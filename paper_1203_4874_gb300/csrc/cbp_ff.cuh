@@ -24,9 +24,23 @@ __device__ __forceinline__ fx fx_norm(float s, float e) {
   const float h = s + e;
   return {h, e - (h - s)};
 }
+// x split on the integer pipe: the mantissa's upper 24 bits rounded to nearest,
+// the rest as a signed integer (both conversions from integers are exact or
+// rounded once).  Two float/double conversions and a double subtraction hold
+// the double units for ~200 cycles; this takes about 60.  Outside 2^-70 ..
+// 2^120 (and for 0) the conversions.
 __device__ __forceinline__ fx fx_of(double x) {
-  const float h = (float)x;
-  return {h, (float)(x - (double)h)};
+  const long long b = __double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff) - 1023;
+  if (ex < -70 || ex > 120) {
+    const float h = (float)x;
+    return {h, (float)(x - (double)h)};
+  }
+  const long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
+  const int h = (int)((m + (1ll << 28)) >> 29), l = (int)(m - ((long long)h << 29));
+  const int sg = (int)((unsigned)(b >> 32) & 0x80000000u);
+  const float sh = __int_as_float(((ex - 23 + 127) << 23) | sg), sl = __int_as_float(((ex - 52 + 127) << 23) | sg);
+  return {(float)h * sh, (float)l * sl};
 }
 __device__ __forceinline__ double fx_val(fx a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ fx fx_add(fx a, fx b) {
@@ -45,6 +59,13 @@ __device__ __forceinline__ fx fx_scale(fx a, float s) {   // a * s, s a single-p
   return fx_norm(p, fmaf(a.hi, s, -p) + a.lo * s);
 }
 __device__ __forceinline__ fx fx_sub(fx a, fx b) { return fx_add(a, fx_neg(b)); }
+// a - m b with one renormalisation
+__device__ __forceinline__ fx fx_fnma(fx a, fx m, fx b) {
+  const float p = m.hi * b.hi;
+  const float e = fmaf(m.hi, b.lo, fmaf(m.lo, b.hi, fmaf(m.hi, b.hi, -p)));
+  const fx s = fx_two_sum(a.hi, -p);
+  return fx_norm(s.hi, s.lo + (a.lo - e));
+}
 // a / b: a single-precision quotient, corrected once by the exactly formed
 // remainder a - q b (long division with two digits)
 __device__ __forceinline__ fx fx_div(fx a, fx b) {

@@ -114,6 +114,14 @@ struct SizePlan {
   size_t total;
 };
 
+// The M-th roots of unity cos, sin (2 pi k / M), k < M, as a kernel argument:
+// their double-precision evaluation on the device (about 5000 cycles on its
+// narrow double units) would precede every small launch's real work.
+struct Roots {
+  double c[kMaxM], s[kMaxM];
+};
+const Roots& make_roots(int M);
+
 // ---- planning (cbp_plan.cpp) ----
 int next_7_smooth(int n);
 bool make_fft_plan(int n, FftPlan* p);

@@ -2,6 +2,7 @@
 // the per-call device workspace.
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include "cbp_common.cuh"
 #include "cbp_internal.h"
 
@@ -14,6 +15,34 @@ int next_7_smooth(int n) {
       while (r % p == 0) r /= p;
     if (r == 1) return k;
   }
+}
+
+// Long double arithmetic (in software on some hosts, hence kept per M: a
+// constant table of at most kMaxM entries each), folded into the first octant
+// (exact zeros and ones where they belong).
+static Roots compute_roots(int M) {
+  Roots r = {};
+  const long double pi = 3.14159265358979323846264338327950288L;
+  for (int k = 0; k < M && k < kMaxM; ++k) {
+    // angle 2 pi k / M = (pi / 2) q + (pi / 2) f, f = (4 k - q M) / M in [-1/2, 1/2]
+    const int q = (8 * k + M) / (2 * M);
+    const long double x = pi * 0.5L * (long double)(4 * k - q * M) / (long double)M;
+    const double c = (double)cosl(x), s = (double)sinl(x);
+    switch (q & 3) {
+      case 0: r.c[k] = c, r.s[k] = s; break;
+      case 1: r.c[k] = -s, r.s[k] = c; break;
+      case 2: r.c[k] = -c, r.s[k] = -s; break;
+      default: r.c[k] = s, r.s[k] = -c; break;
+    }
+  }
+  return r;
+}
+const Roots& make_roots(int M) {
+  static std::once_flag once[kMaxM + 1];
+  static Roots table[kMaxM + 1];
+  const int m = M < 1 ? 1 : M > kMaxM ? kMaxM : M;
+  std::call_once(once[m], [m] { table[m] = compute_roots(m); });
+  return table[m];
 }
 
 static uint32_t magic_div(int d) {

@@ -41,7 +41,20 @@ namespace {
 
 constexpr int kSolveThreads = 256;
 #ifndef CBP_SOLVE_WPC
-#define CBP_SOLVE_WPC 4
+#define CBP_SOLVE_WPC 4      // complex samples per CTA of the sample solve (a warp each)
+#endif
+#ifndef CBP_TEAM_CTAS
+// Up to this many samples a call, each complex one has a CTA to itself: two per
+// SM.  Mixed path: a CTA per sample takes half a warp's time for one, but four
+// warps a CTA fill the GPU's schedulers better once there are more samples than
+// that (60 1080p pairs, 540 samples a chunk: 6.45 ms against 6.48).  FP64 path:
+// the double units bound either form and the CTA's needs fewer double
+// instructions (40 pairs of 25 / 20 kernels, 520 samples a chunk: 4.44 ms
+// against 5.19; 30 480p pairs, 180 samples a chunk: 1.71 against 2.33).
+#define CBP_TEAM_CTAS 304
+#endif
+#ifndef CBP_TEAM_CTAS_F64
+#define CBP_TEAM_CTAS_F64 4096
 #endif
 
 // Optional per-phase cycle counts (build with -DCBP_PHASE_TIMING): thread 0 of
@@ -56,19 +69,6 @@ constexpr int kSolveThreads = 256;
   do {                   \
   } while (0)
 #endif
-
-// ------------------------------------------------------------ block helpers
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  v = warp_sum(v);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  double t = 0;
-  const int nw = blockDim.x >> 5;
-  for (int i = 0; i < nw; ++i) t += red[i];
-  return t;
-}
 
 // Scalar helpers so one solver serves real (float, double) and complex data.
 __device__ __forceinline__ float re_(float x) { return x; }
@@ -133,6 +133,8 @@ struct SampleArgs {
   cd* G;                     // [n][2][ns][nn][nn] normal matrices
   int Lmax, C, ns, t1, t2, nn, M, mixed;
   int nfr;                   // pairs in the call
+  int gsplit;                // CTAs a sample's lags are split over (normal matrices)
+  int wpc;                   // complex samples (warps) per CTA, when not a CTA each
 };
 
 // Sample polynomial element m of frame k (0: b1, 1: b2) as cpx<TA>.
@@ -159,13 +161,22 @@ __device__ SamplePolys<TP, TA> sample_polys(const cpx<TP>* const base[2], const 
   return P;
 }
 
+// The lags of a normal matrix are split over the CTAs of a sample where a batch
+// is too small to fill the GPU: CTA `first` of `step` takes the lags
+// j = first (mod step).
+struct LagSplit {
+  int first, step;
+  __device__ __forceinline__ bool mine(int j) const { return j % step == first; }
+};
+
 // rho jobs: j < t1: rho_22(j); j < t1+t2: rho_11(j - t1);
 // else rho_21(d), d = j - t1 - t2 - (t2 - 1) in [-(t2-1), t1-1].
 template <typename TP, typename TA>
-__device__ void correlations(const SamplePolys<TP, TA>& P, int C, int t1, int t2, cd* rho) {
+__device__ void correlations(const SamplePolys<TP, TA>& P, int C, int t1, int t2, cd* rho,
+                             LagSplit sp = {0, 1}) {
   const int J = 2 * (t1 + t2) - 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int j = warp; j < J; j += nw) {
+  for (int j = warp * sp.step + sp.first; j < J; j += nw * sp.step) {
     int ka, kb, d;
     if (j < t1) { ka = 1; kb = 1; d = j; }
     else if (j < t1 + t2) { ka = 0; kb = 0; d = j - t1; }
@@ -185,10 +196,10 @@ __device__ void correlations(const SamplePolys<TP, TA>& P, int C, int t1, int t2
 // rho jobs as above for real samples (z = 1, and z = -1 when M is even):
 // real double correlations of the real parts.
 __device__ void correlations_real(const SamplePolys<double, double>& P, int C, int t1, int t2,
-                                  cd* rho) {
+                                  cd* rho, LagSplit sp = {0, 1}) {
   const int J = 2 * (t1 + t2) - 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int j = warp; j < J; j += nw) {
+  for (int j = warp * sp.step + sp.first; j < J; j += nw * sp.step) {
     int ka, kb, d;
     if (j < t1) { ka = 1; kb = 1; d = j; }
     else if (j < t1 + t2) { ka = 0; kb = 0; d = j - t1; }
@@ -258,7 +269,8 @@ constexpr int kGramLags = 8;     // lags per warp and pass
 constexpr int kGramPre = (2 * kGramTile + kSolveThreads - 1) / kSolveThreads;
 
 __device__ void correlations_ff(const cdf* const base[2], const int len[2], int f, int C, int ns,
-                                int s, int t1, int t2, cd* rho, cdf* tile /* [2][kGramTile] */) {
+                                int s, int t1, int t2, cd* rho, cdf* tile /* [2][kGramTile] */,
+                                LagSplit sp) {
   const int J = 2 * (t1 + t2) - 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int maxlen = max(len[0], len[1]);
@@ -276,7 +288,7 @@ __device__ void correlations_ff(const cdf* const base[2], const int len[2], int 
         pre[q] = base[k][((int64_t)(f * C + ch) * ns + s) * len[k] + g];
     }
   };
-  for (int j0 = 0; j0 < J; j0 += kGramLags * nw) {     // passes over the lags
+  for (int j0 = 0; j0 * sp.step < J; j0 += kGramLags * nw) {     // passes over the lags
     FF re[kGramLags], im[kGramLags];
     cdf pre[kGramPre];
     fetch(0, pre);
@@ -291,7 +303,7 @@ __device__ void correlations_ff(const cdf* const base[2], const int len[2], int 
       if (it + 1 < iters) fetch(it + 1, pre);
 #pragma unroll
       for (int q = 0; q < kGramLags; ++q) {
-        const int j = j0 + warp + q * nw;
+        const int j = (j0 + warp + q * nw) * sp.step + sp.first;
         if (j >= J) break;
         int ka, kb, d;
         if (j < t1) { ka = 1; kb = 1; d = j; }
@@ -313,7 +325,7 @@ __device__ void correlations_ff(const cdf* const base[2], const int len[2], int 
     }
 #pragma unroll
     for (int q = 0; q < kGramLags; ++q) {
-      const int j = j0 + warp + q * nw;
+      const int j = (j0 + warp + q * nw) * sp.step + sp.first;
       const FF sr = warp_sum_ff(re[q]), si = warp_sum_ff(im[q]);
       if (j < J && lane == 0) rho[j] = mk(sr.value(), si.value());
     }
@@ -321,28 +333,35 @@ __device__ void correlations_ff(const cdf* const base[2], const int len[2], int 
   __syncthreads();
 }
 
-// G[p][q] from the correlations (Toeplitz blocks).
-__device__ void gram_from_rho(const cd* rho, int t1, int t2, cd* G) {
+// G[p][q] from the correlations (Toeplitz blocks), the entries of this CTA's lags.
+__device__ void gram_from_rho(const cd* rho, int t1, int t2, cd* G, LagSplit sp = {0, 1}) {
   const int n = t1 + t2;
   for (int i = threadIdx.x; i < n * n; i += blockDim.x) {
-    int p = i / n, q = i % n;
-    cd g;
+    const int p = i / n, q = i % n;
+    int j;            // the lag's index
+    bool cj, neg;     // its conjugate, its negative
     if (p < t1 && q < t1) {
-      int d = p - q;
-      g = d >= 0 ? rho[d] : conj(rho[-d]);
+      const int d = p - q;
+      j = abs(d);
+      cj = d < 0;
+      neg = false;
     } else if (p >= t1 && q >= t1) {
-      int d = (p - t1) - (q - t1);
-      g = d >= 0 ? rho[t1 + d] : conj(rho[t1 - d]);
+      const int d = p - q;
+      j = t1 + abs(d);
+      cj = d < 0;
+      neg = false;
     } else if (p < t1) {
-      int d = p - (q - t1);               // rho_21(d)
-      cd v = rho[t1 + t2 + d + t2 - 1];
-      g = mk(-v.re, -v.im);
+      j = t1 + t2 + (p - (q - t1)) + t2 - 1;      // rho_21(d)
+      cj = false;
+      neg = true;
     } else {
-      int d = q - (p - t1);
-      cd v = rho[t1 + t2 + d + t2 - 1];
-      g = mk(-v.re, v.im);                // -conj(rho_21(d))
+      j = t1 + t2 + (q - (p - t1)) + t2 - 1;      // -conj(rho_21(d))
+      cj = true;
+      neg = true;
     }
-    G[i] = g;
+    if (!sp.mine(j)) continue;
+    const cd v = rho[j];
+    G[i] = neg ? mk(-v.re, cj ? v.im : -v.im) : mk(v.re, cj ? -v.im : v.im);
   }
   __syncthreads();
 }
@@ -350,6 +369,7 @@ __device__ void gram_from_rho(const cd* rho, int t1, int t2, cd* G) {
 // Accurate S^H S x for the FP64 path: y = S x per channel in the global
 // scratch, then the correlations with b1, b2.
 #include "cbp_tri.cuh"
+#include "cbp_tri_team.cuh"
 
 // S^H S x from the double samples (the exact operator of the refinement
 // steps; y holds S x), by the whole CTA (BLOCK) or by the calling warp.
@@ -599,32 +619,35 @@ struct SylvesterApply {
 __global__ void __launch_bounds__(kSolveThreads) k_sample_gram(SampleArgs a) {
   __shared__ cd rho[4 * kMaxN];
   __shared__ cdf tile[2 * kGramTile];
-  const int f = blockIdx.x, ps = blockIdx.y, s = blockIdx.z;
+  const int f = blockIdx.x, ps = blockIdx.y, s = blockIdx.z / a.gsplit;
+  const LagSplit sp{(int)blockIdx.z - s * a.gsplit, a.gsplit};
   if (a.accepted && a.accepted[f]) return;   // the proposal stands; nothing to solve
   if (!CBP_CHECK(a.t1 + a.t2 <= kMaxN && s < a.ns && ps < 2, 1)) return;   // rho's size (whole block)
   // Real samples (z = 1; z = -1 when M is even) have real Gram matrices.
   const bool real = s == 0 || 2 * s == a.M;
   const SamplePolys<double, double> P64 =
       sample_polys<double, double>(a.pz[ps], a.len[ps], f, a.C, a.ns, s);
-  if (real) correlations_real(P64, a.C, a.t1, a.t2, rho);
-  else if (a.mixed) correlations_ff(a.pzf[ps], a.len[ps], f, a.C, a.ns, s, a.t1, a.t2, rho, tile);
-  else correlations(P64, a.C, a.t1, a.t2, rho);
+  if (real) correlations_real(P64, a.C, a.t1, a.t2, rho, sp);
+  else if (a.mixed) correlations_ff(a.pzf[ps], a.len[ps], f, a.C, a.ns, s, a.t1, a.t2, rho, tile, sp);
+  else correlations(P64, a.C, a.t1, a.t2, rho, sp);
   const int64_t o = ((int64_t)f * 2 + ps) * a.ns + s;
-  gram_from_rho(rho, a.t1, a.t2, a.G + o * a.nn * a.nn);
+  gram_from_rho(rho, a.t1, a.t2, a.G + o * a.nn * a.nn, sp);
 }
 
 // A3: the null vector of every sample's normal matrix (tridiagonal
 // reduction, Sturm multisection, inverse iteration, refinement steps against
 // S^H S as configured below).  The first nreal CTAs take one real sample each
 // (z = 1, and z = -1 for even M: their refinement, the costliest step, runs
-// on the whole CTA); the others take one complex sample per warp.
-__global__ void k_sample_solve(SampleArgs a, int nreal) {
+// on the whole CTA).  TEAM: the others take one complex sample each as well;
+// else one complex sample per warp.
+template <bool TEAM>
+__global__ void __launch_bounds__(kTeamThreads, 3) k_sample_solve(SampleArgs a, int nreal) {
   extern __shared__ __align__(16) char smem[];
 #ifdef CBP_SCHED_TRACE
   unsigned long long t_start;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_start));
 #endif
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpc = blockDim.x >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n = a.nn;
   const int nrs = (a.M % 2 == 0) ? 2 : 1, ncs = a.ns - nrs;   // real / complex samples per pass
   const bool real = (int)blockIdx.x < nreal;
@@ -635,17 +658,18 @@ __global__ void k_sample_solve(SampleArgs a, int nreal) {
     ps = (r / nrs) & 1;
     s = (r % nrs) ? a.M / 2 : 0;
   } else {
-    const int c = ((int)blockIdx.x - nreal) * wpc + warp;
-    if (c >= a.nfr * 2 * ncs) return;          // whole warp leaves together
+    const int b = (int)blockIdx.x - nreal, c = TEAM ? b : b * a.wpc + warp;
+    if (c >= a.nfr * 2 * ncs || (!TEAM && warp >= a.wpc)) return;   // whole warp leaves together
     f = c / (2 * ncs);
     ps = (c / ncs) & 1;
     s = 1 + c % ncs;
   }
   if (a.accepted && a.accepted[f]) return;   // the proposal stands; nothing to solve
-  // a real sample's whole CTA, or a complex sample's warp, leaves together
+  // a sample's whole CTA, or its warp, leaves together
   if (!CBP_CHECK(f < a.nfr && s < a.ns && n <= kMaxN, 2)) return;
   const int64_t o = ((int64_t)f * 2 + ps) * a.ns + s;
-  const TriWs W = carve_tri(smem + (real ? 0 : (size_t)warp * tri_ws_bytes(n)), n);
+  const bool whole = TEAM || real;             // the CTA works on this sample
+  const TriWs W = carve_tri(smem + (whole ? 0 : (size_t)warp * tri_ws_bytes(n)), n);
   const cd* G = a.G + o * n * n;
 #ifdef CBP_PHASE_TIMING
   long long tkv[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -661,9 +685,7 @@ __global__ void k_sample_solve(SampleArgs a, int nreal) {
   // leaves ~1e-4 in x), none elsewhere.
   const int far = a.mixed ? 0 : 1;
   const double gap = a.mixed ? 1e-6 : 1e-4;
-  TriResult res;
-  if (real) {
-    SylvesterApply<true> ap;
+  auto setup = [&](auto& ap) {
     ap.P = sample_polys<double, double>(a.pz[ps], a.len[ps], f, a.C, a.ns, s);
     ap.C = a.C;
     ap.t1 = a.t1;
@@ -671,43 +693,38 @@ __global__ void k_sample_solve(SampleArgs a, int nreal) {
     ap.L = a.len[ps][0] + a.t2 - 1;
     ap.y = a.resid + o * a.C * (int64_t)a.Lmax;
     ap.F[0] = ap.F[1] = nullptr;
-    if (a.mixed) {   // the refinement step in float-float arithmetic
+    if (a.mixed) {   // real samples: the step in float-float; complex ones are kept as float-float pairs only
       for (int k = 0; k < 2; ++k) {
         ap.F[k] = a.pzf[ps][k] + ((int64_t)f * a.C * a.ns + s) * a.len[ps][k];
         ap.fstride[k] = (int64_t)a.len[ps][k] * a.ns;
       }
     }
-    ap.real = true;
+    ap.real = real;
+  };
+  TriResult res;
+  if (real) {
+    SylvesterApply<true> ap;
+    setup(ap);
     ap.part = reinterpret_cast<float2*>(W.part);   // free once the reduction is done
     {
       unsigned dsm;
       asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dsm));
-      const size_t per = tri_ws_bytes(n);          // this CTA's other sample slots hold S x
+      const size_t per = tri_ws_bytes(n);          // the CTA's shared memory behind W holds S x
       if (dsm > per) {
         ap.ys = reinterpret_cast<float2*>(smem + per);
         ap.ys_cap = (int)((dsm - per) / sizeof(float2));
       }
     }
-    // mixed path with a CTA of three or more warps: float-float steps 2-5
-    res = tri_smallest<double, true>(W, G, n, far, 1, gap, ap, tk, false, nullptr,
-                                     a.mixed && blockDim.x >= 96);
+    res = tri_smallest_team<double>(W, G, n, far, 1, gap, ap, tk, false, nullptr, a.mixed != 0);
+    if (warp != 0) return;
+  } else if constexpr (TEAM) {
+    SylvesterApply<true> ap;
+    setup(ap);
+    res = tri_smallest_team<cd>(W, G, n, far, 1, gap, ap, tk, a.mixed != 0);
     if (warp != 0) return;
   } else {
     SylvesterApply<false> ap;
-    ap.P = sample_polys<double, double>(a.pz[ps], a.len[ps], f, a.C, a.ns, s);
-    ap.C = a.C;
-    ap.t1 = a.t1;
-    ap.t2 = a.t2;
-    ap.L = a.len[ps][0] + a.t2 - 1;
-    ap.y = a.resid + o * a.C * (int64_t)a.Lmax;
-    ap.F[0] = ap.F[1] = nullptr;
-    if (a.mixed) {   // the mixed path keeps complex samples as float-float pairs only
-      for (int k = 0; k < 2; ++k) {
-        ap.F[k] = a.pzf[ps][k] + ((int64_t)f * a.C * a.ns + s) * a.len[ps][k];
-        ap.fstride[k] = (int64_t)a.len[ps][k] * a.ns;
-      }
-    }
-    ap.real = false;
+    setup(ap);
     // mixed path: single-precision T and Newton steps against G first
     res = tri_smallest<cd, false>(W, G, n, far, 1, gap, ap, tk, a.mixed != 0);
   }
@@ -756,6 +773,7 @@ struct ScaleArgs {
   int M, ns, t1, t2, nn, mixed, Ph, Pw;
   int mode;             // kScaleLS, kScaleK1, kScaleSupport
   int ffx;              // mixed path with room for the float-float stage (scale_ff_offset)
+  Roots w;              // the M-th roots
 };
 
 // Scale fixes: both kernels' two-order least squares; kernel 1's equations
@@ -836,12 +854,10 @@ struct SupportApply {
   }
 };
 
-// Shared memory of k_scale_solve: the normal matrix (2M x 2M complex), block
-// reduction scratch (32 doubles), X and T (3 M^2 complex), then the
-// tridiagonal solver's work area.
+// Shared memory of k_scale_solve: the normal matrix (2M x 2M complex), X
+// (2 M^2 complex), then the tridiagonal solver's work area.
 __host__ __device__ inline size_t scale_tri_offset(int M) {
-  return (sizeof(cd) * 4 * M * M + 32 * sizeof(double) + sizeof(cd) * 3 * M * M + 127) &
-         ~size_t(127);
+  return (sizeof(cd) * 6 * M * M + 127) & ~size_t(127);
 }
 // then the mixed path's float-float cofactors [2][M][nn] and lifted spectra [4][M][M]
 __host__ __device__ inline size_t scale_ff_offset(int M, int nn) {
@@ -851,7 +867,7 @@ __host__ __device__ inline size_t scale_ff_bytes(int M, int nn) {
   return sizeof(cfx) * (2 * (size_t)M * nn + 4 * (size_t)M * M);
 }
 
-__global__ void __launch_bounds__(kSolveThreads) k_scale_solve(ScaleArgs a) {
+__global__ void __launch_bounds__(kSolveThreads, 1) k_scale_solve(ScaleArgs a) {
   extern __shared__ __align__(16) char smem[];
   const int f = blockIdx.x;
   if (a.accepted && a.accepted[f]) {
@@ -895,16 +911,11 @@ __global__ void __launch_bounds__(kSolveThreads) k_scale_solve(ScaleArgs a) {
 #endif
   CBP_TICK(ph, 0);
   cd* Gs = (cd*)smem;                   // [n][n] normal matrix
-  double* red = (double*)(Gs + n * n);   // block reductions
-  char* p = (char*)(red + 32);
-  cd* X = (cd*)p;                 // [2][M][M] kernel spectra, then full inverse DFTs
-  cd* T = X + 2 * MM;             // [M][M] temporary
+  cd* X = Gs + 4 * MM;                  // [2][M][M] kernel spectra, then their half inverse DFTs
   __shared__ cd wt[kMaxM];
   __shared__ cfx wtx[kMaxM];
   for (int k = threadIdx.x; k < M; k += blockDim.x) {
-    double sn, cs;
-    sincospi(-2.0 * (double)k / (double)M, &sn, &cs);
-    wt[k] = mk(cs, sn);
+    wt[k] = mk(a.w.c[k], -a.w.s[k]);
     wtx[k] = cfx_of(wt[k]);
   }
   __syncthreads();
@@ -928,7 +939,11 @@ __global__ void __launch_bounds__(kSolveThreads) k_scale_solve(ScaleArgs a) {
       const cfx* u = cof + ((isB ? M : 0) + (isB ? i : j)) * a.nn + lo;
       const int mult = isB ? j : i;
       cfx_acc acc;
-      for (int q = 0; q < t; ++q) acc.mac(u[q], wtx[(mult * q) % M]);
+      for (int q = 0, e = 0; q < t; ++q) {      // e = mult q mod M
+        acc.mac(u[q], wtx[e]);
+        e += mult;
+        if (e >= M) e -= M;
+      }
       const cfx v = acc.value();
       abx[idx] = v;
       ab[idx] = cfx_val(v);
@@ -948,34 +963,42 @@ __global__ void __launch_bounds__(kSolveThreads) k_scale_solve(ScaleArgs a) {
   }
   __syncthreads();
   CBP_TICK(ph, 1);
-  // normal matrix of the scale system
+  // normal matrix of the scale system: the diagonal (a column's or row's energy
+  // over the kernels) by eight lanes an entry, the rest an entry a thread
   if (ffx) {
+    for (int e0 = threadIdx.x >> 3; e0 < ((n + 3) & ~3); e0 += kSolveThreads / 8) {   // whole warps
+      const int r = min(e0, n - 1), sub = threadIdx.x & 7;
+      fx_acc g;
+      for (int t = sub; t < nk * M; t += 8) {
+        const int k = t >= M, i = t - k * M;
+        const cfx v = r < M ? abx[k * MM + i * M + r] : abx[(2 + k) * MM + (r - M) * M + i];
+        g.mac(v.re, v.re);
+        g.mac(v.im, v.im);
+      }
+      fx v = g.value();
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1)
+        v = fx_add(v, {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+      if (sub == 0 && e0 < n) Gs[r * n + r] = mk(fx_val(v), 0.0);
+    }
     for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
       const int r = idx / n, c = idx % n;
+      if (r == c) continue;
       cfx_acc g;
-      if (r < M && c < M) {
-        if (r == c)
-          for (int k = 0; k < nk; ++k)
-            for (int i = 0; i < M; ++i) g.macc(abx[k * MM + i * M + r], abx[k * MM + i * M + r]);
-      } else if (r >= M && c >= M) {
-        if (r == c)
-          for (int k = 0; k < nk; ++k)
-            for (int j = 0; j < M; ++j)
-              g.macc(abx[(2 + k) * MM + (r - M) * M + j], abx[(2 + k) * MM + (r - M) * M + j]);
-      } else if (r < M) {   // (gamma_j, delta_i) = -sum_k conj(A_k[i][j]) B_k[i][j]
+      if (r < M && c >= M) {   // (gamma_j, delta_i) = -sum_k conj(A_k[i][j]) B_k[i][j]
         const int j = r, i = c - M;
         for (int k = 0; k < nk; ++k) {
           const cfx av = abx[k * MM + i * M + j];
           g.macc({fx_neg(av.re), fx_neg(av.im)}, abx[(2 + k) * MM + i * M + j]);
         }
-      } else {
+      } else if (r >= M && c < M) {
         const int j = c, i = r - M;
         for (int k = 0; k < nk; ++k) {
           const cfx bv = abx[(2 + k) * MM + i * M + j];
           g.macc({fx_neg(bv.re), fx_neg(bv.im)}, abx[k * MM + i * M + j]);
         }
       }
-      Gs[idx] = cfx_val(g.value());
+      Gs[idx] = (r < M) == (c < M) ? mk(0.0, 0.0) : cfx_val(g.value());
     }
   }
   for (int idx = threadIdx.x; !ffx && idx < n * n; idx += blockDim.x) {
@@ -1029,10 +1052,10 @@ __global__ void __launch_bounds__(kSolveThreads) k_scale_solve(ScaleArgs a) {
   TriResult res;
   if (mode == kScaleSupport) {
     SupportApply ap{ab, wt, X, M, t1, t2};      // X is free until the combination below
-    res = tri_smallest<cd, true>(W, Gs, n, 1, 1, 1e300, ap, tk, a.mixed != 0);
+    res = tri_smallest_team<cd>(W, Gs, n, 1, 1, 1e300, ap, tk, a.mixed != 0);
   } else {
     ScaleApply ap{ab, M, nk};
-    res = tri_smallest<cd, true>(W, Gs, n, 1, 1, 1e300, ap, tk, a.mixed != 0, Gx);
+    res = tri_smallest_team<cd>(W, Gs, n, 1, 1, 1e300, ap, tk, a.mixed != 0, Gx);
   }
   __syncthreads();
   CBP_TICK(ph, 3);
@@ -1047,97 +1070,161 @@ __global__ void __launch_bounds__(kSolveThreads) k_scale_solve(ScaleArgs a) {
   }
   __syncthreads();
   __shared__ cd x00[2];
-  if (threadIdx.x < 2) x00[threadIdx.x] = X[threadIdx.x * MM];
-  __syncthreads();
   CBP_TICK(ph, 4);
-  // inverse DFT, separable: T[i][q] = sum_j X[i][j] w^{-jq};  K[p][q] = sum_i w^{-ip} T[i][q] / M^2
-  for (int k = 0; k < 2; ++k) {
-    if (k >= nk) {
-      // k1-only: no kernel 2 (its internal copy zeroed, the caller's buffer untouched)
-      double* kd2 = a.kd + (int64_t)f * (t1 * t1 + t2 * t2) + t1 * t1;
-      for (int e = threadIdx.x; e < t2 * t2; e += blockDim.x) kd2[e] = 0.0;
-      continue;
-    }
-    cd* Xk = X + k * MM;
-    const cd inv00 = [&] {
-      cd z = x00[k];
-      double d = abs2(z);
-      return d > 0 ? mk(z.re / d, -z.im / d) : mk(0.0, 0.0);
-    }();
-    cfx* Yx = (cfx*)Xk;   // float-float: Xk inv00 in place, then the stages on Tx
-    cfx* Tx = (cfx*)T;
-    if (ffx) {
-      const cfx inv = cfx_of(inv00);
-      for (int idx = threadIdx.x; idx < MM; idx += blockDim.x) Yx[idx] = cfx_mul(cfx_of(Xk[idx]), inv);
-      __syncthreads();
-      for (int idx = threadIdx.x; idx < MM; idx += blockDim.x) {
-        const int i = idx / M, q = idx % M;
-        cfx_acc acc;
-        for (int j = 0; j < M; ++j) {
-          const cfx w = wtx[(j * q) % M];
-          acc.mac(Yx[i * M + j], {w.re, fx_neg(w.im)});
-        }
-        Tx[idx] = acc.value();
-      }
-    }
-    for (int idx = threadIdx.x; !ffx && idx < MM; idx += blockDim.x) {
-      const int i = idx / M, q = idx % M;
-      cd acc = mk(0.0, 0.0);
-      for (int j = 0; j < M; ++j) cfma(acc, Xk[i * M + j] * inv00, root(wt, j * q, M, 1.0));
-      T[idx] = acc;
-    }
-    __syncthreads();
-    const int t = k ? t2 : t1;
-    double* kd = a.kd + (int64_t)f * (t1 * t1 + t2 * t2) + (k ? t1 * t1 : 0);
-    double l_im = 0, l_re = 0, l_out = 0;
-    for (int idx = threadIdx.x; idx < MM; idx += blockDim.x) {
-      const int pp = idx / M, q = idx % M;
-      cd acc = mk(0.0, 0.0);
-      if (ffx) {
-        cfx_acc ax;
-        for (int i = 0; i < M; ++i) {
-          const cfx w = wtx[(i * pp) % M];
-          ax.mac({w.re, fx_neg(w.im)}, Tx[i * M + q]);
-        }
-        acc = cfx_val(ax.value());
-      } else {
-        for (int i = 0; i < M; ++i) cfma(acc, root(wt, i * pp, M, 1.0), T[i * M + q]);
-      }
-      acc = (1.0 / (double)MM) * acc;
-      l_re += acc.re * acc.re;
-      l_im += acc.im * acc.im;
-      if (pp >= t || q >= t) l_out += abs2(acc);
-      if (pp < t && q < t && CBP_CHECK(pp < a.M && q < a.M, 3)) {
-        kd[pp * t + q] = acc.re;
-        void* out = k ? a.k2_out : a.k1_out;
-        int64_t oi = (int64_t)f * t * t + pp * t + q;
-        const uint64_t* tab = k ? a.k2_tab : a.k1_tab;
-        if (tab) {
-          out = (void*)tab[f];
-          oi = pp * t + q;
-        }
-        if (out) {
-          if (a.out_f64) ((double*)out)[oi] = acc.re;
-          else ((float*)out)[oi] = (float)acc.re;
-        }
-      }
-    }
-    l_re = block_sum(l_re, red);
-    l_im = block_sum(l_im, red);
-    l_out = block_sum(l_out, red);
-    if (threadIdx.x == 0) {
-      double ir = l_re > 0 ? sqrt(l_im / l_re) : 0.0;
-      double sr = (l_re + l_im) > 0 ? l_out / (l_re + l_im) : 0.0;
-      if (k == 0) {
-        a.diag[f].imag_ratio = ir;
-        a.diag[f].support_ratio = sr;
-      } else {
-        a.diag[f].imag_ratio = fmax(a.diag[f].imag_ratio, ir);
-        a.diag[f].support_ratio = fmax(a.diag[f].support_ratio, sr);
-      }
-    }
-    __syncthreads();
+  // inverse DFT, separable: T[i][q] = sum_j X[i][j] w^{-jq};  K[p][q] = sum_i w^{-ip} T[i][q] / M^2,
+  // both kernels side by side, T in place of X (each row by the threads that read it)
+  __shared__ cd inv00[2];
+  if (threadIdx.x < 2) {
+    const cd z = X[threadIdx.x * MM];
+    x00[threadIdx.x] = z;
+    const double d = abs2(z);
+    inv00[threadIdx.x] = d > 0 ? mk(z.re / d, -z.im / d) : mk(0.0, 0.0);
   }
+  if (nk < 2) {
+    // k1-only: no kernel 2 (its internal copy zeroed, the caller's buffer untouched)
+    double* kd2 = a.kd + (int64_t)f * (t1 * t1 + t2 * t2) + t1 * t1;
+    for (int e = threadIdx.x; e < t2 * t2; e += blockDim.x) kd2[e] = 0.0;
+  }
+  __syncthreads();
+  cfx* Xx = (cfx*)X;   // float-float: X inv00 in place (the same 16 bytes an entry)
+  for (int idx = threadIdx.x; idx < nk * MM; idx += blockDim.x) {
+    const int k = idx >= MM;
+    if (ffx) Xx[idx] = cfx_mul(cfx_of(X[idx]), cfx_of(inv00[k]));
+    else X[idx] = X[idx] * inv00[k];
+  }
+  __syncthreads();
+  // a thread keeps one (kernel, q) and its T values until all of X's rows are read
+  constexpr int kTPer = (2 * kMaxM * kMaxM + kSolveThreads - 1) / kSolveThreads;
+  cd tv[kTPer];
+#pragma unroll
+  for (int r = 0; r < kTPer; ++r) {
+    const int idx = threadIdx.x + r * kSolveThreads;
+    if (idx < nk * MM) {
+      const int i0 = idx / M, q = idx - i0 * M;           // row i0 = k M + i
+      if (ffx) {
+        cfx_acc acc;
+        for (int j = 0, e = 0; j < M; ++j) {
+          const cfx w = wtx[e];
+          acc.mac(Xx[i0 * M + j], {w.re, fx_neg(w.im)});
+          e += q;
+          if (e >= M) e -= M;
+        }
+        const cfx v = acc.value();             // kept as its 16 bytes
+        tv[r] = mk(__hiloint2double(__float_as_int(v.re.lo), __float_as_int(v.re.hi)),
+                   __hiloint2double(__float_as_int(v.im.lo), __float_as_int(v.im.hi)));
+      } else {
+        cd acc = mk(0.0, 0.0);
+        for (int j = 0, e = 0; j < M; ++j) {
+          cfma(acc, X[i0 * M + j], conj(wt[e]));
+          e += q;
+          if (e >= M) e -= M;
+        }
+        tv[r] = acc;
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kTPer; ++r) {
+    const int idx = threadIdx.x + r * kSolveThreads;
+    if (idx < nk * MM) X[idx] = tv[r];
+  }
+  __syncthreads();
+  double sums[6] = {0, 0, 0, 0, 0, 0};   // per kernel: Re^2, Im^2, energy outside t x t
+  for (int idx = threadIdx.x; idx < nk * MM; idx += blockDim.x) {
+    const int k = idx >= MM, e0 = idx - k * MM;
+    const int pp = e0 / M, q = e0 - pp * M, t = k ? t2 : t1;
+    cd acc = mk(0.0, 0.0);
+    if (ffx) {
+      cfx_acc ax;
+      for (int i = 0, e = 0; i < M; ++i) {
+        const cfx w = wtx[e];
+        ax.mac({w.re, fx_neg(w.im)}, Xx[k * MM + i * M + q]);
+        e += pp;
+        if (e >= M) e -= M;
+      }
+      acc = cfx_val(ax.value());
+    } else {
+      for (int i = 0, e = 0; i < M; ++i) {
+        cfma(acc, conj(wt[e]), X[k * MM + i * M + q]);
+        e += pp;
+        if (e >= M) e -= M;
+      }
+    }
+    acc = (1.0 / (double)MM) * acc;
+    const double r2 = acc.re * acc.re, i2 = acc.im * acc.im;
+    const bool outside = pp >= t || q >= t;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (h == k) {
+        sums[3 * h] += r2;
+        sums[3 * h + 1] += i2;
+        if (outside) sums[3 * h + 2] += r2 + i2;
+      }
+    if (!outside && CBP_CHECK(pp < a.M && q < a.M, 3)) {
+      a.kd[(int64_t)f * (t1 * t1 + t2 * t2) + (k ? t1 * t1 : 0) + pp * t + q] = acc.re;
+      void* out = k ? a.k2_out : a.k1_out;
+      int64_t oi = (int64_t)f * t * t + pp * t + q;
+      const uint64_t* tab = k ? a.k2_tab : a.k1_tab;
+      if (tab) {
+        out = (void*)tab[f];
+        oi = pp * t + q;
+      }
+      if (out) {
+        if (a.out_f64) ((double*)out)[oi] = acc.re;
+        else ((float*)out)[oi] = (float)acc.re;
+      }
+    }
+  }
+  __shared__ double dsum[6][kSolveThreads / 32], dtot[6];
+#pragma unroll
+  for (int h = 0; h < 6; h += 2) {
+    lane_sum2(sums[h], sums[h + 1]);
+    if ((threadIdx.x & 31) == 0) {
+      dsum[h][threadIdx.x >> 5] = sums[h];
+      dsum[h + 1][threadIdx.x >> 5] = sums[h + 1];
+    }
+  }
+  // the samples' diagnostics by warp 1: every quantity is a maximum or minimum
+  // of non-negative doubles, compared as integers
+  __shared__ double agg[4];   // gap^2 (min), (theta / lambda_max) (max), flagged, hard
+  if (threadIdx.x >= 32 && threadIdx.x < 64) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long gmin = 0x7fefffffffffffffull, smax = 0;
+    int flagged = 0, hard = 0;
+    for (int i = lane; i < 2 * a.ns; i += 32) {
+      const double* d = a.sdiag + ((int64_t)f * 2 * a.ns + i) * 4;
+      const double lmax = d[0] > 0 ? d[0] : 1e-300;
+      const double g = fmax(d[1], 0.0) / lmax, m = fmax(d[2], 0.0) / lmax;
+      const unsigned long long gb = (unsigned long long)__double_as_longlong(g),
+                               mb = (unsigned long long)__double_as_longlong(m);
+      if (gb < gmin) gmin = gb;
+      if (mb > smax) smax = mb;
+      if (sqrt(g) < 1e-8) ++flagged;
+      hard += (int)d[3];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long g2 = __shfl_xor_sync(0xffffffffu, gmin, o), m2 = __shfl_xor_sync(0xffffffffu, smax, o);
+      if (g2 < gmin) gmin = g2;
+      if (m2 > smax) smax = m2;
+    }
+    flagged = __reduce_add_sync(0xffffffffu, flagged);
+    hard = __reduce_add_sync(0xffffffffu, hard);
+    if (lane == 0) {
+      agg[0] = __longlong_as_double((long long)gmin);
+      agg[1] = __longlong_as_double((long long)smax);
+      agg[2] = (double)flagged;
+      agg[3] = (double)hard;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    double t = 0.0;
+    for (int w = 0; w < kSolveThreads / 32; ++w) t += dsum[threadIdx.x][w];
+    dtot[threadIdx.x] = t;
+  }
+  __syncwarp();
   CBP_TICK(ph, 5);
 #ifdef CBP_PHASE_TIMING
   if (tk && threadIdx.x == 0)
@@ -1148,18 +1235,17 @@ __global__ void __launch_bounds__(kSolveThreads) k_scale_solve(ScaleArgs a) {
 #endif
   // aggregate diagnostics
   if (threadIdx.x == 0) {
-    double kappa = 0, gap = 1e300, smin = 0;
-    int flagged = 0, hard = 0;
-    for (int i = 0; i < 2 * a.ns; ++i) {
-      const double* d = a.sdiag + ((int64_t)f * 2 * a.ns + i) * 4;
-      const double lmax = d[0] > 0 ? d[0] : 1e-300;
-      const double g = sqrt(fmax(d[1], 0.0) / lmax);
-      gap = fmin(gap, g);
-      kappa = fmax(kappa, g > 0 ? 1.0 / g : 1e300);
-      smin = fmax(smin, sqrt(fmax(d[2], 0.0) / lmax));
-      if (g < 1e-8) ++flagged;
-      hard += (int)d[3];
+    double ir = 0.0, sr = 0.0;
+    for (int k = 0; k < nk; ++k) {
+      const double* t = dtot + 3 * k;
+      ir = fmax(ir, t[0] > 0 ? sqrt(t[1] / t[0]) : 0.0);
+      sr = fmax(sr, (t[0] + t[1]) > 0 ? t[2] / (t[0] + t[1]) : 0.0);
     }
+    a.diag[f].imag_ratio = ir;
+    a.diag[f].support_ratio = sr;
+    const double gap = sqrt(agg[0]), smin = sqrt(agg[1]);
+    const double kappa = gap > 0 ? 1.0 / gap : 1e300;
+    const int flagged = (int)agg[2], hard = (int)agg[3];
     cbp_diag& dg = a.diag[f];
     dg.kappa_max = kappa;
     dg.gap_min = gap;
@@ -1253,7 +1339,7 @@ struct NoApply {
   __device__ void operator()(const cd*, cd*) const {}
 };
 
-__global__ void __launch_bounds__(kSolveThreads) k_size_scan(SizeScanArgs a) {
+__global__ void __launch_bounds__(kSolveThreads, 1) k_size_scan(SizeScanArgs a) {
   extern __shared__ __align__(16) char smem[];
   const int cand = blockIdx.x, ps = blockIdx.y, f = blockIdx.z;
   const int t1 = a.t_min + cand, t2 = t1 - a.d, n = t1 + t2;
@@ -1313,7 +1399,7 @@ struct CoprimeArgs {
   int* pass;            // [n][2][ns]
 };
 
-__global__ void __launch_bounds__(kSolveThreads) k_coprime_test(CoprimeArgs a) {
+__global__ void __launch_bounds__(kSolveThreads, 1) k_coprime_test(CoprimeArgs a) {
   extern __shared__ __align__(16) char smem[];
   const int j = blockIdx.x, order = blockIdx.y, f = blockIdx.z;
   if (!a.active[f]) return;
@@ -1423,17 +1509,34 @@ void launch_sample_solve(const Plan& p, char* ws, cudaStream_t st) {
   a.mixed = p.mixed;
   a.accepted = p.learned ? (const int*)(ws + p.off_acc) : nullptr;
   a.G = (cd*)(ws + p.off_gall);
-  dim3 grid(p.n, 2, p.ns);
+  // about four CTAs per SM: a sample's lags split over up to eight CTAs (three
+  // 720p colour pairs, 13 / 11 kernels: 73 us with a CTA per sample)
+  a.gsplit = std::max(1, std::min(8, 608 / (p.n * 2 * p.ns)));
+  dim3 grid(p.n, 2, p.ns * a.gsplit);
   k_sample_gram<<<grid, kSolveThreads, 0, st>>>(a);
-  // warps (samples) per CTA: up to CBP_SOLVE_WPC within ~110 KB of shared memory
   const int nrs = (p.M % 2 == 0) ? 2 : 1, ncs = p.ns - nrs;
   const int nreal = p.n * 2 * nrs, ncomplex = p.n * 2 * ncs;
   const size_t per = tri_ws_bytes(p.nn);
-  const int wpc = (int)std::max<size_t>(1, std::min<size_t>(CBP_SOLVE_WPC, (110u << 10) / per));
-  const size_t sm = per * wpc;
   a.nfr = p.n;
-  cudaFuncSetAttribute(k_sample_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_sample_solve<<<nreal + (ncomplex + wpc - 1) / wpc, 32 * wpc, sm, st>>>(a, nreal);
+  a.wpc = 1;
+  if (nreal + ncomplex <= (p.mixed ? CBP_TEAM_CTAS : CBP_TEAM_CTAS_F64)) {
+    // a CTA per sample; behind its work area the real samples' float-float
+    // refinement keeps a channel's S x and both polynomials where they fit
+    size_t sm = per;
+    if (p.mixed) {
+      const int lz2 = p.H1 + p.H2 + p.H1 + p.t2 - 1, lz1 = p.W1 + p.W2 + p.W1 + p.t2 - 1;
+      const size_t need = per + sizeof(float2) * (size_t)std::max(lz1, lz2);
+      if (need <= (110u << 10)) sm = need;
+    }
+    cudaFuncSetAttribute(k_sample_solve<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_sample_solve<true><<<nreal + ncomplex, kTeamThreads, sm, st>>>(a, nreal);
+    return;
+  }
+  // warps (samples) per CTA: up to CBP_SOLVE_WPC within ~110 KB of shared memory
+  a.wpc = (int)std::max<size_t>(1, std::min<size_t>(CBP_SOLVE_WPC, (110u << 10) / per));
+  const size_t sm = per * a.wpc;
+  cudaFuncSetAttribute(k_sample_solve<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_sample_solve<false><<<nreal + (ncomplex + a.wpc - 1) / a.wpc, kTeamThreads, sm, st>>>(a, nreal);
 }
 
 void launch_scale_solve(const Plan& p, char* ws, void* k1_out, void* k2_out, int out_f64,
@@ -1462,6 +1565,7 @@ void launch_scale_solve(const Plan& p, char* ws, void* k1_out, void* k2_out, int
   a.accepted = p.learned ? (const int*)(ws + p.off_acc) : nullptr;
   a.rho = p.learned ? (const double*)(ws + p.off_rho) : nullptr;
   a.mode = p.scale_mode;
+  a.w = make_roots(p.M);
   // the mixed path's float-float stage where its shared memory fits
   const size_t ff_end = scale_ff_offset(p.M, p.nn) + scale_ff_bytes(p.M, p.nn);
   int dev = 0, smem_max = 0;
