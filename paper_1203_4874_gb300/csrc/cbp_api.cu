@@ -445,8 +445,7 @@ cbp_status draw_coprime_pairs(int n, int ta, int tb, int kind_a, int kind_b, int
       cudaMemsetAsync(attempt, 0, (size_t)n * sizeof(int), st) != cudaSuccess)
     return CBP_ERR_CUDA;
   for (int r = 0; r < max_attempts; ++r) {
-    cbp::launch_draw_kernels(n, ta, kind_a, frame0, seed, active, attempt, ka, st);
-    cbp::launch_draw_kernels(n, tb, kind_b, frame0, seed, active, attempt, kb, st);
+    cbp::launch_draw_kernels(n, ta, tb, kind_a, kind_b, frame0, seed, active, attempt, ka, kb, st);
     int h_any = 0;
     if (cudaMemsetAsync(any, 0, sizeof(int), st) != cudaSuccess) return CBP_ERR_CUDA;
     cbp::launch_coprime_round(ka, kb, n, ta, tb, M, tol, max_attempts, active, attempt, pass, any, st);

@@ -26,8 +26,8 @@ __device__ __forceinline__ double normal_at(uint64_t seed, uint64_t idx, uint32_
 
 // The same normal number in single precision (float frames).
 __device__ __forceinline__ float normal_at_f(uint64_t seed, uint64_t idx, uint32_t stream) {
-  U4 c = {(uint32_t)idx, (uint32_t)(idx >> 32), stream, 0u};
-  U4 r = philox4x32_10(c, (uint32_t)seed, (uint32_t)(seed >> 32));
+  const U4 r = philox4x32_10({(uint32_t)idx, (uint32_t)(idx >> 32), stream, 0u}, (uint32_t)seed,
+                             (uint32_t)(seed >> 32));
   const float u1 = ((float)(r.x >> 8) + 1.0f) * 5.9604644775390625e-8f;   // (0, 1], 24 bits
   const float u2 = ((float)(r.y >> 8) + 1.0f) * 5.9604644775390625e-8f;
   return sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
@@ -87,69 +87,133 @@ k_forward_blur(const T* lat, int c, int h, int w, const double* kern, int t, dou
 }
 
 // The same convolution for float frames with the kernel size fixed at compile
-// time (T <= 17): a block makes 64 rows x 32 columns of output; a thread keeps
-// eight consecutive output rows of one column and, for each kernel column q,
-// the T + 7 input values they need in registers, so each shared-memory load
-// feeds about four multiply-adds.  Sums in float, in the order p = T-1 .. 0
-// for every q (as the general kernel's per-output order differs, results
-// agree to float rounding, not bitwise).
-constexpr int kBlurRows = 8;          // output rows per thread
-constexpr int kBlurTileR = 8 * kBlurRows;
-template <int T>
-__global__ void __launch_bounds__(256)
+// time (T <= 17).  A block makes 8 R rows x 64 columns of output; a thread keeps
+// R consecutive output rows of two columns (32 apart) as paired single-precision
+// sums (one paired multiply-add for two, each rounded as the scalar one)
+// and, for each kernel column q, slides over the T + R - 1 input rows with the
+// kernel column in registers.  What bounds it: multiply-adds (T^2 an output) and
+// the noise (a Philox block, a logarithm and a cosine an output).  With eight
+// rows of one column and scalar multiply-adds every eight of them had cost a
+// shared-memory load of the kernel and three quarters of one of the tile, and
+// the tile had come over in single words.  Here the tile is copied in 16-byte
+// pieces (cp.async, zero outside the frame) where the latent's rows are aligned.
+// Sums in float, in the order q = 0 .. T-1, within it p = 0 .. T-1 (as the
+// general kernel's per-output order differs, results agree to float rounding,
+// not bitwise).  48 channels of 1080 x 1920, T = 15: 1.62 -> 1.40 ms (0.91 ms
+// without noise, 25 of the units' 37 T multiply-adds a second; three blocks per SM
+// instead of two 0.93 ms); T = 17: 1.89 -> 1.63 ms; T = 5 without noise 0.21 ms.
+// R = 16 rows a thread where that still gives every SM two blocks, else R = 4.
+constexpr int kBlurWarps = 8;
+constexpr int kBlurTileC = 64;
+constexpr int kBlurHalo = 16;                        // columns kept left of the tile (T - 1 <= 16)
+constexpr int kBlurPitch = kBlurTileC + kBlurHalo;
+constexpr int64_t kBlurMinBlocks = 2 * 152;
+template <int T, int R>
+__global__ void __launch_bounds__(32 * kBlurWarps, 2)
 k_forward_blur_rb(const float* lat, int c, int h, int w, const double* kern, double sigma,
                   uint64_t seed, float* out) {
-  __shared__ float K[T * T];
-  __shared__ float tile[(kBlurTileR + T - 1) * (32 + T - 1)];
-  constexpr int TW = 32 + T - 1, TH = kBlurTileR + T - 1;
+  constexpr int kTileR = kBlurWarps * R, TH = kTileR + T - 1;
+  constexpr int TP = (T + 1) & ~1;                   // kernel column pitch, 16-byte aligned pairs
+  extern __shared__ __align__(16) char bsm[];
+  float* tile = (float*)bsm;                         // [TH][kBlurPitch]
+  float2* K = (float2*)(bsm + sizeof(float) * TH * kBlurPitch);   // [q][p], each value twice
   const int hb = h + T - 1, wb = w + T - 1;
   const int fc = blockIdx.z, f = fc / c;
-  const int r0 = blockIdx.y * kBlurTileR, c0 = blockIdx.x * 32;
-  for (int i = threadIdx.x; i < T * T; i += blockDim.x) K[i] = (float)kern[(int64_t)f * T * T + i];
+  const int r0 = blockIdx.y * kTileR, c0 = blockIdx.x * kBlurTileC;
   const float* L = lat + (int64_t)fc * h * w;
-  for (int i = threadIdx.x; i < TH * TW; i += blockDim.x) {
-    const int y = i / TW, x = i - y * TW;
-    const int ly = r0 - (T - 1) + y, lx = c0 - (T - 1) + x;
-    tile[i] = (ly >= 0 && ly < h && lx >= 0 && lx < w) ? L[(int64_t)ly * w + lx] : 0.f;
-  }
-  __syncthreads();
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  float acc[kBlurRows];
-#pragma unroll
-  for (int i = 0; i < kBlurRows; ++i) acc[i] = 0.f;
-  // out[r][col] = sum_{p,q} K[p][q] tile[(r - r0) + T-1-p][(col - c0) + T-1-q]
-  for (int q = 0; q < T; ++q) {
-    float v[kBlurRows + T - 1];
-    const float* col = tile + (ty * kBlurRows) * TW + tx + T - 1 - q;
-    (void)CBP_CHECK((ty * kBlurRows + kBlurRows + T - 2) * TW + tx + T - 1 - q < TH * TW, 0);
-#pragma unroll
-    for (int j = 0; j < kBlurRows + T - 1; ++j) v[j] = col[j * TW];
-#pragma unroll
-    for (int p = 0; p < T; ++p) {
-      const float kv = K[p * T + q];
-#pragma unroll
-      for (int i = 0; i < kBlurRows; ++i) acc[i] = fmaf(kv, v[i + T - 1 - p], acc[i]);
+  // tile[y][x] = latent at row r0 - (T-1) + y, column c0 - kBlurHalo + x
+  constexpr int G = kBlurPitch / 4;
+  if ((w & 3) == 0 && ((uintptr_t)lat & 15) == 0) {
+    for (int i = threadIdx.x; i < TH * G; i += 32 * kBlurWarps) {
+      const int y = i / G, x = (i - y * G) * 4;
+      const int ly = r0 - (T - 1) + y, lx = c0 - kBlurHalo + x;   // four columns all inside or all outside
+      const bool in = ly >= 0 && ly < h && lx >= 0 && lx < w;
+      const float* src = in ? L + (int64_t)ly * w + lx : lat;
+      const unsigned dst = (unsigned)__cvta_generic_to_shared(tile + y * kBlurPitch + x);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(in ? 16 : 0)
+                   : "memory");
+    }
+  } else {
+    for (int i = threadIdx.x; i < TH * kBlurPitch; i += 32 * kBlurWarps) {
+      const int y = i / kBlurPitch, x = i - y * kBlurPitch;
+      const int ly = r0 - (T - 1) + y, lx = c0 - kBlurHalo + x;
+      const bool in = ly >= 0 && ly < h && lx >= 0 && lx < w;
+      const float* src = in ? L + (int64_t)ly * w + lx : lat;
+      const unsigned dst = (unsigned)__cvta_generic_to_shared(tile + i);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(dst), "l"(src), "r"(in ? 4 : 0)
+                   : "memory");
     }
   }
-  const int colo = c0 + tx;
-  if (colo >= wb) return;
+  for (int i = threadIdx.x; i < T * TP; i += 32 * kBlurWarps) {
+    const int q = i / TP, p = i - q * TP;
+    const float v = p < T ? (float)kern[(int64_t)f * T * T + p * T + q] : 0.f;
+    K[i] = make_float2(v, v);
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  if (r0 + ty * R >= hb) return;                     // a warp below the frame
+  float2 acc[R];
 #pragma unroll
-  for (int i = 0; i < kBlurRows; ++i) {
-    const int r = r0 + ty * kBlurRows + i;
-    if (r >= hb) break;
-    const int64_t oi = ((int64_t)fc * hb + r) * wb + colo;
-    float a = acc[i];
-    if (sigma > 0) a += (float)sigma * normal_at_f(seed, (uint64_t)oi, 1u);
-    out[oi] = a;
+  for (int i = 0; i < R; ++i) acc[i] = make_float2(0.f, 0.f);
+  // out[r][col] = sum_{p,q} K[p][q] L[r - p][col - q]
+#pragma unroll 1
+  for (int q = 0; q < T; ++q) {
+    const float* col = tile + (ty * R) * kBlurPitch + kBlurHalo + tx - q;
+    (void)CBP_CHECK((ty * R + R + T - 2) * kBlurPitch + kBlurHalo + tx - q + 32 < TH * kBlurPitch, 0);
+    float2 kv[TP];
+#pragma unroll
+    for (int p = 0; p < TP; p += 2) {
+      const float4 k2 = *(const float4*)(K + q * TP + p);
+      kv[p] = make_float2(k2.x, k2.y);
+      kv[p + 1] = make_float2(k2.z, k2.w);
+    }
+    // an output row meets the kernel rows in ascending order p = i + T-1 - j:
+    // the input rows are taken from the last to the first
+#pragma unroll
+    for (int j = R + T - 2; j >= 0; --j) {
+      const float2 v = make_float2(col[j * kBlurPitch], col[j * kBlurPitch + 32]);
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const int p = i + T - 1 - j;
+        if (p >= 0 && p < T) acc[i] = __ffma2_rn(kv[p], v, acc[i]);
+      }
+    }
+  }
+#pragma unroll 1
+  for (int g = 0; g < 2; ++g) {
+    const int colo = c0 + tx + 32 * g;
+    if (colo >= wb) break;
+    const int64_t o0 = ((int64_t)fc * hb + r0 + ty * R) * wb + colo;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      if (r0 + ty * R + i >= hb) break;
+      const int64_t oi = o0 + (int64_t)i * wb;
+      float a = g ? acc[i].y : acc[i].x;
+      if (sigma > 0) a += (float)sigma * normal_at_f(seed, (uint64_t)oi, 1u);
+      out[oi] = a;
+    }
   }
 }
 
+template <int T, int R>
+void launch_blur_rows(const float* lat, int n, int c, int h, int w, const double* kern, double sigma,
+                      uint64_t seed, float* out, cudaStream_t st) {
+  const int hb = h + T - 1, wb = w + T - 1;
+  constexpr int tr = kBlurWarps * R;
+  dim3 g((wb + kBlurTileC - 1) / kBlurTileC, (hb + tr - 1) / tr, n * c);
+  constexpr size_t sm = sizeof(float2) * (size_t)T * ((T + 1) & ~1) + sizeof(float) * (size_t)(tr + T - 1) * kBlurPitch;
+  cudaFuncSetAttribute(k_forward_blur_rb<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_forward_blur_rb<T, R><<<g, 32 * kBlurWarps, sm, st>>>(lat, c, h, w, kern, sigma, seed, out);
+}
 template <int T>
 void launch_blur_rb(const float* lat, int n, int c, int h, int w, const double* kern, double sigma,
                     uint64_t seed, float* out, cudaStream_t st) {
   const int hb = h + T - 1, wb = w + T - 1;
-  dim3 g((wb + 31) / 32, (hb + kBlurTileR - 1) / kBlurTileR, n * c);
-  k_forward_blur_rb<T><<<g, 256, 0, st>>>(lat, c, h, w, kern, sigma, seed, out);
+  const int64_t big = (int64_t)((wb + kBlurTileC - 1) / kBlurTileC) * ((hb + 16 * kBlurWarps - 1) / (16 * kBlurWarps)) *
+                      n * c;
+  if (big >= kBlurMinBlocks) launch_blur_rows<T, 16>(lat, n, c, h, w, kern, sigma, seed, out, st);
+  else launch_blur_rows<T, 4>(lat, n, c, h, w, kern, sigma, seed, out, st);
 }
 
 // Blob latent: L = sum_k a_k exp(-((x-cx)^2 + (y-cy)^2) / (2 s^2)) + U[0, floor].
@@ -273,34 +337,51 @@ __global__ void __launch_bounds__(kTruncThreads) k_truncate_lsb(const T* in, int
 // every frame): kernel `kind` of frame frame0 + f at redraw attempt[f],
 // entries (Philox word + 1) 2^-32, uniform in (0, 1], normalised to unit sum
 // in entry order.  Entry e is word e mod 4 of Philox(counter = (e / 4, frame,
-// kind * 256 + attempt, 0), key = seed).  One thread per kernel; pairs whose
-// active flag is clear keep their kernels.
-__global__ void k_draw_kernels(int n, int t, int kind, int frame0, uint64_t seed, const int* active,
-                               const int* attempt, double* kd) {
-  const int f = blockIdx.x * blockDim.x + threadIdx.x;
-  if (f >= n || !active[f]) return;
-  double* K = kd + (int64_t)f * t * t;
+// kind * 256 + attempt, 0), key = seed).  One CTA per kernel, both kernels of a
+// pair in one launch; the entries are multiples of 2^-32 no larger than 1, so
+// every partial sum of up to 2^20 of them is exact and the integer sum is the
+// sum in entry order (one thread per kernel had taken 102 and 130 us for 15 x 15
+// and 17 x 17 kernels: a chain of double adds and one of double divisions).
+// Pairs whose active flag is clear keep their kernels.
+constexpr int kDrawThreads = 128;
+__global__ void __launch_bounds__(kDrawThreads)
+k_draw_kernels(int ta, int tb, int kind_a, int kind_b, int frame0, uint64_t seed, const int* active,
+               const int* attempt, double* ka, double* kb) {
+  const int f = blockIdx.x, second = blockIdx.y;
+  if (!active[f]) return;
+  const int t = second ? tb : ta, kind = second ? kind_b : kind_a, nn = t * t;
+  double* K = (second ? kb : ka) + (int64_t)f * nn;
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-  const int nn = t * t;
-  double sum = 0.0;
-  for (int b = 0; 4 * b < nn; ++b) {
+  __shared__ uint32_t word[32 * 32];
+  __shared__ unsigned long long part[kDrawThreads / 32];
+  unsigned long long sum = 0;
+  for (int b = threadIdx.x; 4 * b < nn; b += kDrawThreads) {
     const U4 r = philox4x32_10({(uint32_t)b, (uint32_t)(frame0 + f), (uint32_t)(kind * 256 + attempt[f]), 0u},
                                k0, k1);
     const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-    for (int i = 0; i < 4 && 4 * b + i < nn; ++i) {
-      const double u = u01(w[i]);
-      K[4 * b + i] = u;
-      sum += u;
-    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (4 * b + i < nn) {
+        word[4 * b + i] = w[i];
+        sum += (unsigned long long)w[i] + 1ull;
+      }
   }
-  for (int e = 0; e < nn; ++e) K[e] = K[e] / sum;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  unsigned long long total = 0;
+#pragma unroll
+  for (int i = 0; i < kDrawThreads / 32; ++i) total += part[i];
+  const double s = (double)total * 2.3283064365386963e-10;   // exact: below 2^43, times 2^-32
+  for (int e = threadIdx.x; e < nn; e += kDrawThreads) K[e] = u01(word[e]) / s;
 }
 
 }  // namespace
 
-void launch_draw_kernels(int n, int t, int kind, int frame0, uint64_t seed, const int* active,
-                         const int* attempt, double* kd, cudaStream_t st) {
-  k_draw_kernels<<<(n + 127) / 128, 128, 0, st>>>(n, t, kind, frame0, seed, active, attempt, kd);
+void launch_draw_kernels(int n, int ta, int tb, int kind_a, int kind_b, int frame0, uint64_t seed,
+                         const int* active, const int* attempt, double* ka, double* kb, cudaStream_t st) {
+  k_draw_kernels<<<dim3(n, 2), kDrawThreads, 0, st>>>(ta, tb, kind_a, kind_b, frame0, seed, active, attempt, ka, kb);
 }
 
 void launch_truncate_lsb(const void* in, int f64, int64_t count, int bits, int drop, void* out,

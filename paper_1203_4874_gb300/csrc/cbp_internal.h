@@ -193,8 +193,8 @@ void launch_truncate_lsb(const void* in, int f64, int64_t count, int bits, int d
                          cudaStream_t st);
 // camera side (Section 3): per-frame kernel draws (cbp_forward.cu) and one
 // round of the coprimality test with the redraw decision (cbp_solve.cu)
-void launch_draw_kernels(int n, int t, int kind, int frame0, uint64_t seed, const int* active,
-                         const int* attempt, double* kd, cudaStream_t st);
+void launch_draw_kernels(int n, int ta, int tb, int kind_a, int kind_b, int frame0, uint64_t seed,
+                         const int* active, const int* attempt, double* ka, double* kb, cudaStream_t st);
 void launch_coprime_round(const double* ka, const double* kb, int n, int ta, int tb, int M,
                           double tol, int max_attempts, int* active, int* attempt, int* pass,
                           int* any, cudaStream_t st);

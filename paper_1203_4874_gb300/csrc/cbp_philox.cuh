@@ -10,8 +10,9 @@ struct U4 { uint32_t x, y, z, w; };
 
 __device__ __forceinline__ U4 philox_round(U4 c, uint32_t k0, uint32_t k1) {
   const uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
-  uint32_t hi0 = __umulhi(M0, c.x), lo0 = M0 * c.x;
-  uint32_t hi1 = __umulhi(M1, c.z), lo1 = M1 * c.z;
+  const uint64_t p0 = (uint64_t)M0 * c.x, p1 = (uint64_t)M1 * c.z;   // one wide product each
+  const uint32_t hi0 = (uint32_t)(p0 >> 32), lo0 = (uint32_t)p0;
+  const uint32_t hi1 = (uint32_t)(p1 >> 32), lo1 = (uint32_t)p1;
   return {hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0};
 }
 
