@@ -108,6 +108,7 @@ struct SizePlan {
   int n, C, d, t_min, ncand;
   double tol;
   size_t off_rows[2], off_cols[2];   // cd [n][C][H_k] row sums, [n][C][W_k] column sums
+  size_t off_rho;                    // double [n][2][2 (t1 + t2) - 1] lags of the largest candidate
   size_t off_ratio;                  // double [n][2][ncand] per order
   size_t off_rmax;                   // double [n][ncand] the larger of the two (-1: excluded)
   size_t off_t;                      // int [n][3]: t1, t2, found

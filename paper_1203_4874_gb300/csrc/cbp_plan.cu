@@ -286,6 +286,7 @@ cbp_status make_size_plan(const cbp_frames* b1, const cbp_frames* b2, const cbp_
   p.off_rows[1] = take(n * C * (size_t)b2->h * 16);
   p.off_cols[0] = take(n * C * (size_t)b1->w * 16);
   p.off_cols[1] = take(n * C * (size_t)b2->w * 16);
+  p.off_rho = take(n * 2 * (size_t)(2 * (2 * (p.t_min + p.ncand - 1) - d) - 1) * 8);
   p.off_ratio = take(n * 2 * (size_t)p.ncand * 8);
   p.off_rmax = take(n * (size_t)p.ncand * 8);
   p.off_t = take(n * 3 * sizeof(int));

@@ -193,28 +193,32 @@ __device__ void correlations(const SamplePolys<TP, TA>& P, int C, int t1, int t2
   __syncthreads();
 }
 
-// rho jobs as above for real samples (z = 1, and z = -1 when M is even):
-// real double correlations of the real parts.
+// Lag j of the rho jobs above for real samples (z = 1, and z = -1 when M is
+// even): a real double correlation of the real parts by the calling warp.
+__device__ __forceinline__ double lag_real(const SamplePolys<double, double>& P, int C, int t1, int t2, int j) {
+  const int lane = threadIdx.x & 31;
+  int ka, kb, d;
+  if (j < t1) { ka = 1; kb = 1; d = j; }
+  else if (j < t1 + t2) { ka = 0; kb = 0; d = j - t1; }
+  else { ka = 1; kb = 0; d = j - t1 - t2 - (t2 - 1); }
+  const int la = P.len[ka], lb = P.len[kb];
+  const int m0 = d < 0 ? -d : 0;
+  const int m1 = min(la, lb - d);
+  double acc = 0;
+  for (int ch = 0; ch < C; ++ch) {
+    const cd* a = P.c[ka] + ch * P.cstride[ka];
+    const cd* b = P.c[kb] + ch * P.cstride[kb];
+    for (int m = m0 + lane; m < m1; m += 32) acc = fma(a[m].re, b[m + d].re, acc);
+  }
+  return warp_sum(acc);
+}
 __device__ void correlations_real(const SamplePolys<double, double>& P, int C, int t1, int t2,
-                                  cd* rho, LagSplit sp = {0, 1}) {
+                                  cd* rho, LagSplit sp) {
   const int J = 2 * (t1 + t2) - 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int j = warp * sp.step + sp.first; j < J; j += nw * sp.step) {
-    int ka, kb, d;
-    if (j < t1) { ka = 1; kb = 1; d = j; }
-    else if (j < t1 + t2) { ka = 0; kb = 0; d = j - t1; }
-    else { ka = 1; kb = 0; d = j - t1 - t2 - (t2 - 1); }
-    const int la = P.len[ka], lb = P.len[kb];
-    const int m0 = d < 0 ? -d : 0;
-    const int m1 = min(la, lb - d);
-    double acc = 0;
-    for (int ch = 0; ch < C; ++ch) {
-      const cd* a = P.c[ka] + ch * P.cstride[ka];
-      const cd* b = P.c[kb] + ch * P.cstride[kb];
-      for (int m = m0 + lane; m < m1; m += 32) acc = fma(a[m].re, b[m + d].re, acc);
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) rho[j] = mk(acc, 0.0);
+    const double r = lag_real(P, C, t1, t2, j);
+    if (lane == 0) rho[j] = mk(r, 0.0);
   }
   __syncthreads();
 }
@@ -1305,34 +1309,100 @@ __global__ void k_kernels_in(const void* k1, const void* k2, int in_f64, int n, 
 // (no refinement steps): ratio = sqrt(theta / lambda_max), theta the
 // Rayleigh quotient of the smallest eigenvector.
 
-// z = 1 samples of a frame batch: row sums [n][C][h] and column sums
-// [n][C][w] (imaginary parts zero), accumulated in double.
-__global__ void k_plane_sums(FrameDesc fr, cd* rows, cd* cols) {
-  const int fc = blockIdx.y, f = fc / fr.c, ch = fc % fr.c;
-  const char* base = (const char*)frame_base(fr, f) + (int64_t)ch * fr.cs * (fr.f64 ? 8 : 4);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (blockIdx.z == 0) {
-    for (int r = blockIdx.x * nw + warp; r < fr.h; r += gridDim.x * nw) {
-      double acc = 0.0;
-      for (int c = lane; c < fr.w; c += 32) acc += ld_frame<double>(base, (int64_t)r * fr.rs + c, fr.f64);
-      acc = warp_sum(acc);
-      if (lane == 0) rows[(int64_t)fc * fr.h + r] = mk(acc, 0.0);
-    }
-  } else {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < fr.w; c += gridDim.x * blockDim.x) {
-      double acc = 0.0;
-      for (int r = 0; r < fr.h; ++r) acc += ld_frame<double>(base, (int64_t)r * fr.rs + c, fr.f64);
-      cols[(int64_t)fc * fr.w + c] = mk(acc, 0.0);
-    }
+// float -> double on the integer pipe (a conversion instruction shares the
+// double units); zeros included, denormals and non-finite values by the
+// conversion, in a function of its own so that it costs a branch only.
+__device__ __noinline__ double widen_slow(float x) { return (double)x; }
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), a = u & 0x7fffffffu, sg = u & 0x80000000u;
+  if (a != 0u && a - 0x00800000u >= 0x7f000000u) return widen_slow(x);
+  return __hiloint2double((int)(a ? (sg | ((a >> 3) + 0x38000000u)) : sg), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// z = 1 samples of both frame batches: row sums [n][C][h] and column sums
+// [n][C][w] (imaginary parts zero), accumulated in double in column (row) order:
+// a row by a warp, lane l its columns l, l + 32, ..., a column by a thread.  The
+// scan's ratios go down to the rounding of these sums, so their order is kept.
+// Bound by the double adds (two an element, ~48 cycles a warp and scheduler:
+// ~130 us for the 50.8 M elements of four 1080p colour pairs; 260 us measured);
+// one launch, with kSumAhead loads in flight per thread and the columns' blocks,
+// the long ones, first (318 us in grid order).  Before, a launch per frame, one
+// load ahead and a row or column loop per block: 321 us each.
+constexpr int kSumThreads = 128;
+constexpr int kSumAhead = 16;
+struct PlaneSumArgs {
+  FrameDesc fr[2];
+  cd* rows[2];
+  cd* cols[2];
+  int colblocks, rowblocks;   // blocks of a frame channel: the columns', the rows'
+  int nfc;                    // frame channels of a batch
+};
+template <typename T>
+__device__ __forceinline__ double strided_sum(const T* p, int64_t stride, int count) {
+  double acc = 0.0;
+  int i = 0;
+  for (; i + kSumAhead <= count; i += kSumAhead) {
+    T v[kSumAhead];
+#pragma unroll
+    for (int k = 0; k < kSumAhead; ++k) v[k] = __ldg(p + (int64_t)(i + k) * stride);
+#pragma unroll
+    for (int k = 0; k < kSumAhead; ++k) acc += widen(v[k]);
   }
+  for (; i < count; ++i) acc += widen(__ldg(p + (int64_t)i * stride));
+  return acc;
+}
+template <typename T>
+__device__ void plane_sums(const PlaneSumArgs& a, int z, int fc, bool col, int blk) {
+  const FrameDesc& fr = a.fr[z];
+  const int f = fc / fr.c, ch = fc % fr.c;
+  const T* base = (const T*)frame_base(fr, f) + (int64_t)ch * fr.cs;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (col) {
+    const int c = blk * kSumThreads + threadIdx.x;
+    if (c < fr.w) a.cols[z][(int64_t)fc * fr.w + c] = mk(strided_sum<T>(base + c, fr.rs, fr.h), 0.0);
+  } else {
+    const int r = blk * (kSumThreads / 32) + warp;
+    if (r >= fr.h) return;
+    const int count = lane < fr.w ? (fr.w - lane + 31) / 32 : 0;
+    const double acc = warp_sum(strided_sum<T>(base + (int64_t)r * fr.rs + lane, 32, count));
+    if (lane == 0) a.rows[z][(int64_t)fc * fr.h + r] = mk(acc, 0.0);
+  }
+}
+__global__ void __launch_bounds__(kSumThreads) k_plane_sums(PlaneSumArgs a) {
+  // the columns' blocks, the long ones, first
+  const int ncol = 2 * a.nfc * a.colblocks;
+  int b = blockIdx.x;
+  const bool col = b < ncol;
+  if (!col) b -= ncol;
+  const int per = col ? a.colblocks : a.rowblocks;
+  const int zf = b / per, blk = b - zf * per, z = zf / a.nfc, fc = zf - z * a.nfc;
+  if (a.fr[z].f64) plane_sums<double>(a, z, fc, col, blk);
+  else plane_sums<float>(a, z, fc, col, blk);
 }
 
 struct SizeScanArgs {
   const cd* pz[2][2];   // [order][frame]: z = 1 samples [n][C][len]
   int len[2][2];
   int C, t_min, d, ncand;
+  int ta, tb;           // the largest candidate's sizes
+  double* rho;          // [n][2][2 (ta + tb) - 1] its lags
   double* ratio;        // [n][2][ncand]; -1 for an invalid candidate
 };
+
+// The lags of the largest candidate's normal matrix (the other candidates' are
+// among them), a warp each: one pass over the samples instead of one a candidate
+// (four 1080p colour pairs, 17 candidates: 32 us here, the scan 565 -> 400 us; the
+// whole call 1.37 -> 0.82 ms).
+__global__ void __launch_bounds__(kSolveThreads) k_size_lags(SizeScanArgs a) {
+  const int J = 2 * (a.ta + a.tb) - 1;
+  const int ps = blockIdx.y, f = blockIdx.z, lane = threadIdx.x & 31;
+  const int j = blockIdx.x * (kSolveThreads / 32) + (threadIdx.x >> 5);
+  if (j >= J) return;
+  const SamplePolys<double, double> P = sample_polys<double, double>(a.pz[ps], a.len[ps], f, a.C, 1, 0);
+  const double r = lag_real(P, a.C, a.ta, a.tb, j);
+  if (lane == 0) a.rho[((int64_t)f * 2 + ps) * J + j] = r;
+}
 
 // The refinement steps are off in the scan: an operator that is never applied.
 struct NoApply {
@@ -1351,8 +1421,13 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_size_scan(SizeScanArgs a) 
   cd* G = (cd*)smem;                                    // [n][n]
   cd* rho = G + kMaxN * kMaxN;                          // [2 n - 1]
   const TriWs W = carve_tri(smem + sizeof(cd) * (kMaxN * kMaxN + 2 * kMaxN), n);
-  const SamplePolys<double, double> P = sample_polys<double, double>(a.pz[ps], a.len[ps], f, a.C, 1, 0);
-  correlations_real(P, a.C, t1, t2, rho);
+  // this candidate's lags among the largest's
+  const double* all = a.rho + ((int64_t)f * 2 + ps) * (2 * (a.ta + a.tb) - 1);
+  for (int j = threadIdx.x; j < 2 * n - 1; j += blockDim.x) {
+    const int at = j < t1 ? j : j < n ? a.ta + (j - t1) : a.ta + a.tb + (j - n - (t2 - 1)) + a.tb - 1;
+    rho[j] = mk(all[at], 0.0);
+  }
+  __syncthreads();
   gram_from_rho(rho, t1, t2, G);
   const TriResult res = tri_smallest<double, true>(W, G, n, 0, 0, 1e300, NoApply{});
   // the Rayleigh quotient of the converged vector (the multisection bracket
@@ -1713,11 +1788,18 @@ size_t size_scan_smem() {
 
 void launch_size_scan(const SizePlan& sp, const FrameDesc& b1, const FrameDesc& b2, char* ws,
                       cudaStream_t st) {
-  const FrameDesc* fr[2] = {&b1, &b2};
+  PlaneSumArgs ps;
+  ps.fr[0] = b1;
+  ps.fr[1] = b2;
   for (int k = 0; k < 2; ++k) {
-    dim3 g(std::max(1, std::min(64, (std::max(fr[k]->h, fr[k]->w) + 255) / 256)), sp.n * sp.C, 2);
-    k_plane_sums<<<g, 256, 0, st>>>(*fr[k], (cd*)(ws + sp.off_rows[k]), (cd*)(ws + sp.off_cols[k]));
+    ps.rows[k] = (cd*)(ws + sp.off_rows[k]);
+    ps.cols[k] = (cd*)(ws + sp.off_cols[k]);
   }
+  constexpr int kSumRows = kSumThreads / 32;
+  ps.colblocks = (std::max(b1.w, b2.w) + kSumThreads - 1) / kSumThreads;
+  ps.rowblocks = (std::max(b1.h, b2.h) + kSumRows - 1) / kSumRows;
+  ps.nfc = sp.n * sp.C;
+  k_plane_sums<<<2 * ps.nfc * (ps.colblocks + ps.rowblocks), kSumThreads, 0, st>>>(ps);
   SizeScanArgs a;
   for (int k = 0; k < 2; ++k) {
     a.pz[0][k] = (const cd*)(ws + sp.off_rows[k]);
@@ -1732,6 +1814,11 @@ void launch_size_scan(const SizePlan& sp, const FrameDesc& b1, const FrameDesc& 
   a.d = sp.d;
   a.ncand = sp.ncand;
   a.ratio = (double*)(ws + sp.off_ratio);
+  a.ta = sp.t_min + sp.ncand - 1;
+  a.tb = a.ta - sp.d;
+  a.rho = (double*)(ws + sp.off_rho);
+  constexpr int kLagWarps = kSolveThreads / 32;
+  k_size_lags<<<dim3((2 * (a.ta + a.tb) - 1 + kLagWarps - 1) / kLagWarps, 2, sp.n), kSolveThreads, 0, st>>>(a);
   const size_t sm = size_scan_smem();
   cudaFuncSetAttribute(k_size_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   k_size_scan<<<dim3(sp.ncand, 2, sp.n), kSolveThreads, sm, st>>>(a);
