@@ -5,8 +5,9 @@
 //   conv 3x3 s2 p1 (2 -> 32) + ReLU, conv 3x3 s2 p1 (32 -> 32) + ReLU,
 //   conv 3x3 s4 p1 (32 -> 32) + ReLU, conv 2x2 s1 p0 (32 -> 2),
 //   softmax over each output channel's 15 x 15 logits -> K1, K2.
-// Activations are stored as bfloat16 and weights kept as float32 master
-// copies.  The forward convolutions run on the tensor cores (tcgen05, BF16
+// Activations are stored as bfloat16, a position's channels side by side
+// ([pair][position][channel]; the gradients of the hidden layers likewise in
+// float32), and weights kept as float32 master copies.  The forward convolutions run on the tensor cores (tcgen05, BF16
 // operands with the weights rounded to BF16, FP32 accumulation in tensor
 // memory) as implicit GEMMs over 128 output positions per CTA; the backward
 // pass (training only) stays on the FP32 units with the float32 weights, a
@@ -91,19 +92,40 @@ using TcT3 = ConvTcT<32, 2, 2>;
 __host__ __device__ constexpr int tct_img_offset(int li) {
   return (li > 1 ? TcT1::kBBytes : 0) + (li > 2 ? TcT1::kBBytes : 0) + (li > 3 ? TcT3::kBBytes : 0);
 }
-constexpr int kTcWPos = 64;      // positions per step: four MMAs of K = 16
-constexpr int kTcWChunk = 1024;  // positions per CTA
-__host__ __device__ constexpr int tc_mtiles(int kw) { return (kw + kTcM - 1) / kTcM; }
-int64_t tc_wchunks(int n, const Layer& L) {
-  return ((int64_t)n * L.hout * L.hout + kTcWChunk - 1) / kTcWChunk;
+// Shapes of the weight-gradient products: KW weight rows in tiles of 128,
+// kPos positions per step.  The three 128-row tiles of a 3 x 3 layer share a CTA.
+template <int CIN, int KS, int N>
+struct ConvTcW {
+  static constexpr int kW = KS * KS * CIN;
+  static constexpr int kTiles = (kW + kTcM - 1) / kTcM;
+  static constexpr int kPos = CIN == 32 && KS == 3 ? 64 : 128;
+  static constexpr int kThreads = CIN == 32 && KS == 3 ? 288 : 256;   // one per (tap, 8 channels, 8 positions)
+  static constexpr int kATile = kTcM * kPos * 2;            // bytes
+  static constexpr int kABytes = kTiles * kATile;
+  static constexpr int kBBytes = N * kPos * 2;
+  static constexpr int kSmem = 2 * (kABytes + kBBytes);
+  static constexpr uint32_t kCols = kTiles * N <= 32 ? 32 : 128;   // tensor-memory columns
+  static constexpr int kPart = kTiles * kTcM * N + N;       // floats of a chunk's partials (weights, biases)
+};
+// Positions of a layer are split into chunks, a CTA each: about two per SM.
+struct WChunks {
+  int chunk, count;
+};
+__host__ inline WChunks tc_wchunks(int64_t positions, int step) {
+  const int64_t want = (positions + 303) / 304;
+  const int64_t chunk = (want + step - 1) / step * step;
+  return {(int)chunk, (int)((positions + chunk - 1) / chunk)};
+}
+template <int CIN, int KS, int N>
+size_t tc_wpart_of(int li, int n) {
+  using W = ConvTcW<CIN, KS, N>;
+  const Layer L = cnn_layer(li);
+  return (size_t)tc_wchunks((int64_t)n * L.hout * L.hout, W::kPos).count * W::kPart;
 }
 // Floats of the partial-gradient buffer for n pairs (the largest layer's).
 size_t tc_wpart_floats(int n) {
-  size_t m = 0;
-  const int kw[4] = {18, 288, 288, 128}, nn[4] = {32, 32, 32, 16};
-  for (int li = 0; li < 4; ++li)
-    m = std::max(m, (size_t)tc_wchunks(n, cnn_layer(li)) * (tc_mtiles(kw[li]) * kTcM + 1) * nn[li]);
-  return m;
+  return std::max({tc_wpart_of<2, 3, 32>(0, n), tc_wpart_of<32, 3, 32>(1, n), tc_wpart_of<32, 3, 32>(2, n),
+                   tc_wpart_of<32, 2, 16>(3, n)});
 }
 
 
@@ -174,7 +196,7 @@ __global__ void __launch_bounds__(kCnnThreads) k_cnn_input(FrameDesc f1, FrameDe
   }
   // weights were in 1/S units of an input cell; the cell area is h w / S^2
   const float norm = 1.0f / ((float)fr.h * (float)fr.w * (float)fr.c);
-  x0[((int64_t)f * 2 + z) * kCnnSide * kCnnSide + o] = __float2bfloat16(acc * norm);
+  x0[((int64_t)f * kCnnSide * kCnnSide + o) * 2 + z] = __float2bfloat16(acc * norm);
 }
 
 // The same resampling with one CTA per output row: the input rows of the row's
@@ -269,14 +291,13 @@ k_cnn_input_rows(FrameDesc f1, FrameDesc f2, bf16* x0) {
       const int wx = min(xb, (c + 1) * kCnnSide) - max(xa, c * kCnnSide);
       acc = fmaf((float)wx, prof[c], acc);
     }
-    x0[((int64_t)f * 2 + z) * kCnnSide * kCnnSide + (int64_t)y * kCnnSide + x] =
-        __float2bfloat16(acc * norm);
+    x0[(((int64_t)f * kCnnSide + y) * kCnnSide + x) * 2 + z] = __float2bfloat16(acc * norm);
   }
 }
 
-template <typename TO> __device__ __forceinline__ TO to_out(float v);
-template <> __device__ __forceinline__ bf16 to_out<bf16>(float v) { return __float2bfloat16(v); }
-template <> __device__ __forceinline__ float to_out<float>(float v) { return v; }
+__device__ __forceinline__ uint32_t bf16_bits(float v) {
+  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16(v));
+}
 
 // Convolutions on the tensor cores (tcgen05), as implicit GEMMs:
 //   y[n][co][o] = b[co] + sum_k A[o][k] B[co][k],
@@ -285,7 +306,10 @@ template <> __device__ __forceinline__ float to_out<float>(float v) { return v; 
 // B[co][k] = w[co][ci][u][v] rounded to BF16.  A CTA takes 128 consecutive
 // output positions (tcgen05's M) and all output channels (N = 32; 16 for the
 // two-channel head, its rows 2..15 zero): its eight warps gather A from the
-// BF16 activations into shared memory, one thread issues the K / 16 MMAs into
+// BF16 activations into shared memory -- a position's channels lie next to each
+// other (NHWC), so eight channels of a tap are one 16-byte load, a sector a lane
+// pair (as planes they were eight 2-byte loads from eight planes, and the
+// gathers' latency was the kernel's time) -- one thread issues the K / 16 MMAs into
 // an FP32 accumulator in tensor memory, and each warp reads back 16 channels
 // of 32 positions for the epilogue (bias, ReLU, store).  K is padded with
 // zeros to a multiple of 16.
@@ -334,42 +358,37 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const bf16* __restrict__
   if (tid == 0) tc::bar_init(&done, 1);
   for (int i = tid; i < C::kBBytes / 16; i += kTcThreads)
     ((uint4*)sB)[i] = __ldg((const uint4*)wimg + i);
-  // A: thread-chunk (m, g) holds k = 8g .. 8g + 7 of position m0 + m; the
-  // warp's 32 chunks are 32 consecutive positions, stored as 512 contiguous bytes
-  const unsigned short* xs = reinterpret_cast<const unsigned short*>(x) + (int64_t)n * CIN * L.hin * L.hin;
-  const int64_t plane = (int64_t)L.hin * L.hin;
-#pragma unroll 2
-  for (int c = tid; c < kTcM * C::kGroups; c += kTcThreads) {
-    const int m = c & (kTcM - 1), g = c / kTcM;
-    const int o = m0 + m;
-    uint32_t q[4] = {0u, 0u, 0u, 0u};
-    if (o < npos) {
-      const int oy = o / L.hout, ox = o - oy * L.hout;
-      const int iy0 = oy * L.s - L.p, ix0 = ox * L.s - L.p;
+  // A: a thread keeps one position m and every second group g of eight k's
+  {
+    static_assert(C::kGroups % 2 == 0 && kTcThreads == 2 * kTcM, "a thread per position and half the groups");
+    const int m = tid >> 1, o = m0 + m;
+    const bool in = o < npos;
+    const int oy = o / L.hout, ox = o - oy * L.hout;
+    const int iy0 = oy * L.s - L.p, ix0 = ox * L.s - L.p;
+    const bf16* xn = x + (int64_t)n * CIN * L.hin * L.hin;
+    auto inside = [&](int tap, int& at) {
+      const int u = tap / KS, iy = iy0 + u, ix = ix0 + tap - u * KS;
+      at = iy * L.hin + ix;
+      return in && tap < KS * KS && iy >= 0 && iy < L.hin && ix >= 0 && ix < L.hin;
+    };
+#pragma unroll 6
+    for (int g = tid & 1; g < C::kGroups; g += 2) {
+      uint4 q = make_uint4(0u, 0u, 0u, 0u);
+      int at;
       if constexpr (CIN % 8 == 0) {   // the group is 8 channels of one tap
         const int tap = g / (CIN / 8), ci0 = (g - tap * (CIN / 8)) * 8;
-        const int u = tap / KS, v = tap - u * KS;
-        const int iy = iy0 + u, ix = ix0 + v;
-        if (tap < KS * KS && iy >= 0 && iy < L.hin && ix >= 0 && ix < L.hin) {
-          const unsigned short* px = xs + ci0 * plane + (int64_t)iy * L.hin + ix;
-          if (CBP_CHECK(ci0 + 7 < CIN && (int64_t)iy * L.hin + ix < plane, 0))
+        if (inside(tap, at) && CBP_CHECK(at < L.hin * L.hin && ci0 + 7 < CIN, 0))
+          q = __ldg((const uint4*)(xn + (int64_t)at * CIN + ci0));
+      } else {                        // the two channels of four taps
+        static_assert(CIN == 2 || CIN % 8 == 0, "channel pairs");
+        uint32_t* qw = &q.x;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) q[e >> 1] |= (uint32_t)__ldg(px + e * plane) << (16 * (e & 1));
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const int k = g * 8 + e;
-          const int tap = k / CIN, ci = k - tap * CIN;
-          const int u = tap / KS, v = tap - u * KS;
-          const int iy = iy0 + u, ix = ix0 + v;
-          if (tap < KS * KS && iy >= 0 && iy < L.hin && ix >= 0 && ix < L.hin)
-            q[e >> 1] |= (uint32_t)__ldg(xs + ci * plane + (int64_t)iy * L.hin + ix) << (16 * (e & 1));
-        }
+        for (int e = 0; e < 4; ++e)
+          if (inside(4 * g + e, at)) qw[e] = __ldg((const uint32_t*)(xn + (int64_t)at * CIN));
       }
+      if (CBP_CHECK(tc::kmajor_offset(kTcM, m, 8 * g) + 16 <= (uint32_t)C::kABytes, 1))
+        *(uint4*)(sA + tc::kmajor_offset(kTcM, m, 8 * g)) = q;
     }
-    if (CBP_CHECK(tc::kmajor_offset(kTcM, m, 8 * g) + 16 <= (uint32_t)C::kABytes, 1))
-      *(uint4*)(sA + tc::kmajor_offset(kTcM, m, 8 * g)) = make_uint4(q[0], q[1], q[2], q[3]);
   }
   tc::fence_smem_to_async();
   tc::fence_before_sync();
@@ -405,15 +424,27 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const bf16* __restrict__
     }
     const int o = m0 + quarter * 32 + lane;
     if (o < npos) {
-      TO* yo = y + (int64_t)n * L.cout * npos + o;
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const int co = half * 16 + j;
         if (co < L.cout) {
-          float a = v[j] + __ldg(prm + L.boff + co);
-          if (L.relu) a = fmaxf(a, 0.f);
-          yo[(int64_t)co * npos] = to_out<TO>(a);
+          v[j] += __ldg(prm + L.boff + co);
+          if (L.relu) v[j] = fmaxf(v[j], 0.f);
         }
+      }
+      if constexpr (sizeof(TO) == sizeof(bf16)) {   // 16 of the position's 32 channels
+        uint4 q[2];
+        uint32_t* w = &q[0].x;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[j] = bf16_bits(v[2 * j]) | bf16_bits(v[2 * j + 1]) << 16;
+        uint4* yo = (uint4*)(y + ((int64_t)n * npos + o) * L.cout + half * 16);
+        yo[0] = q[0];
+        yo[1] = q[1];
+      } else {                                      // the head's logits, by planes
+        TO* yo = y + (int64_t)n * L.cout * npos + o;
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (half * 16 + j < L.cout) yo[(int64_t)(half * 16 + j) * npos] = v[j];
       }
     }
   }
@@ -476,13 +507,9 @@ __global__ void k_loss_sum(const float* lossp, int m, float denom, float* out) {
   }
 }
 
-__device__ __forceinline__ uint32_t bf16_bits(float v) {
-  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16(v));
-}
-
 // Input gradients on the tensor cores, an implicit GEMM over the layer's
 // input positions i (128 per CTA):
-//   dx[n][ci][i] = [x[n][ci][i] > 0] sum_k G[i][k] W^T[ci][k],
+//   dx[n][i][ci] = [x[n][i][ci] > 0] sum_k G[i][k] W^T[ci][k],
 // k = (u KS + v) COUT + co, G[i][k] = dy[n][co][oy][ox] where iy + p - u = oy s
 // and ix + p - v = ox s land on an output position (zero elsewhere: the
 // strided transpose of the forward product), rounded to BF16, and
@@ -528,41 +555,46 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_bwd_data_tc(const float* __
   if (tid == 0) tc::bar_init(&done, 1);
   for (int i = tid; i < C::kBBytes / 16; i += kTcThreads)
     ((uint4*)sB)[i] = __ldg((const uint4*)wtimg + i);
-  const float* dyn = dy + (int64_t)n * COUT * hw;
-#pragma unroll 2
-  for (int c = tid; c < kTcM * C::kGroups; c += kTcThreads) {
-    const int m = c & (kTcM - 1), g = c / kTcM;
-    const int i = m0 + m;
-    uint32_t q[4] = {0u, 0u, 0u, 0u};
-    if (i < nin) {
-      const int iy = i / L.hin, ix = i - iy * L.hin;
+  // G: a thread keeps one input position m and every second group of eight k's;
+  // eight output channels of a tap are two 16-byte loads (the head's gradients,
+  // two channels by planes, a load each)
+  {
+    static_assert(C::kGroups % 2 == 0 && kTcThreads == 2 * kTcM, "a thread per position and half the groups");
+    const float* dyn = dy + (int64_t)n * COUT * hw;
+    const int m = tid >> 1, i = m0 + m;
+    const bool in = i < nin;
+    const int iy = i / L.hin, ix = i - iy * L.hin;
+    const int sh = __ffs(L.s) - 1, odd = L.s - 1;   // the strides are powers of two
+    auto lands = [&](int tap, int& at) {
+      const int u = tap / KS, ty = iy + L.p - u, tx = ix + L.p - (tap - u * KS);
+      at = (ty >> sh) * L.hout + (tx >> sh);
+      return in && tap < KS * KS && ty >= 0 && tx >= 0 && ((ty | tx) & odd) == 0 && (ty >> sh) < L.hout &&
+             (tx >> sh) < L.hout;
+    };
+#pragma unroll 6
+    for (int g = tid & 1; g < C::kGroups; g += 2) {
+      uint4 q = make_uint4(0u, 0u, 0u, 0u);
+      uint32_t* qw = &q.x;
+      int at;
       if constexpr (COUT % 8 == 0) {   // the group is 8 channels of one tap
         const int tap = g / (COUT / 8), co0 = (g - tap * (COUT / 8)) * 8;
-        const int u = tap / KS, v = tap - u * KS;
-        const int ty = iy + L.p - u, tx = ix + L.p - v;
-        if (tap < KS * KS && ty >= 0 && tx >= 0 && ty % L.s == 0 && tx % L.s == 0 &&
-            ty / L.s < L.hout && tx / L.s < L.hout) {
-          const float* pg = dyn + (int64_t)co0 * hw + (ty / L.s) * L.hout + tx / L.s;
-          if (CBP_CHECK(co0 + 7 < COUT && (ty / L.s) * L.hout + tx / L.s < hw, 3))
-#pragma unroll
-            for (int e = 0; e < 8; ++e) q[e >> 1] |= bf16_bits(__ldg(pg + e * hw)) << (16 * (e & 1));
+        if (lands(tap, at) && CBP_CHECK(co0 + 7 < COUT && at < hw, 3)) {
+          const float4* pg = (const float4*)(dyn + (int64_t)at * COUT + co0);
+          const float4 f0 = __ldg(pg), f1 = __ldg(pg + 1);
+          qw[0] = bf16_bits(f0.x) | bf16_bits(f0.y) << 16;
+          qw[1] = bf16_bits(f0.z) | bf16_bits(f0.w) << 16;
+          qw[2] = bf16_bits(f1.x) | bf16_bits(f1.y) << 16;
+          qw[3] = bf16_bits(f1.z) | bf16_bits(f1.w) << 16;
         }
       } else {
+        static_assert(COUT == 2 || COUT % 8 == 0, "channel pairs");
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const int k = g * 8 + e;
-          const int tap = k / COUT, co = k - tap * COUT;
-          const int u = tap / KS, v = tap - u * KS;
-          const int ty = iy + L.p - u, tx = ix + L.p - v;
-          if (tap < KS * KS && ty >= 0 && tx >= 0 && ty % L.s == 0 && tx % L.s == 0 &&
-              ty / L.s < L.hout && tx / L.s < L.hout)
-            q[e >> 1] |= bf16_bits(__ldg(dyn + (int64_t)co * hw + (ty / L.s) * L.hout + tx / L.s))
-                         << (16 * (e & 1));
-        }
+        for (int e = 0; e < 4; ++e)
+          if (lands(4 * g + e, at)) qw[e] = bf16_bits(__ldg(dyn + at)) | bf16_bits(__ldg(dyn + hw + at)) << 16;
       }
+      if (CBP_CHECK(tc::kmajor_offset(kTcM, m, 8 * g) + 16 <= (uint32_t)C::kABytes, 2))
+        *(uint4*)(sA + tc::kmajor_offset(kTcM, m, 8 * g)) = q;
     }
-    if (CBP_CHECK(tc::kmajor_offset(kTcM, m, 8 * g) + 16 <= (uint32_t)C::kABytes, 2))
-      *(uint4*)(sA + tc::kmajor_offset(kTcM, m, 8 * g)) = make_uint4(q[0], q[1], q[2], q[3]);
   }
   tc::fence_smem_to_async();
   tc::fence_before_sync();
@@ -594,12 +626,18 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_bwd_data_tc(const float* __
     for (int j = 0; j < 16; ++j) v[j] = __int_as_float(0x7fc00000);
   }
   const int i = m0 + quarter * 32 + lane;
-  if (i < nin) {
+  if (i < nin) {   // 16 of the position's 32 channels
+    const int64_t at = ((int64_t)n * nin + i) * CIN + half * 16;
+    const uint4 m0q = __ldg((const uint4*)(xact + at)), m1q = __ldg((const uint4*)(xact + at) + 1);
+    const uint32_t mw[8] = {m0q.x, m0q.y, m0q.z, m0q.w, m1q.x, m1q.y, m1q.z, m1q.w};
+    float4* o = (float4*)(dx + at);
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
-      const int64_t at = ((int64_t)n * CIN + half * 16 + j) * nin + i;
-      dx[at] = __bfloat162float(xact[at]) > 0.f ? v[j] : 0.f;
+      const float act = __uint_as_float((j & 1) ? mw[j >> 1] & 0xffff0000u : mw[j >> 1] << 16);
+      v[j] = act > 0.f ? v[j] : 0.f;
     }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -614,39 +652,44 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_bwd_data_tc(const float* __
 // over the output positions o of all pairs:
 //   D[k][co] = sum_o X[k][o] dY[co][o],
 // k = (u KS + v) CIN + ci a weight's tap and input channel, X[k][o] = the layer
-// input x[n][ci][oy s - p + u][ox s - p + v] (zero outside), dY = dy rounded to
-// BF16.  A CTA takes 128 rows of k (M) and kTcWChunk positions, in steps of
-// kTcWPos positions through two shared-memory buffers: the MMAs of one step run
-// while the other buffer is filled, each buffer's MMAs completing on its own
-// mbarrier before it is refilled.  The bias gradients sum dy itself in FP32
-// (the CTAs of the first row tile, from the values they stage).  Each CTA
-// writes its partials; a second kernel sums them over the position chunks in
-// a fixed order (deterministic) into the gradient vector.
+// input x[n][oy s - p + u][ox s - p + v][ci] (zero outside), dY = dy rounded to
+// BF16.  A CTA takes all rows of k (tiles of 128, an accumulator each) and one
+// chunk of positions, in steps of kPos through two shared-memory buffers: the
+// MMAs of one step run while the other buffer is filled, each buffer's MMAs
+// completing on its own mbarrier before it is refilled.  A thread fetches eight
+// channels of a tap at eight positions (16 bytes each) and turns the 8 x 8 block
+// in registers, since the operand wants a row's positions side by side; dY is
+// read a warp per position, a lane per channel, once for all rows.  The bias
+// gradients sum dy itself in FP32 from the values staged.  Each CTA writes its
+// partials; a second kernel sums them over the chunks in a fixed order
+// (deterministic) into the gradient vector.  Bound by the gathers' latency and by
+// L2; with a CTA per 1024 positions and row tile and 2-byte gathers from channel
+// planes the four layers took 913 us for 32 pairs (24 and 8 CTAs in the last two);
+// with the channels side by side throughout, the whole training step of 32 1080p
+// pairs went from 1.52 to 0.58 ms.
 template <int CIN, int KS, int N>
-__global__ void __launch_bounds__(kTcThreads) k_conv_bwd_w_tc(const float* __restrict__ dy,
-                                                               const bf16* __restrict__ x,
-                                                               float* __restrict__ part, Layer L,
-                                                               int npairs, int* err) {
-  constexpr int KW = KS * KS * CIN;
-  constexpr int kABytes = kTcM * kTcWPos * 2, kBBytes = N * kTcWPos * 2;
+__global__ void __launch_bounds__(ConvTcW<CIN, KS, N>::kThreads)
+k_conv_bwd_w_tc(const float* __restrict__ dy, const bf16* __restrict__ x, float* __restrict__ part,
+                Layer L, int npairs, int chunk, int* err) {
+  using W = ConvTcW<CIN, KS, N>;
+  constexpr int kNT = W::kThreads;
   extern __shared__ __align__(128) uint8_t tsm[];
   __shared__ uint64_t bars[2];
   __shared__ uint32_t tslot;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int hw = L.hout * L.hout;
-  const int64_t P = (int64_t)npairs * hw;
-  const int kk0 = blockIdx.x * kTcM;
-  const int64_t pbeg = (int64_t)blockIdx.y * kTcWChunk, pend = min(P, pbeg + kTcWChunk);
-  const int steps = (int)((pend - pbeg + kTcWPos - 1) / kTcWPos);
-  const unsigned short* xs = reinterpret_cast<const unsigned short*>(x);
-
   __shared__ float bred[8][N];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int hw = L.hout * L.hout, hin2 = L.hin * L.hin;
+  const int64_t P = (int64_t)npairs * hw;
+  const int64_t pbeg = (int64_t)blockIdx.x * chunk, pend = min(P, pbeg + chunk);
+  const int steps = (int)((pend - pbeg + W::kPos - 1) / W::kPos);
   float bsum = 0.f;   // this thread's FP32 share of the bias gradient
-  if (warp == 0) tc::tmem_alloc(&tslot, kTcCols);
+  if (warp == 0) tc::tmem_alloc(&tslot, W::kCols);
   if (tid == 0) {
     tc::bar_init(&bars[0], 1);
     tc::bar_init(&bars[1], 1);
   }
+  // rows past KW and unused channels stay zero
+  for (int i = tid; i < W::kSmem / 16; i += kNT) ((uint4*)tsm)[i] = make_uint4(0u, 0u, 0u, 0u);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -657,50 +700,79 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_bwd_w_tc(const float* __res
 #pragma unroll 1
   for (int t = 0; t < steps; ++t) {
     const int b = t & 1;
-    uint8_t* sA = tsm + b * (kABytes + kBBytes);
-    uint8_t* sB = sA + kABytes;
+    uint8_t* sA = tsm + b * (W::kABytes + W::kBBytes);
+    uint8_t* sB = sA + W::kABytes;
     // the MMAs of step t - 2 read this buffer
     if (t >= 2) ok = tc::bar_wait(&bars[b], ((t - 2) >> 1) & 1, kTcWaitLimit) && ok;
-    const int64_t ob = pbeg + (int64_t)t * kTcWPos;
-    // X rows kk0 + r, positions ob + 8 g + e; a warp's lanes are 32 consecutive rows
-    for (int c = tid; c < kTcM * (kTcWPos / 8); c += kTcThreads) {
-      const int r = c & (kTcM - 1), g = c / kTcM, kk = kk0 + r;
-      uint32_t q[4] = {0u, 0u, 0u, 0u};
-      if (kk < KW) {
-        const int tap = kk / CIN, ci = kk - tap * CIN;
-        const int u = tap / KS, v = tap - u * KS;
+    const int64_t ob = pbeg + (int64_t)t * W::kPos;
+    // X: task (tap, group of 8 positions, group of 8 channels / the channel pair)
+    constexpr int kCg = CIN == 2 ? 1 : CIN / 8;
+    constexpr int kPg = W::kPos / 8;
+    if (tid < KS * KS * kCg * kPg) {
+      const int cg = tid % kCg, pg = (tid / kCg) % kPg, tap = tid / (kCg * kPg);
+      const int u = tap / KS, v = tap - u * KS;
+      const int64_t o0 = ob + 8 * pg;
+      int pr = (int)(o0 / hw);
+      int loc = (int)(o0 - (int64_t)pr * hw);
+      int oy = loc / L.hout, ox = loc - oy * L.hout;
+      uint4 w[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const int64_t o = ob + 8 * g + e;
-          if (o >= pend) break;
-          const int pr = (int)(o / hw), loc = (int)(o - (int64_t)pr * hw);
-          const int oy = loc / L.hout, ox = loc - oy * L.hout;
-          const int iy = oy * L.s - L.p + u, ix = ox * L.s - L.p + v;
-          if (iy >= 0 && iy < L.hin && ix >= 0 && ix < L.hin)
-            q[e >> 1] |= (uint32_t)__ldg(xs + (((int64_t)pr * CIN + ci) * L.hin + iy) * L.hin + ix)
-                         << (16 * (e & 1));
+      for (int e = 0; e < 8; ++e) {
+        const int iy = oy * L.s - L.p + u, ix = ox * L.s - L.p + v;
+        w[e] = make_uint4(0u, 0u, 0u, 0u);
+        if (o0 + e < pend && iy >= 0 && iy < L.hin && ix >= 0 && ix < L.hin) {
+          const bf16* px = x + ((int64_t)pr * hin2 + iy * L.hin + ix) * CIN + 8 * cg;
+          if constexpr (CIN == 2) w[e].x = __ldg((const uint32_t*)px);
+          else w[e] = __ldg((const uint4*)px);
+        }
+        if (++ox == L.hout) {
+          ox = 0;
+          if (++oy == L.hout) {
+            oy = 0;
+            ++pr;
+          }
         }
       }
-      if (CBP_CHECK(tc::kmajor_offset(kTcM, r, 8 * g) + 16 <= (uint32_t)kABytes, 4))
-        *(uint4*)(sA + tc::kmajor_offset(kTcM, r, 8 * g)) = make_uint4(q[0], q[1], q[2], q[3]);
+      // row r = tap CIN + 8 cg + j of its 128-row tile: channel j of the eight positions
+#pragma unroll
+      for (int j = 0; j < (CIN == 2 ? 2 : 8); ++j) {
+        const int row = tap * CIN + 8 * cg + j;
+        const uint32_t sel = (j & 1) ? 0x7632u : 0x5410u;
+        uint4 q;
+        q.x = __byte_perm((&w[0].x)[j >> 1], (&w[1].x)[j >> 1], sel);
+        q.y = __byte_perm((&w[2].x)[j >> 1], (&w[3].x)[j >> 1], sel);
+        q.z = __byte_perm((&w[4].x)[j >> 1], (&w[5].x)[j >> 1], sel);
+        q.w = __byte_perm((&w[6].x)[j >> 1], (&w[7].x)[j >> 1], sel);
+        const uint32_t off = (row / kTcM) * W::kATile + tc::kmajor_offset(kTcM, row % kTcM, 8 * pg);
+        if (CBP_CHECK(off + 16 <= (uint32_t)W::kABytes, 4)) *(uint4*)(sA + off) = q;
+      }
     }
-    // dY rows co, the same positions
-    for (int c = tid; c < N * (kTcWPos / 8); c += kTcThreads) {
-      const int co = c % N, g = c / N;
-      uint32_t q[4] = {0u, 0u, 0u, 0u};
-      if (co < L.cout) {
+    // dY: channel c, eight positions a task
+    constexpr int kCo = N == 32 ? 32 : 2;       // output channels
+    for (int c = tid; c < kCo * kPg; c += kNT) {
+      const int co = c % kCo, pg = c / kCo;
+      const int64_t o0 = ob + 8 * pg;
+      float d[8];
+      if constexpr (kCo == 32) {                // [position][channel]
+#pragma unroll
+        for (int e = 0; e < 8; ++e) d[e] = o0 + e < pend ? __ldg(dy + (o0 + e) * 32 + co) : 0.f;
+      } else {                                  // the head: [pair][channel][position]
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          const int64_t o = ob + 8 * g + e;
-          if (o >= pend) break;
-          const int pr = (int)(o / hw), loc = (int)(o - (int64_t)pr * hw);
-          const float d = __ldg(dy + ((int64_t)pr * L.cout + co) * hw + loc);
-          bsum += d;
-          q[e >> 1] |= bf16_bits(d) << (16 * (e & 1));
+          const int pr = (int)((o0 + e) / hw);
+          d[e] = o0 + e < pend ? __ldg(dy + ((int64_t)pr * kCo + co) * hw + (o0 + e - (int64_t)pr * hw)) : 0.f;
         }
       }
-      if (CBP_CHECK(tc::kmajor_offset(N, co, 8 * g) + 16 <= (uint32_t)kBBytes, 5))
-        *(uint4*)(sB + tc::kmajor_offset(N, co, 8 * g)) = make_uint4(q[0], q[1], q[2], q[3]);
+      uint4 q;
+      uint32_t* qw = &q.x;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        bsum += d[2 * e];
+        bsum += d[2 * e + 1];
+        qw[e] = bf16_bits(d[2 * e]) | bf16_bits(d[2 * e + 1]) << 16;
+      }
+      if (CBP_CHECK(tc::kmajor_offset(N, co, 8 * pg) + 16 <= (uint32_t)W::kBBytes, 5))
+        *(uint4*)(sB + tc::kmajor_offset(N, co, 8 * pg)) = q;
     }
     tc::fence_smem_to_async();
     tc::fence_before_sync();
@@ -709,23 +781,39 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_bwd_w_tc(const float* __res
     if (late) break;
     if (tid == 0) {
       const uint32_t a0 = tc::saddr(sA), b0 = tc::saddr(sB);
+#pragma unroll 1
+      for (int m = 0; m < W::kTiles; ++m)
 #pragma unroll
-      for (int s = 0; s < kTcWPos / 16; ++s)
-        tc::mma_bf16(tmem, tc::sdesc(a0 + 2 * s * kTcM * 16, kTcM * 16, 128),
-                     tc::sdesc(b0 + 2 * s * N * 16, N * 16, 128), idesc, t > 0 || s > 0);
+        for (int s = 0; s < W::kPos / 16; ++s)
+          tc::mma_bf16(tmem + m * N, tc::sdesc(a0 + m * W::kATile + 2 * s * kTcM * 16, kTcM * 16, 128),
+                       tc::sdesc(b0 + 2 * s * N * 16, N * 16, 128), idesc, t > 0 || s > 0);
       tc::mma_commit(&bars[b]);
     }
     ++issued;
   }
-  // the bias partial of this chunk: the eight position groups in order
-  // (every thread c < 8 N staged one (co, g) in each step)
-  if (tid < 8 * N) bred[tid / N][tid % N] = bsum;
-  __syncthreads();
-  if (blockIdx.x == 0 && tid < N) {
-    float b = 0.f;
+  // the bias partial of this chunk: a thread's channel is tid mod 32 (the head:
+  // mod 2) in every step and task; its threads in order
+  float* pc = part + (int64_t)blockIdx.x * W::kPart;
+  if constexpr (N == 32) {
+    if (warp < 8) bred[warp][lane] = bsum;
+    __syncthreads();
+    if (tid < N) {
+      float s = 0.f;
 #pragma unroll
-    for (int g = 0; g < 8; ++g) b += bred[g][tid];
-    part[(int64_t)gridDim.y * gridDim.x * kTcM * N + (int64_t)blockIdx.y * N + tid] = b;
+      for (int g = 0; g < 8; ++g) s += bred[g][tid];
+      pc[W::kTiles * kTcM * N + tid] = s;
+    }
+  } else {
+#pragma unroll
+    for (int o = 16; o > 1; o >>= 1) bsum += __shfl_xor_sync(0xffffffffu, bsum, o);
+    if (lane < 2 && warp < 8) bred[warp][lane] = bsum;
+    __syncthreads();
+    if (tid < N) {
+      float s = 0.f;
+      if (tid < 2)
+        for (int g = 0; g < 8; ++g) s += bred[g][tid];
+      pc[W::kTiles * kTcM * N + tid] = s;
+    }
   }
   // the last commit completes after every MMA issued before it
   bool fin = true;
@@ -739,45 +827,56 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_bwd_w_tc(const float* __res
   }
   tc::fence_after_sync();
   const int quarter = warp & 3, half = warp >> 2;
-  if (half * 16 < N) {
-    float v[16];
-    if (!bad) {
-      tc::tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + half * 16, v);
-    } else {
+  if (half * 16 < N && warp < 8) {
+#pragma unroll 1
+    for (int m = 0; m < W::kTiles; ++m) {
+      float v[16];
+      if (!bad) {
+        tc::tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + m * N + half * 16, v);
+      } else {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = __int_as_float(0x7fc00000);
+        for (int j = 0; j < 16; ++j) v[j] = __int_as_float(0x7fc00000);
+      }
+      float4* o = (float4*)(pc + (int64_t)(m * kTcM + quarter * 32 + lane) * N + half * 16);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) o[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
     }
-    float4* o = (float4*)(part + (((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kTcM + quarter * 32 +
-                                  lane) * N + half * 16);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) o[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
   }
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) {
     tc::fence_after_sync();
-    tc::tmem_free(tmem, kTcCols);
+    tc::tmem_free(tmem, W::kCols);
   }
 }
 
-// The gradient vector from the partials, summed over the position chunks in
-// order: weights [co][ci][u][v] from rows k < KS^2 CIN, then the biases.
+// The gradient vector from the partials, summed over the position chunks in a
+// fixed order (eight runs of chunks, then the runs): weights [co][ci][u][v] from
+// rows k < KS^2 CIN, then the biases.
+constexpr int kWSumOut = 32, kWSumRuns = 8;
 template <int CIN, int KS, int N>
-__global__ void k_conv_bwd_w_sum(const float* __restrict__ part, float* __restrict__ grad, Layer L,
-                                 int nchunks, int mtiles) {
-  constexpr int KW = KS * KS * CIN;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (KW + 1) * L.cout) return;
+__global__ void __launch_bounds__(kWSumOut * kWSumRuns)
+k_conv_bwd_w_sum(const float* __restrict__ part, float* __restrict__ grad, Layer L, int nchunks) {
+  using W = ConvTcW<CIN, KS, N>;
+  __shared__ float run[kWSumRuns][kWSumOut];
+  const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+  const int idx = blockIdx.x * kWSumOut + lane;
+  const bool in = idx < (W::kW + 1) * L.cout;
   const int kk = idx / L.cout, co = idx - kk * L.cout;
+  const float* p = part + (kk < W::kW ? kk * N + co : W::kTiles * kTcM * N + co);
+  const int per = (nchunks + kWSumRuns - 1) / kWSumRuns, c1 = min(nchunks, (r + 1) * per);
   float s = 0.f;
-  if (kk < KW) {
-    for (int c = 0; c < nchunks; ++c)
-      s += part[(((int64_t)c * mtiles + kk / kTcM) * kTcM + kk % kTcM) * N + co];
-  } else {
-    const float* bp = part + (int64_t)nchunks * mtiles * kTcM * N;
-    for (int c = 0; c < nchunks; ++c) s += bp[(int64_t)c * N + co];
+  if (in) {
+#pragma unroll 8
+    for (int c = r * per; c < c1; ++c) s += p[(int64_t)c * W::kPart];
   }
-  if (kk < KW) {
+  run[r][lane] = s;
+  __syncthreads();
+  if (r != 0 || !in) return;
+  s = 0.f;
+#pragma unroll
+  for (int g = 0; g < kWSumRuns; ++g) s += run[g][lane];
+  if (kk < W::kW) {
     const int tap = kk / CIN, ci = kk - tap * CIN;
     grad[L.woff + (co * CIN + ci) * KS * KS + tap] = s;
   } else {
@@ -788,15 +887,14 @@ __global__ void k_conv_bwd_w_sum(const float* __restrict__ part, float* __restri
 template <int CIN, int KS, int N>
 void run_bwd_w_tc(const float* dy, const bf16* x, float* part, float* grad, int li, int n, int* err,
                   cudaStream_t st) {
+  using W = ConvTcW<CIN, KS, N>;
   const Layer L = cnn_layer(li);
-  constexpr int KW = KS * KS * CIN;
-  const int mt = tc_mtiles(KW);
-  const int nch = (int)tc_wchunks(n, L);
-  const int sm = 2 * (kTcM * kTcWPos * 2 + N * kTcWPos * 2);
+  const WChunks wc = tc_wchunks((int64_t)n * L.hout * L.hout, W::kPos);
   auto kfn = k_conv_bwd_w_tc<CIN, KS, N>;
-  cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  kfn<<<dim3(mt, nch), kTcThreads, sm, st>>>(dy, x, part, L, n, err);
-  k_conv_bwd_w_sum<CIN, KS, N><<<((KW + 1) * L.cout + 255) / 256, 256, 0, st>>>(part, grad, L, nch, mt);
+  cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, W::kSmem);
+  kfn<<<wc.count, W::kThreads, W::kSmem, st>>>(dy, x, part, L, n, wc.chunk, err);
+  k_conv_bwd_w_sum<CIN, KS, N><<<((W::kW + 1) * L.cout + kWSumOut - 1) / kWSumOut, kWSumOut * kWSumRuns, 0, st>>>(
+      part, grad, L, wc.count);
 }
 
 template <int CIN, int KS, int COUT>
@@ -825,10 +923,14 @@ __global__ void k_adamw(float* p, const float* g, float* m, float* v, int count,
   p[i] -= hp.lr * mh / (sqrtf(vh) + hp.eps) + hp.lr * hp.weight_decay * p[i];
 }
 
-__global__ void k_bf16_to_f32(const bf16* a, float* b, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    b[i] = __bfloat162float(a[i]);
+// [pair][position][channel] -> float [pair][channel][position]
+__global__ void k_planes_f32(const bf16* a, float* b, int n, int c, int hw) {
+  const int64_t total = (int64_t)n * c * hw;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t pc = i / hw, pos = i - pc * hw, pr = pc / c;
+    b[i] = __bfloat162float(a[(pr * hw + pos) * c + (pc - pr * c)]);
+  }
 }
 
 // Proposals into the double kernel buffer [n][t1^2 + t2^2] of the estimation
@@ -851,8 +953,8 @@ void launch_conv_fwd(const bf16* x, const uint8_t* wimg, const float* prm, void*
   }
 }
 
-void copy_f32(const bf16* a, float* b, int64_t n, cudaStream_t st) {
-  if (b) k_bf16_to_f32<<<256, 256, 0, st>>>(a, b, n);
+void copy_planes(const bf16* a, float* b, int n, int c, int hw, cudaStream_t st) {
+  if (b) k_planes_f32<<<256, 256, 0, st>>>(a, b, n, c, hw);
 }
 
 }  // namespace
@@ -878,10 +980,10 @@ void cnn_forward(const FrameDesc& b1, const FrameDesc& b2, int n, const float* p
   k_softmax<<<(n * 2 * 32 + 127) / 128, 128, 0, st>>>((const float*)(ws + L.z4), (float*)(ws + L.k),
                                                       nullptr, nullptr, nullptr, n);
   if (tr) {
-    copy_f32(x0, tr->input, (int64_t)n * 2 * kCnnSide * kCnnSide, st);
+    copy_planes(x0, tr->input, n, 2, kCnnSide * kCnnSide, st);
     for (int i = 0; i < 3; ++i) {
       const Layer Ly = cnn_layer(i);
-      copy_f32(a[i], tr->act[i], (int64_t)n * Ly.cout * Ly.hout * Ly.hout, st);
+      copy_planes(a[i], tr->act[i], n, Ly.cout, Ly.hout * Ly.hout, st);
     }
     if (tr->logits)
       cudaMemcpyAsync(tr->logits, ws + L.z4, (size_t)n * 2 * kT2 * 4, cudaMemcpyDeviceToDevice, st);
