@@ -13,9 +13,9 @@
 //     does not fit; a request that cannot fit even alone fails with
 //     CBP_ERR_BUDGET;
 //   - runs each batch on one of kSlots streams as a CUDA graph captured once
-//     per (slot, bucket, batch size): the graph owns a fixed workspace and
-//     reads the per-pair addresses from device tables that are refreshed
-//     before each replay;
+//     per (bucket, batch size) running at a time: the graph owns a fixed
+//     workspace, reads the per-pair addresses from device tables that are
+//     refreshed before each replay, and runs on whichever stream is free;
 //   - notices completion by event polling, records per-request latency
 //     (submit to completion) and wakes pollers.
 // The kernels treat every pair of a batch independently, so a request's
@@ -33,9 +33,15 @@
 namespace cbp {
 namespace serve {
 
-constexpr int kSlots = 4;          // concurrent batches, one stream each
+constexpr int kSlots = 8;          // concurrent batches, one stream each (as many as the process's
+                                   // hardware queues let run: with four of them 2.31 ms for 16
+                                   // cameras' requests, with eight 1.60, against 2.53 and 2.5 with
+                                   // four slots)
 constexpr int kMaxBatch = 16;      // requests per batch
-constexpr int kCachePerSlot = 8;   // captured batches kept per slot
+// Captured batches kept, whatever the streams.  (A cache of eight per stream
+// captured a batch again, ~0.35 ms of the scheduler's time, whenever the stream
+// that was free had not run it before: with sixteen cameras, on every pass.)
+constexpr int kCache = 64;
 constexpr int kTables = 5;         // b1, b2, k1, k2, latent addresses
 using Clock = std::chrono::steady_clock;
 
@@ -100,6 +106,8 @@ struct Entry {
   uint64_t* tab = nullptr;    // device [kTables][B]
   cudaGraphExec_t exec = nullptr;
   uint64_t last_use = 0;
+  cudaStream_t st = nullptr;  // the stream its memory was allocated on
+  bool busy = false;          // its batch is on the GPU
 };
 
 struct Slot {
@@ -111,7 +119,6 @@ struct Slot {
   std::vector<Request*> batch;
   Entry* cur = nullptr;
   bool busy = false;
-  std::vector<Entry*> cache;
 };
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -129,6 +136,7 @@ struct ServeState {
   std::unordered_map<uint64_t, Request*> tickets;
   uint64_t next_ticket = 1, tick = 0;
   Slot slots[kSlots];
+  std::vector<Entry*> cache;        // captured batches (scheduler thread only, like the slots)
   bool stop = false, ready = false;
   cbp_status init_status = CBP_OK;
   std::vector<double> lat_ms;
@@ -145,11 +153,25 @@ struct ServeState {
     ++completed;
   }
 
-  void free_entry(Slot& s, Entry* e) {
+  // An idle entry: its last batch's completion has been seen on the host, so
+  // the order of streams does not matter.
+  void free_entry(Entry* e) {
     if (e->exec) cudaGraphExecDestroy(e->exec);
-    if (e->mem) cudaFreeAsync(e->mem, s.st);
+    if (e->mem) cudaFreeAsync(e->mem, e->st);
     ctx->release(e->bytes);
     delete e;
+  }
+
+  // Free the idle cached batch used least recently; false if none is idle.
+  bool evict_one() {
+    auto it = cache.end();
+    for (auto i = cache.begin(); i != cache.end(); ++i)
+      if (!(*i)->busy && (it == cache.end() || (*i)->last_use < (*it)->last_use)) it = i;
+    if (it == cache.end()) return false;
+    Entry* e = *it;
+    cache.erase(it);
+    free_entry(e);
+    return true;
   }
 
   // Free idle cached batches, least recently used first, until `bytes` more
@@ -160,21 +182,7 @@ struct ServeState {
         std::lock_guard<std::mutex> g(ctx->mem_mu);
         if (ctx->used + bytes <= ctx->budget) return;
       }
-      Slot* bs = nullptr;
-      size_t bi = 0;
-      for (Slot& s : slots)
-        for (size_t i = 0; i < s.cache.size(); ++i) {
-          Entry* e = s.cache[i];
-          if (s.busy && e == s.cur) continue;
-          if (!bs || e->last_use < bs->cache[bi]->last_use) {
-            bs = &s;
-            bi = i;
-          }
-        }
-      if (!bs) return;
-      Entry* e = bs->cache[bi];
-      bs->cache.erase(bs->cache.begin() + bi);
-      free_entry(*bs, e);
+      if (!evict_one()) return;
     }
   }
 
@@ -201,6 +209,7 @@ struct ServeState {
     e->B = B;
     e->plan = p;
     e->bytes = bytes;
+    e->st = s.st;
     if (cudaMallocAsync((void**)&e->mem, bytes, s.st) != cudaSuccess) {
       cudaGetLastError();
       e->mem = nullptr;
@@ -229,18 +238,13 @@ struct ServeState {
     if (rs != CBP_OK) {
       cudaGetLastError();
       e->exec = nullptr;
-      free_entry(s, e);
+      free_entry(e);
       *st = rs;
       return nullptr;
     }
-    if ((int)s.cache.size() >= kCachePerSlot) {
-      auto it = std::min_element(s.cache.begin(), s.cache.end(),
-                                 [](Entry* a, Entry* b) { return a->last_use < b->last_use; });
-      Entry* old = *it;
-      s.cache.erase(it);
-      free_entry(s, old);
+    while ((int)cache.size() >= kCache && evict_one()) {
     }
-    s.cache.push_back(e);
+    cache.push_back(e);
     return e;
   }
 
@@ -250,7 +254,7 @@ struct ServeState {
     return false;
   }
 
-  void launch(Slot& s, Entry* e, std::vector<Request*>& batch) {
+  void launch(Slot& s, Entry* e, std::vector<Request*>& batch, std::unique_lock<std::mutex>& lk) {
     NvtxScope range("cbp.serve_batch");
     const int B = e->B;
     for (int i = 0; i < B; ++i) {
@@ -261,6 +265,7 @@ struct ServeState {
       s.tab_host[3 * B + i] = (uint64_t)r->k2;
       s.tab_host[4 * B + i] = (uint64_t)r->lat;
     }
+    lk.unlock();
     bool ok = cudaEventRecord(s.t0, s.st) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(e->tab, s.tab_host, (size_t)kTables * B * sizeof(uint64_t),
                                cudaMemcpyHostToDevice, s.st) == cudaSuccess;
@@ -269,7 +274,9 @@ struct ServeState {
     ok = ok && cudaMemcpyAsync(s.diag_host, e->mem + e->plan.off_diag, (size_t)B * sizeof(cbp_diag),
                                cudaMemcpyDeviceToHost, s.st) == cudaSuccess;
     ok = ok && cudaEventRecord(s.ev, s.st) == cudaSuccess;
+    lk.lock();
     e->last_use = ++tick;
+    e->busy = true;
     s.batch = batch;
     s.cur = e;
     s.busy = true;
@@ -279,21 +286,17 @@ struct ServeState {
       const auto now = Clock::now();
       for (Request* r : s.batch) finish(r, CBP_ERR_CUDA, nullptr, now);
       s.batch.clear();
-      s.busy = false;
+      s.busy = e->busy = false;
       done_cv.notify_all();
     }
   }
 
-  // Admit and launch pending batches while a slot is free.
-  void schedule() {
+  // Admit and launch pending batches while a slot is free.  Slots, caches and
+  // captured batches belong to the scheduler thread alone, and a request taken
+  // from `pending` is not released before it is done, so the lock is given up
+  // while a batch is captured or launched: submitters go on meanwhile.
+  void schedule(std::unique_lock<std::mutex>& lk) {
     while (!pending.empty()) {
-      Slot* s = nullptr;
-      for (Slot& x : slots)
-        if (!x.busy) {
-          s = &x;
-          break;
-        }
-      if (!s) return;
       Request* r0 = pending.front();
       const Bucket key = bucket_of(*r0);
       std::vector<Request*> batch;
@@ -302,21 +305,32 @@ struct ServeState {
           batch.push_back(r);
           if ((int)batch.size() == kMaxBatch) break;
         }
-      // a cached graph of exactly this size, else a new one; when memory is
-      // short, the largest cached one that fits, else halve
+      Slot* s = nullptr;
+      for (Slot& x : slots)
+        if (!x.busy) {
+          s = &x;
+          break;
+        }
+      if (!s) return;
+      // an idle captured batch of exactly this size, else a new one; when memory
+      // is short, the largest captured one that fits, else halve
       auto cached = [&](int maxB, bool exact) {
         Entry* best = nullptr;
-        for (Entry* c : s->cache)
-          if (same(c->key, key) && (exact ? c->B == maxB : c->B <= maxB) && (!best || c->B > best->B))
+        for (Entry* c : cache)
+          if (!c->busy && same(c->key, key) && (exact ? c->B == maxB : c->B <= maxB) && (!best || c->B > best->B))
             best = c;
         return best;
       };
       const int want = (int)batch.size();
       cbp_status st = CBP_OK;
       Entry* e = cached(want, true);
-      if (!e) e = create_entry(*s, key, want, *r0, &st);
-      if (!e && st == CBP_OK) e = cached(want, false);
-      for (int B = want / 2; B >= 1 && !e && st == CBP_OK; B /= 2) e = create_entry(*s, key, B, *r0, &st);
+      if (!e) {
+        lk.unlock();
+        e = create_entry(*s, key, want, *r0, &st);
+        if (!e && st == CBP_OK) e = cached(want, false);
+        for (int B = want / 2; B >= 1 && !e && st == CBP_OK; B /= 2) e = create_entry(*s, key, B, *r0, &st);
+        lk.lock();
+      }
       if (!e) {
         if (st == CBP_OK && any_busy()) return;   // wait for memory to come back
         // cannot run even alone (or cannot be planned / captured): fail it
@@ -327,7 +341,7 @@ struct ServeState {
       }
       batch.resize(e->B);
       for (Request* r : batch) pending.erase(std::find(pending.begin(), pending.end(), r));
-      launch(*s, e, batch);
+      launch(*s, e, batch, lk);
     }
   }
 
@@ -352,7 +366,7 @@ struct ServeState {
         finish(s.batch[i], q == cudaSuccess ? (cbp_status)d.status : CBP_ERR_CUDA, &d, now);
       }
       s.batch.clear();
-      s.busy = false;
+      s.busy = s.cur->busy = false;
       done_cv.notify_all();
     }
   }
@@ -378,16 +392,16 @@ struct ServeState {
     if (is == CBP_OK) {
       for (;;) {
         reap();
-        schedule();
+        schedule(lk);
         const bool busy = any_busy();
         if (stop && pending.empty() && !busy) break;
         if (busy) wake.wait_for(lk, std::chrono::microseconds(50));
         else wake.wait(lk, [&] { return stop || !pending.empty(); });
       }
     }
+    for (Entry* e : cache) free_entry(e);
+    cache.clear();
     for (Slot& s : slots) {
-      for (Entry* e : s.cache) free_entry(s, e);
-      s.cache.clear();
       if (s.st) cudaStreamSynchronize(s.st);
       if (s.ev) cudaEventDestroy(s.ev);
       if (s.t0) cudaEventDestroy(s.t0);
