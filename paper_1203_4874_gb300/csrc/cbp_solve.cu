@@ -8,8 +8,8 @@
 // the normal matrix G = S^H S is formed on the device from correlations --
 // its blocks are Toeplitz, (C_t(a)^H C_s(b))[p][q] = rho_ab(p - q) with
 // rho_ab(d) = sum_m conj(a[m]) b[m + d] -- by one CTA per sample
-// (k_sample_gram), and its smallest eigenvector is found by one warp per
-// sample (k_sample_solve, cbp_tri.cuh):
+// (k_sample_gram), and its smallest eigenvector is found by one CTA per
+// sample (k_sample_solve, cbp_tri_team.cuh):
 //   1. Householder reduction to a real tridiagonal T in double precision;
 //   2. Sturm-count multisection for the two smallest eigenvalues of T;
 //   3. inverse iteration on T, x = Q y;
@@ -40,22 +40,6 @@ CBP_CHECKS_TU(kChkSolve)
 namespace {
 
 constexpr int kSolveThreads = 256;
-#ifndef CBP_SOLVE_WPC
-#define CBP_SOLVE_WPC 4      // complex samples per CTA of the sample solve (a warp each)
-#endif
-#ifndef CBP_TEAM_CTAS
-// Up to this many samples a call, each complex one has a CTA to itself: two per
-// SM.  Mixed path: a CTA per sample takes half a warp's time for one, but four
-// warps a CTA fill the GPU's schedulers better once there are more samples than
-// that (60 1080p pairs, 540 samples a chunk: 6.45 ms against 6.48).  FP64 path:
-// the double units bound either form and the CTA's needs fewer double
-// instructions (40 pairs of 25 / 20 kernels, 520 samples a chunk: 4.44 ms
-// against 5.19; 30 480p pairs, 180 samples a chunk: 1.71 against 2.33).
-#define CBP_TEAM_CTAS 304
-#endif
-#ifndef CBP_TEAM_CTAS_F64
-#define CBP_TEAM_CTAS_F64 4096
-#endif
 
 // Optional per-phase cycle counts (build with -DCBP_PHASE_TIMING): thread 0 of
 // a few blocks prints the clock64 deltas between the solver's phases.
@@ -134,7 +118,6 @@ struct SampleArgs {
   int Lmax, C, ns, t1, t2, nn, M, mixed;
   int nfr;                   // pairs in the call
   int gsplit;                // CTAs a sample's lags are split over (normal matrices)
-  int wpc;                   // complex samples (warps) per CTA, when not a CTA each
 };
 
 // Sample polynomial element m of frame k (0: b1, 1: b2) as cpx<TA>.
@@ -376,11 +359,10 @@ __device__ void gram_from_rho(const cd* rho, int t1, int t2, cd* G, LagSplit sp 
 #include "cbp_tri_team.cuh"
 
 // S^H S x from the double samples (the exact operator of the refinement
-// steps; y holds S x), by the whole CTA (BLOCK) or by the calling warp.
+// steps; y holds S x), by the whole CTA.
 // S = [-C_t1(b2) | C_t2(b1)] (channels' rows stacked):
 //   (S x)[ch][i] = sum_q b1[ch][i - q] v_q - sum_p b2[ch][i - p] u_p,
 //   (S^H y)_u[p] = -sum_ch sum_m conj(b2[ch][m]) y[ch][m + p], likewise v with b1.
-template <bool BLOCK>
 struct SylvesterApply {
   SamplePolys<double, double> P;
   const cdf* F[2];  // float-float samples (mixed path, complex samples) or null: read instead of P
@@ -396,13 +378,8 @@ struct SylvesterApply {
   float2* part = nullptr;
   __device__ void operator()(const cd* x, cd* out) const {
     if (real) {
-      if constexpr (BLOCK) {
-        if (F[0]) {
-          run_ff_real(x, out);
-          return;
-        }
-      }
-      run<true, false>(x, out);
+      if (F[0]) run_ff_real(x, out);
+      else run<true, false>(x, out);
     } else if (F[0]) {
       run<false, true>(x, out);
     } else {
@@ -428,7 +405,7 @@ struct SylvesterApply {
     // one channel at a time: both polynomials (hi, lo) and that channel's S x
     // in shared memory when they fit, else read and written in place
     const bool stage = ys && ys_cap >= L + len0 + len1;
-    team_sync<BLOCK>();
+    __syncthreads();
     for (int i = threadIdx.x; i < n; i += nth) {
       const float h = (float)x[i].re;
       xf[i] = make_float2(h, (float)(x[i].re - (double)h));
@@ -442,7 +419,7 @@ struct SylvesterApply {
       const float2* pb[2] = {g0, g1};
       int bs = 2;                              // float2 per coefficient
       float2* yc = reinterpret_cast<float2*>(y) + ch * L;
-      team_sync<BLOCK>();                      // the last channel's reads are done
+      __syncthreads();                      // the last channel's reads are done
       if (stage) {
         float2* s0 = ys + L;
         float2* s1 = s0 + len0;
@@ -458,7 +435,7 @@ struct SylvesterApply {
         pb[1] = s1;
         bs = 1;
         yc = ys;
-        team_sync<BLOCK>();
+        __syncthreads();
       }
       // y = S x: each thread R consecutive outputs, the coefficient window slid
       // by one per term (R independent sums)
@@ -493,7 +470,7 @@ struct SylvesterApply {
           }
         }
       }
-      team_sync<BLOCK>();
+      __syncthreads();
       // S^H y, this channel's terms: lane <-> output o, warp <-> a slice of
       // the terms; four sums per lane (renormalised every 16 terms)
 #pragma unroll
@@ -541,7 +518,7 @@ struct SylvesterApply {
       const int o = 32 * c + lane;
       if (o < n) part[wid * n + o] = make_float2(tot[c].hi, tot[c].lo);
     }
-    team_sync<BLOCK>();
+    __syncthreads();
     for (int o = threadIdx.x; o < n; o += nth) {
       double s = 0.0;
       for (int w = 0; w < nw; ++w) {
@@ -550,7 +527,7 @@ struct SylvesterApply {
       }
       out[o] = o < t1 ? mk(-s, 0.0) : mk(s, 0.0);
     }
-    team_sync<BLOCK>();
+    __syncthreads();
   }
   template <bool FFS>
   __device__ __forceinline__ cd ld(const void* row, int m) const {
@@ -567,10 +544,9 @@ struct SylvesterApply {
   template <bool REAL, bool FFS>
   __device__ void run(const cd* x, cd* out) const {
     const int lane = threadIdx.x & 31;
-    const int tid = BLOCK ? threadIdx.x : lane, nth = BLOCK ? blockDim.x : 32;
-    const int wid = BLOCK ? threadIdx.x >> 5 : 0, nw = BLOCK ? blockDim.x >> 5 : 1;
+    const int tid = threadIdx.x, nth = blockDim.x, wid = tid >> 5, nw = nth >> 5;
     const int len0 = P.len[0], len1 = P.len[1];
-    team_sync<BLOCK>();
+    __syncthreads();
     for (int idx = tid; idx < C * L; idx += nth) {
       const int ch = idx / L, i = idx - ch * L;
       const void* r0 = row(0, ch, FFS);
@@ -595,7 +571,7 @@ struct SylvesterApply {
       }
       y[idx] = acc;
     }
-    team_sync<BLOCK>();
+    __syncthreads();
     const int n = t1 + t2;
     for (int o = wid; o < n; o += nw) {
       const int k = o < t1 ? 1 : 0;       // u rows use b2, v rows use b1
@@ -614,7 +590,7 @@ struct SylvesterApply {
       const double re = warp_sum(acc.re), im = REAL ? 0.0 : warp_sum(acc.im);
       if (lane == 0) out[o] = o < t1 ? mk(-re, -im) : mk(re, im);
     }
-    team_sync<BLOCK>();
+    __syncthreads();
   }
 };
 
@@ -640,11 +616,14 @@ __global__ void __launch_bounds__(kSolveThreads) k_sample_gram(SampleArgs a) {
 
 // A3: the null vector of every sample's normal matrix (tridiagonal
 // reduction, Sturm multisection, inverse iteration, refinement steps against
-// S^H S as configured below).  The first nreal CTAs take one real sample each
-// (z = 1, and z = -1 for even M: their refinement, the costliest step, runs
-// on the whole CTA).  TEAM: the others take one complex sample each as well;
-// else one complex sample per warp.
-template <bool TEAM>
+// S^H S as configured below), a CTA a sample; the real samples (z = 1, and
+// z = -1 for even M), whose refinement is the longest, come first.  One form for
+// every batch, so that a pair's kernels do not depend on its neighbours.  A warp
+// a sample, four to a CTA, fills the schedulers a little better once there are
+// several samples to an SM (60 1080p pairs, 540 samples a chunk: 6.45 ms against
+// 6.48), takes twice as long for one, and on the FP64 path, where the double
+// units bound either form, loses throughout (40 pairs of 25 / 20 kernels, 520
+// samples a chunk: 5.19 ms against 4.44).
 __global__ void __launch_bounds__(kTeamThreads, 3) k_sample_solve(SampleArgs a, int nreal) {
   extern __shared__ __align__(16) char smem[];
 #ifdef CBP_SCHED_TRACE
@@ -662,18 +641,16 @@ __global__ void __launch_bounds__(kTeamThreads, 3) k_sample_solve(SampleArgs a, 
     ps = (r / nrs) & 1;
     s = (r % nrs) ? a.M / 2 : 0;
   } else {
-    const int b = (int)blockIdx.x - nreal, c = TEAM ? b : b * a.wpc + warp;
-    if (c >= a.nfr * 2 * ncs || (!TEAM && warp >= a.wpc)) return;   // whole warp leaves together
+    const int c = (int)blockIdx.x - nreal;
+    if (c >= a.nfr * 2 * ncs) return;
     f = c / (2 * ncs);
     ps = (c / ncs) & 1;
     s = 1 + c % ncs;
   }
   if (a.accepted && a.accepted[f]) return;   // the proposal stands; nothing to solve
-  // a sample's whole CTA, or its warp, leaves together
   if (!CBP_CHECK(f < a.nfr && s < a.ns && n <= kMaxN, 2)) return;
   const int64_t o = ((int64_t)f * 2 + ps) * a.ns + s;
-  const bool whole = TEAM || real;             // the CTA works on this sample
-  const TriWs W = carve_tri(smem + (whole ? 0 : (size_t)warp * tri_ws_bytes(n)), n);
+  const TriWs W = carve_tri(smem, n);
   const cd* G = a.G + o * n * n;
 #ifdef CBP_PHASE_TIMING
   long long tkv[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -689,49 +666,36 @@ __global__ void __launch_bounds__(kTeamThreads, 3) k_sample_solve(SampleArgs a, 
   // leaves ~1e-4 in x), none elsewhere.
   const int far = a.mixed ? 0 : 1;
   const double gap = a.mixed ? 1e-6 : 1e-4;
-  auto setup = [&](auto& ap) {
-    ap.P = sample_polys<double, double>(a.pz[ps], a.len[ps], f, a.C, a.ns, s);
-    ap.C = a.C;
-    ap.t1 = a.t1;
-    ap.t2 = a.t2;
-    ap.L = a.len[ps][0] + a.t2 - 1;
-    ap.y = a.resid + o * a.C * (int64_t)a.Lmax;
-    ap.F[0] = ap.F[1] = nullptr;
-    if (a.mixed) {   // real samples: the step in float-float; complex ones are kept as float-float pairs only
-      for (int k = 0; k < 2; ++k) {
-        ap.F[k] = a.pzf[ps][k] + ((int64_t)f * a.C * a.ns + s) * a.len[ps][k];
-        ap.fstride[k] = (int64_t)a.len[ps][k] * a.ns;
-      }
+  SylvesterApply ap;
+  ap.P = sample_polys<double, double>(a.pz[ps], a.len[ps], f, a.C, a.ns, s);
+  ap.C = a.C;
+  ap.t1 = a.t1;
+  ap.t2 = a.t2;
+  ap.L = a.len[ps][0] + a.t2 - 1;
+  ap.y = a.resid + o * a.C * (int64_t)a.Lmax;
+  ap.F[0] = ap.F[1] = nullptr;
+  if (a.mixed) {   // real samples: the step in float-float; complex ones are kept as float-float pairs only
+    for (int k = 0; k < 2; ++k) {
+      ap.F[k] = a.pzf[ps][k] + ((int64_t)f * a.C * a.ns + s) * a.len[ps][k];
+      ap.fstride[k] = (int64_t)a.len[ps][k] * a.ns;
     }
-    ap.real = real;
-  };
+  }
+  ap.real = real;
   TriResult res;
   if (real) {
-    SylvesterApply<true> ap;
-    setup(ap);
     ap.part = reinterpret_cast<float2*>(W.part);   // free once the reduction is done
-    {
-      unsigned dsm;
-      asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dsm));
-      const size_t per = tri_ws_bytes(n);          // the CTA's shared memory behind W holds S x
-      if (dsm > per) {
-        ap.ys = reinterpret_cast<float2*>(smem + per);
-        ap.ys_cap = (int)((dsm - per) / sizeof(float2));
-      }
+    unsigned dsm;
+    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dsm));
+    const size_t per = tri_ws_bytes(n);            // the CTA's shared memory behind W holds S x
+    if (dsm > per) {
+      ap.ys = reinterpret_cast<float2*>(smem + per);
+      ap.ys_cap = (int)((dsm - per) / sizeof(float2));
     }
     res = tri_smallest_team<double>(W, G, n, far, 1, gap, ap, tk, false, nullptr, a.mixed != 0);
-    if (warp != 0) return;
-  } else if constexpr (TEAM) {
-    SylvesterApply<true> ap;
-    setup(ap);
-    res = tri_smallest_team<cd>(W, G, n, far, 1, gap, ap, tk, a.mixed != 0);
-    if (warp != 0) return;
   } else {
-    SylvesterApply<false> ap;
-    setup(ap);
-    // mixed path: single-precision T and Newton steps against G first
-    res = tri_smallest<cd, false>(W, G, n, far, 1, gap, ap, tk, a.mixed != 0);
+    res = tri_smallest_team<cd>(W, G, n, far, 1, gap, ap, tk, a.mixed != 0);
   }
+  if (warp != 0) return;
 #ifdef CBP_PHASE_TIMING
   if (tk && lane == 0)
     printf("tri pass=%d s=%d real=%d near=%d | reduce %lld bisect %lld invit %lld newton %lld "
@@ -1404,11 +1368,6 @@ __global__ void __launch_bounds__(kSolveThreads) k_size_lags(SizeScanArgs a) {
   if (lane == 0) a.rho[((int64_t)f * 2 + ps) * J + j] = r;
 }
 
-// The refinement steps are off in the scan: an operator that is never applied.
-struct NoApply {
-  __device__ void operator()(const cd*, cd*) const {}
-};
-
 __global__ void __launch_bounds__(kSolveThreads, 1) k_size_scan(SizeScanArgs a) {
   extern __shared__ __align__(16) char smem[];
   const int cand = blockIdx.x, ps = blockIdx.y, f = blockIdx.z;
@@ -1429,7 +1388,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_size_scan(SizeScanArgs a) 
   }
   __syncthreads();
   gram_from_rho(rho, t1, t2, G);
-  const TriResult res = tri_smallest<double, true>(W, G, n, 0, 0, 1e300, NoApply{});
+  const TriResult res = tri_smallest<double>(W, G, n);
   // the Rayleigh quotient of the converged vector (the multisection bracket
   // is only narrowed as far as the eigenvector needs)
   if (threadIdx.x == 0) *out = res.lam_max > 0.0 ? sqrt(fmax(res.theta, 0.0) / res.lam_max) : 0.0;
@@ -1639,7 +1598,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_coprime_test(CoprimeArgs a
     correlations(P, 1, ta - 1, tb - 1, rho);
     gram_from_rho(rho, ta - 1, tb - 1, G);
     const TriWs W = carve_tri(smem + sizeof(cd) * (2 * kMaxN + kMaxN * kMaxN + 2 * kMaxN), n);
-    const TriResult res = tri_smallest<cd, true>(W, G, n, 0, 0, 1e300, NoApply{});
+    const TriResult res = tri_smallest<cd>(W, G, n);
     ratio = res.lam_max > 0.0 ? sqrt(fmax(res.theta, 0.0) / res.lam_max) : 0.0;
   }
   if (threadIdx.x == 0) a.pass[((int64_t)f * 2 + order) * a.ns + j] = (degree && ratio > a.tol) ? 1 : 0;
@@ -1713,25 +1672,16 @@ void launch_sample_solve(const Plan& p, char* ws, cudaStream_t st) {
   const int nreal = p.n * 2 * nrs, ncomplex = p.n * 2 * ncs;
   const size_t per = tri_ws_bytes(p.nn);
   a.nfr = p.n;
-  a.wpc = 1;
-  if (nreal + ncomplex <= (p.mixed ? CBP_TEAM_CTAS : CBP_TEAM_CTAS_F64)) {
-    // a CTA per sample; behind its work area the real samples' float-float
-    // refinement keeps a channel's S x and both polynomials where they fit
-    size_t sm = per;
-    if (p.mixed) {
-      const int lz2 = p.H1 + p.H2 + p.H1 + p.t2 - 1, lz1 = p.W1 + p.W2 + p.W1 + p.t2 - 1;
-      const size_t need = per + sizeof(float2) * (size_t)std::max(lz1, lz2);
-      if (need <= (110u << 10)) sm = need;
-    }
-    cudaFuncSetAttribute(k_sample_solve<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_sample_solve<true><<<nreal + ncomplex, kTeamThreads, sm, st>>>(a, nreal);
-    return;
+  // behind the work area the real samples' float-float refinement keeps a
+  // channel's S x and both polynomials where they fit
+  size_t sm = per;
+  if (p.mixed) {
+    const int lz2 = p.H1 + p.H2 + p.H1 + p.t2 - 1, lz1 = p.W1 + p.W2 + p.W1 + p.t2 - 1;
+    const size_t need = per + sizeof(float2) * (size_t)std::max(lz1, lz2);
+    if (need <= (110u << 10)) sm = need;
   }
-  // warps (samples) per CTA: up to CBP_SOLVE_WPC within ~110 KB of shared memory
-  a.wpc = (int)std::max<size_t>(1, std::min<size_t>(CBP_SOLVE_WPC, (110u << 10) / per));
-  const size_t sm = per * a.wpc;
-  cudaFuncSetAttribute(k_sample_solve<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_sample_solve<false><<<nreal + (ncomplex + a.wpc - 1) / a.wpc, kTeamThreads, sm, st>>>(a, nreal);
+  cudaFuncSetAttribute(k_sample_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_sample_solve<<<nreal + ncomplex, kTeamThreads, sm, st>>>(a, nreal);
 }
 
 void launch_scale_solve(const Plan& p, char* ws, void* k1_out, void* k2_out, int out_f64,

@@ -1,6 +1,7 @@
-// Smallest eigenpair of a Hermitian (or real symmetric) n x n matrix by one
-// warp, n <= 64: the null vector of the per-sample normal matrix G = S^H S
-// (Eq. 4; Section 5 takes it from an SVD of the Bezout/Sylvester matrix).
+// Smallest eigenpair of a Hermitian (or real symmetric) n x n matrix, n <= 64,
+// by one CTA: the reduction on all of it, the rest on its first warp (the size
+// scan and the coprimality test; the deblurring's solves spread every step over
+// four warps, cbp_tri_team.cuh, with the helpers of this file).
 //
 //   1. Householder reduction to a real symmetric tridiagonal T = Q^H G Q
 //      (reflectors H_k = I - tau_k v_k v_k^H chosen so that beta_k is real);
@@ -10,17 +11,12 @@
 //      rounds inside the widened brackets;
 //   3. inverse iteration on T - sigma I (tridiagonal LU with row interchanges)
 //      with sigma inside the bracket of the smallest eigenvalue;
-//   4. x = Q y;
-//   5. optional Newton steps against an exact operator (S^H S applied through
-//      S): the correction equation (G - theta) d = -r, d orthogonal to x, is
-//      solved through T in Olsen's form d = -(G - theta)^{-1} r +
-//      eps (G - theta)^{-1} x.
+//   4. x = Q y.
 //
-// Every step is O(n^2) per lane-column except the reduction (O(n^3) in all),
-// and all but the first bisection rounds run in double precision: a GPU whose
-// double pipe is narrow spends its time on the reduction's rank-2 updates,
-// n^3 / 3 complex multiply-adds in all.  Sign and exponent tests use the
-// integer pipe; reciprocals start from a single-precision seed.
+// All but the first bisection rounds run in double precision: a GPU whose double
+// pipe is narrow spends its time on the reduction's rank-2 updates, n^3 / 3
+// complex multiply-adds in all.  Sign and exponent tests use the integer pipe;
+// reciprocals start from a single-precision seed.
 //
 // Lane l owns the columns l and l + 32.  The matrix is stored in full with row
 // stride n; lane i touches element (j, i) of row j, so every access of a row
@@ -124,94 +120,6 @@ template <class F> __device__ __forceinline__ void cols(int n, const F& f) {
 }
 #define CBP_COLS(n, ...) \
   cols((n), [&](auto col_, const int i) { constexpr int c = decltype(col_)::c; (void)c; __VA_ARGS__ })
-
-// 1. Householder reduction.  On return T = (d, e), tau and the reflectors
-// (row k of A from column k + 1 on, v_k[k + 1] = 1) describe
-// Q = H_0 H_1 ... H_{n-2} with A_in = Q T Q^H.
-template <typename E>
-__device__ void tri_reduce(E* A, E* tau, E* w, typename RealOf<E>::type* d,
-                           typename RealOf<E>::type* e, int n) {
-  using R = typename RealOf<E>::type;
-  const int lane = threadIdx.x & 31;
-  for (int k = 0; k + 1 < n; ++k) {
-    const int k1 = k + 1;
-    E* vk = A + (size_t)k * n;             // row k = conj(column k)
-    const E alpha = cj_(vk[k1]);
-    R xn2 = R(0);
-    for (int i = lane; i < n; i += 32)
-      if (i > k1) xn2 += a2_(vk[i]);
-    xn2 = warp_sum(xn2);
-    const R ar = re_(alpha), ai = im_(alpha);
-    E tk = Ops<E>::z();
-    R beta = ar;
-    if (xn2 > R(0) || ai != R(0)) {
-      // H^H (alpha, x) = (beta, 0) with beta real, |beta| = |(alpha, x)|
-      beta = -copysign(sqrt(ar * ar + ai * ai + xn2), ar);
-      const R ib = R(1) / beta;
-      tk = mk_e<E, R>((beta - ar) * ib, -ai * ib);
-      // v = x / (alpha - beta)
-      const R dr = ar - beta, dn = R(1) / (dr * dr + ai * ai);
-      const E scl = mk_e<E, R>(dr * dn, -ai * dn);
-      __syncwarp();
-      for (int i = lane; i < n; i += 32) {
-        if (i > k1) vk[i] = mul_(cj_(vk[i]), scl);
-        else if (i == k1) vk[i] = Ops<E>::o();
-      }
-    } else {
-      __syncwarp();
-      for (int i = lane; i < n; i += 32)
-        if (i == k1) vk[i] = Ops<E>::o();
-    }
-    if (lane == 0) {
-      d[k] = re_(A[(size_t)k * n + k]);
-      e[k] = beta;
-      tau[k] = tk;
-    }
-    __syncwarp();
-    if (!Ops<E>::nz(tk)) continue;
-    // y = tau A v over the trailing block; w = y - (1/2) conj(tau) (v^H y) v
-    E y[2];
-    E dotl = Ops<E>::z();
-    CBP_COLS(n, {
-      y[c] = Ops<E>::z();
-      if (i > k && i < n) {
-        E acc = Ops<E>::z(), acc1 = Ops<E>::z();   // two chains for latency
-        int j = k1;
-        for (; j + 1 < n; j += 2) {
-          fma_(acc, cj_(A[(size_t)j * n + i]), vk[j]);
-          fma_(acc1, cj_(A[(size_t)(j + 1) * n + i]), vk[j + 1]);
-        }
-        if (j < n) fma_(acc, cj_(A[(size_t)j * n + i]), vk[j]);
-        acc = acc + acc1;
-        y[c] = mul_(tk, acc);
-        fma_(dotl, cj_(vk[i]), y[c]);
-      }
-    });
-    const E dot = warp_sum_e(dotl);
-    const R hc = R(0.5) * re_(mul_(cj_(tk), dot));
-    CBP_COLS(n, {
-      if (i > k && i < n) {
-        y[c] = y[c] - sc_(hc, vk[i]);
-        w[i] = y[c];
-      }
-    });
-    __syncwarp();
-    // A <- A - v w^H - w v^H on the trailing block
-    CBP_COLS(n, {
-      if (i > k && i < n) {
-        const E cw = cj_(y[c]), cv = cj_(vk[i]);
-        for (int j = k1; j < n; ++j) {
-          E t = mul_(vk[j], cw);
-          fma_(t, w[j], cv);
-          A[(size_t)j * n + i] = A[(size_t)j * n + i] - t;
-        }
-      }
-    });
-    __syncwarp();
-  }
-  if (lane == 0) d[n - 1] = re_(A[(size_t)(n - 1) * n + n - 1]);
-  __syncwarp();
-}
 
 // Sign and zero tests of a double on the integer pipe.
 __device__ __forceinline__ bool dneg(double x) { return __double_as_longlong(x) < 0; }
@@ -490,12 +398,11 @@ __device__ __forceinline__ void tri_solve(const TriWs& W, int n, cd* b) {
 
 // Apply Q (back = true: b <- Q b) or Q^H (b <- Q^H b) to b (n, complex V).
 template <typename E, typename V>
-__device__ void tri_apply_q(const E* A, const E* tau, int n, V* b, bool back) {
+__device__ void tri_apply_q(const E* A, const E* tau, int n, V* b) {
   using R = typename RealOf<V>::type;
   const int lane = threadIdx.x & 31;
   __syncwarp();
-  for (int s = 0; s + 1 < n; ++s) {
-    const int k = back ? n - 2 - s : s;
+  for (int k = n - 2; k >= 0; --k) {
     const V tk = to_v(tau[k], V());
     if (tk.re == R(0) && tk.im == R(0)) continue;
     const E* vk = A + (size_t)k * n;
@@ -503,7 +410,7 @@ __device__ void tri_apply_q(const E* A, const E* tau, int n, V* b, bool back) {
     for (int i = lane; i < n; i += 32)
       if (i > k) cfmac(acc, to_v(vk[i], V()), b[i]);   // v^H b
     acc = mk(warp_sum(acc.re), warp_sum(acc.im));
-    const V f = (back ? tk : conj(tk)) * acc;
+    const V f = tk * acc;
     __syncwarp();
     for (int i = lane; i < n; i += 32)
       if (i > k) b[i] = b[i] - f * to_v(vk[i], V());
@@ -513,11 +420,10 @@ __device__ void tri_apply_q(const E* A, const E* tau, int n, V* b, bool back) {
 
 // Real reflectors on a real vector (real samples): half the work of the
 // complex form.
-__device__ void tri_apply_q_r(const double* A, const double* tau, int n, double* b, bool back) {
+__device__ void tri_apply_q_r(const double* A, const double* tau, int n, double* b) {
   const int lane = threadIdx.x & 31;
   __syncwarp();
-  for (int s = 0; s + 1 < n; ++s) {
-    const int k = back ? n - 2 - s : s;
+  for (int k = n - 2; k >= 0; --k) {
     const double tk = tau[k];
     if (tk == 0.0) continue;
     const double* vk = A + (size_t)k * n;
@@ -551,49 +457,21 @@ struct TriResult {
   int near_degenerate;              // lam_2 - lam_min <= 1e-4 lam_max
 };
 
-// CTA- or warp-wide barrier.
-template <bool BLOCK> __device__ __forceinline__ void team_sync() {
-  if (BLOCK) __syncthreads();
-  else __syncwarp();
-}
-
-// Steps 1-4 by one warp: T, the eigenvalue brackets, x.  Returns the number
-// of refinement steps to take; fills res (eigenvalues), gs (the power-of-two
-// scale of G) and tnorm.
+// Steps 2-4 by one warp, after the CTA's reduction of G 2^-ex (zero: G is the
+// zero matrix): the eigenvalue brackets, x; fills res (eigenvalues).
 template <typename E>
-__device__ int tri_solve_lead(const TriWs& W, const cd* G, int n, int steps_far, int steps_near,
-                              double refine_gap, TriResult& res, double& gs, double& tnorm,
-                              long long* tk, bool prereduced = false) {
+__device__ void tri_solve_lead(const TriWs& W, int n, bool zero, int ex, TriResult& res) {
   const int lane = threadIdx.x & 31;
   E* A = (E*)W.A;
   E* tau = (E*)W.tau;
-  // scale by a power of two so that the largest diagonal entry is in [1/2, 1)
-  double gmax = 0.0;
-  for (int i = lane; i < n; i += 32) gmax = fmax(gmax, G[(size_t)i * n + i].re);
-  gmax = warp_max(gmax);
-  if (!(gmax > 0.0)) {   // zero matrix: every vector is a null vector
+  if (zero) {   // every vector is a null vector
     for (int i = lane; i < n; i += 32) W.x[i] = mk(i == 0 ? 1.0 : 0.0, 0.0);
     __syncwarp();
     res.lam_min = res.lam_2 = res.lam_max = 0.0;
     res.near_degenerate = 1;
-    gs = 1.0;
-    tnorm = 0.0;
-    return 0;
+    return;
   }
-  int ex;
-  frexp(gmax, &ex);
-  gs = ldexp(1.0, ex);
-  const double igs = ldexp(1.0, -ex);
-  if (!prereduced) {   // else the caller's CTA has reduced G * igs already
-    for (int idx = lane; idx < n * n; idx += 32) {
-      if constexpr (sizeof(E) == sizeof(double)) A[idx] = mk_e<E, double>(G[idx].re * igs, 0.0);
-      else A[idx] = mk_e<E, double>(G[idx].re * igs, G[idx].im * igs);
-    }
-    __syncwarp();
-    if (tk && lane == 0) tk[0] = clock64();
-    tri_reduce<E>(A, tau, (E*)W.w, W.d, W.e, n);
-    if (tk && lane == 0) tk[1] = clock64();
-  }
+  const double gs = ldexp(1.0, ex);
   // Gershgorin interval of T; single-precision copies
   double glo = 1e300, ghi = -1e300;
   for (int i = lane; i < n; i += 32) {
@@ -607,7 +485,7 @@ __device__ int tri_solve_lead(const TriWs& W, const cd* G, int n, int steps_far,
   }
   glo = -warp_max(-glo);
   ghi = warp_max(ghi);
-  tnorm = fmax(fabs(glo), fabs(ghi));
+  const double tnorm = fmax(fabs(glo), fabs(ghi));
   const double eps = 2.220446049250313e-16;
   glo -= 4.0 * eps * tnorm + 1e-300;
   ghi += 4.0 * eps * tnorm + 1e-300;
@@ -660,7 +538,6 @@ __device__ int tri_solve_lead(const TriWs& W, const cd* G, int n, int steps_far,
     if (w2 <= fmax(tol_abs, 1e-7 * fabs(br[2].hi))) break;
     multisect<false>(W, n, 2, br, 3, which, tiny_f);
   }
-  if (tk && lane == 0) tk[2] = clock64();
   const double lam0 = 0.5 * (br[0].lo + br[0].hi);
   const double lam1 = n > 1 ? 0.5 * (br[1].lo + br[1].hi) : lam0;
   const double lamn = 0.5 * (br[2].lo + br[2].hi);
@@ -678,7 +555,7 @@ __device__ int tri_solve_lead(const TriWs& W, const cd* G, int n, int steps_far,
       for (int i = lane; i < n; i += 32) y[i] = sc * y[i];
       __syncwarp();
     }
-    tri_apply_q_r((const double*)A, (const double*)tau, n, y, true);
+    tri_apply_q_r((const double*)A, (const double*)tau, n, y);
     const double sc = rsqrt_safe(tri_norm2_r(y, n));
     for (int i = lane; i < n; i += 32) W.x[i] = mk(sc * y[i], 0.0);
     __syncwarp();
@@ -694,272 +571,15 @@ __device__ int tri_solve_lead(const TriWs& W, const cd* G, int n, int steps_far,
       __syncwarp();
     }
     for (int i = lane; i < n; i += 32) W.x[i] = W.z[i];
-    tri_apply_q<E, cd>(A, tau, n, W.x, true);
+    tri_apply_q<E, cd>(A, tau, n, W.x);
     const double sc = rsqrt_safe(tri_norm2(W.x, n));
     for (int i = lane; i < n; i += 32) W.x[i] = sc * W.x[i];
     __syncwarp();
   }
-  if (tk && lane == 0) tk[3] = clock64();
   res.lam_min = gs * lam0;
   res.lam_2 = gs * lam1;
   res.lam_max = gs * lamn;
   res.near_degenerate = n > 1 && (lam1 - lam0) <= 1e-4 * lamn ? 1 : 0;
-  const bool near = n > 1 && (lam1 - lam0) <= refine_gap * lamn;
-  return near ? steps_near : steps_far;
-}
-
-// Steps 1-4 in single precision, then Newton steps in Olsen's form against
-// G itself: the residual G x - theta x in double precision, the correction
-// equation solved through the single-precision T (contraction ~n u ||T|| /
-// gap per step), until the correction stops shrinking or falls below 1e-10.
-// For complex matrices whose two smallest eigenvalues single precision
-// separates by more than 3e-5 lambda_max (contraction <~ 0.1 per step, at
-// most 12 steps), or separates at all with a gap above 1e-5 lambda_max (at
-// most 24 steps, which must bring the correction below 1e-9); returns false,
-// having changed nothing but the work area, for the others (they take
-// tri_solve_lead).
-__device__ bool tri_solve_lead_sp(const TriWs& W, const cd* G, int n, TriResult& res, double& gs,
-                                  double& tnorm, long long* tk) {
-  const int lane = threadIdx.x & 31;
-  cf* A = (cf*)W.A;
-  cf* tau = (cf*)W.tau;
-  float* d = W.df;
-  float* e = (float*)W.e;
-  float* u0 = (float*)W.u0;
-  float* u1 = (float*)W.u1;
-  float* u2 = (float*)W.u2;
-  float* lm = (float*)W.lm;
-  double gmax = 0.0;
-  for (int i = lane; i < n; i += 32) gmax = fmax(gmax, G[(size_t)i * n + i].re);
-  gmax = warp_max(gmax);
-  if (!(gmax > 0.0)) return false;
-  int ex;
-  frexp(gmax, &ex);
-  gs = ldexp(1.0, ex);
-  const double igs = ldexp(1.0, -ex);
-  const float igsf = (float)igs;
-  for (int idx = lane; idx < n * n; idx += 32)
-    A[idx] = mk((float)G[idx].re * igsf, (float)G[idx].im * igsf);
-  __syncwarp();
-  if (tk && lane == 0) tk[0] = clock64();
-  tri_reduce<cf>(A, tau, (cf*)W.w, d, e, n);
-  if (tk && lane == 0) tk[1] = clock64();
-  float glo = 1e30f, ghi = -1e30f;
-  for (int i = lane; i < n; i += 32) {
-    const float rad = (i > 0 ? fabsf(e[i - 1]) : 0.f) + (i + 1 < n ? fabsf(e[i]) : 0.f);
-    glo = fminf(glo, d[i] - rad);
-    ghi = fmaxf(ghi, d[i] + rad);
-    W.e2f[i] = i + 1 < n ? e[i] * e[i] : 0.f;
-  }
-  glo = -warp_max(-glo);
-  ghi = warp_max(ghi);
-  tnorm = fmax(fabs((double)glo), fabs((double)ghi));
-  __syncwarp();
-  const int which[3] = {0, 1, n - 1};
-  const double eb = 4e-6 * tnorm;     // single-precision error bound of the counts
-  Bracket br[3];
-  for (int m = 0; m < 3; ++m) br[m] = Bracket{(double)glo - eb, (double)ghi + eb};
-  const float tiny_f = (float)(1e-30 * fmax(tnorm, 1e-8));
-  for (int round = 0; round < 14; ++round) {
-    int t = -1;
-    for (int m = 2; m >= 0; --m)
-      if (br[m].hi - br[m].lo > 0.25 * eb) t = m;
-    if (t < 0) break;
-    multisect<true>(W, n, t, br, 3, which, tiny_f);
-  }
-  const double lam0 = 0.5 * (br[0].lo + br[0].hi), lam1 = 0.5 * (br[1].lo + br[1].hi);
-  const double lamn = 0.5 * (br[2].lo + br[2].hi);
-  // separated beyond the error bounds?  Well beyond (3e-5 lambda_max): at
-  // most 12 Newton steps, contraction <~ 0.1.  Narrowly (apart within the
-  // bounds, gap above 1e-5 lambda_max, contraction <~ 0.3): up to 24 steps,
-  // and the double-precision solve after all unless they converge.
-  const double sep = (br[1].lo - eb) - (br[0].hi + eb);
-  const bool wide = sep > 3e-5 * lamn;
-  if (!wide && !(sep > 0.0 && lam1 - lam0 > 1e-5 * lamn)) {
-#ifdef CBP_PHASE_TIMING
-    if (lane == 0)
-      printf("sp-reject n=%d lam0/lamn %.3e lam1/lamn %.3e eb/lamn %.3e\n", n, lam0 / lamn, lam1 / lamn,
-             eb / lamn);
-#endif
-    return false;
-  }
-  if (tk && lane == 0) tk[2] = clock64();
-  // inverse iteration in single precision (three steps)
-  tri_lu<float>(d, e, u0, u1, u2, lm, W.piv, n, (float)lam0, (float)(1.2e-7 * tnorm));
-  cf* y = (cf*)W.z;
-  for (int i = lane; i < n; i += 32) y[i] = mk(1.0f + 0.25f * (float)((i * 7) % 5), 0.f);
-  __syncwarp();
-  for (int it = 0; it < 3; ++it) {
-    tri_solve<float, cf>(u0, u1, u2, lm, W.piv, n, y);
-    __syncwarp();
-    float s2 = 0.f;
-    for (int i = lane; i < n; i += 32) s2 += abs2(y[i]);
-    s2 = warp_sum(s2);
-    const float sc = s2 > 0.f ? rsqrtf(s2) : 1.f;
-    for (int i = lane; i < n; i += 32) y[i] = sc * y[i];
-    __syncwarp();
-  }
-  // Q explicitly (lane i builds column i: H_0 ... H_{n-2} e_i), row stride n + 1
-  cf* Q = A + (size_t)n * n;
-  const int lq = n + 1;
-  for (int i = lane; i < n; i += 32) {
-    for (int j = 0; j < n; ++j) Q[(size_t)j * lq + i] = mk(j == i ? 1.f : 0.f, 0.f);
-    for (int k = n - 2; k >= 0; --k) {
-      const cf tk = tau[k];
-      if (tk.re == 0.f && tk.im == 0.f) continue;
-      const cf* vk = A + (size_t)k * n;
-      cf s0 = mk(0.f, 0.f), s1 = mk(0.f, 0.f);
-      int j = k + 1;
-      for (; j + 1 < n; j += 2) {
-        cfmac(s0, vk[j], Q[(size_t)j * lq + i]);
-        cfmac(s1, vk[j + 1], Q[(size_t)(j + 1) * lq + i]);
-      }
-      if (j < n) cfmac(s0, vk[j], Q[(size_t)j * lq + i]);
-      const cf f = tk * (s0 + s1);
-      for (int jj = k + 1; jj < n; ++jj) Q[(size_t)jj * lq + i] = Q[(size_t)jj * lq + i] - f * vk[jj];
-    }
-  }
-  __syncwarp();
-  // x = Q y
-  for (int i = lane; i < n; i += 32) {
-    cf acc = mk(0.f, 0.f);
-    for (int j = 0; j < n; ++j) cfma(acc, Q[(size_t)i * lq + j], y[j]);
-    W.x[i] = mk((double)acc.re, (double)acc.im);
-  }
-  __syncwarp();
-  {
-    const double sc = rsqrt_safe(tri_norm2(W.x, n));
-    for (int i = lane; i < n; i += 32) W.x[i] = sc * W.x[i];
-    __syncwarp();
-  }
-  if (tk && lane == 0) tk[3] = clock64();
-  // Newton steps against G
-  cf* rt = (cf*)W.q;          // Q^H r, then u
-  cf* zt = rt + n;            // Q^H x, then z
-  cf* yt = (cf*)W.z;          // Q^H x
-  cf* yq = yt + n;            // x in single precision
-  cf* rq = (cf*)W.r;          // r in single precision, then d~
-  double dprev = 1e300, dn = 1e300;
-  const int max_it = wide ? 12 : 24;
-  const double stall = wide ? 0.25 : 0.5;
-  for (int it = 0; it < max_it; ++it) {
-    cd gx[2];
-    cd th = mk(0.0, 0.0);
-    CBP_COLS(n, {
-      gx[c] = mk(0.0, 0.0);
-      if (i < n) {
-        for (int j = 0; j < n; ++j) cfmac(gx[c], G[(size_t)j * n + i], W.x[j]);   // (G x)_i
-        cfmac(th, W.x[i], gx[c]);
-      }
-    });
-    const double theta = warp_sum(th.re);
-    CBP_COLS(n, {
-      if (i < n) {
-        const cd r = gx[c] - theta * W.x[i];
-        rq[i] = mk((float)r.re, (float)r.im);
-        yq[i] = mk((float)W.x[i].re, (float)W.x[i].im);
-      }
-    });
-    __syncwarp();
-    // r~ = Q^H r, y~ = Q^H x (lane i: column i of Q)
-    for (int i = lane; i < n; i += 32) {
-      cf a0 = mk(0.f, 0.f), a1 = mk(0.f, 0.f);
-      for (int j = 0; j < n; ++j) {
-        const cf q = Q[(size_t)j * lq + i];
-        cfmac(a0, q, yq[j]);
-        cfmac(a1, q, rq[j]);
-      }
-      yt[i] = a0;
-      zt[i] = a0;
-      rt[i] = a1;
-    }
-    tri_lu<float>(d, e, u0, u1, u2, lm, W.piv, n, (float)(theta * igs), (float)(1.2e-7 * tnorm));
-    __syncwarp();
-    tri_solve<float, cf>(u0, u1, u2, lm, W.piv, n, rt);   // u
-    tri_solve<float, cf>(u0, u1, u2, lm, W.piv, n, zt);   // z
-    __syncwarp();
-    cf nu = mk(0.f, 0.f), de = mk(0.f, 0.f);
-    for (int i = lane; i < n; i += 32) {
-      cfmac(nu, yt[i], rt[i]);
-      cfmac(de, yt[i], zt[i]);
-    }
-    nu = mk(warp_sum(nu.re), warp_sum(nu.im));
-    de = mk(warp_sum(de.re), warp_sum(de.im));
-    const float dd = abs2(de);
-    const cf epsn = dd > 0.f ? (1.0f / dd) * (nu * conj(de)) : mk(0.f, 0.f);
-    const float ig = (float)igs;
-    for (int i = lane; i < n; i += 32) rq[i] = ig * (epsn * zt[i] - rt[i]);
-    __syncwarp();
-    float d2 = 0.f;
-    for (int i = lane; i < n; i += 32) {   // d = Q d~ (lane i: row i of Q)
-      cf acc = mk(0.f, 0.f);
-      for (int j = 0; j < n; ++j) cfma(acc, Q[(size_t)i * lq + j], rq[j]);
-      W.x[i] = W.x[i] + mk((double)acc.re, (double)acc.im);
-      d2 += abs2(acc);
-    }
-    d2 = warp_sum(d2);
-    __syncwarp();
-    const double sc = rsqrt_safe(tri_norm2(W.x, n));
-    for (int i = lane; i < n; i += 32) W.x[i] = sc * W.x[i];
-    __syncwarp();
-    dn = sqrt((double)d2);
-    if (dn < 1e-10 || dn > stall * dprev) break;
-    dprev = dn;
-  }
-  if (!wide && !(dn < 1e-9)) {
-#ifdef CBP_PHASE_TIMING
-    if (lane == 0) printf("sp-narrow-fail n=%d last correction %.3e\n", n, dn);
-#endif
-    return false;
-  }
-  res.lam_min = gs * lam0;
-  res.lam_2 = gs * lam1;
-  res.lam_max = gs * lamn;
-  res.near_degenerate = (lam1 - lam0) <= 1e-4 * lamn ? 1 : 0;
-  return true;
-}
-
-// One refinement step by the lead warp after r = (exact operator) x: Olsen's
-// correction through T (step 5).
-template <typename E>
-__device__ void tri_olsen(const TriWs& W, int n, double gs, double tnorm) {
-  const int lane = threadIdx.x & 31;
-  const E* A = (const E*)W.A;
-  const E* tau = (const E*)W.tau;
-  const double eps = 2.220446049250313e-16, igs = 1.0 / gs;
-  cd th = mk(0.0, 0.0);
-  for (int i = lane; i < n; i += 32) cfmac(th, W.x[i], W.r[i]);
-  const double theta = warp_sum(th.re);
-  for (int i = lane; i < n; i += 32) {
-    W.r[i] = W.r[i] - theta * W.x[i];
-    W.q[i] = W.x[i];
-  }
-  // to T coordinates: r~ = Q^H r, y~ = Q^H x
-  tri_apply_q<E, cd>(A, tau, n, W.r, false);
-  tri_apply_q<E, cd>(A, tau, n, W.q, false);
-  tri_lu(W, n, theta * igs, eps * tnorm);
-  for (int i = lane; i < n; i += 32) W.z[i] = W.q[i];
-  __syncwarp();
-  tri_solve(W, n, W.r);    // u = (T - theta)^{-1} r~
-  tri_solve(W, n, W.z);    // z = (T - theta)^{-1} y~
-  __syncwarp();
-  cd nu = mk(0.0, 0.0), de = mk(0.0, 0.0);
-  for (int i = lane; i < n; i += 32) {
-    cfmac(nu, W.q[i], W.r[i]);
-    cfmac(de, W.q[i], W.z[i]);
-  }
-  nu = mk(warp_sum(nu.re), warp_sum(nu.im));
-  de = mk(warp_sum(de.re), warp_sum(de.im));
-  const double dd = abs2(de);
-  const cd epsn = dd > 0.0 ? (1.0 / dd) * (nu * conj(de)) : mk(0.0, 0.0);
-  // d = (-u + eps z) / gs in T coordinates, then back
-  for (int i = lane; i < n; i += 32) W.z[i] = igs * (epsn * W.z[i] - W.r[i]);
-  tri_apply_q<E, cd>(A, tau, n, W.z, true);
-  for (int i = lane; i < n; i += 32) W.x[i] = W.x[i] + W.z[i];
-  __syncwarp();
-  const double sc = rsqrt_safe(tri_norm2(W.x, n));
-  for (int i = lane; i < n; i += 32) W.x[i] = sc * W.x[i];
-  __syncwarp();
 }
 
 // ------------------------------------------------------------------------
@@ -1021,73 +641,42 @@ __device__ __forceinline__ float inv_norm_x(const fx* b, int n) {
 }
 
 // G: the n x n matrix (row-major, global or shared memory).  Result in W.x
-// (unit norm).  Steps of the exact-operator refinement: `steps_far` when the
-// two smallest eigenvalues are more than refine_gap * lam_max apart,
-// `steps_near` otherwise.  apply(x, out): out = (exact operator) x, by the
-// calling warp.  BLOCK (no refinement steps): every thread of the CTA calls and
-// the CTA reduces G together; warp 0 does the rest and holds the result.
-// single: complex matrices try the single-precision solve first.
-template <typename E, bool BLOCK, class Apply>
-__device__ TriResult tri_smallest(const TriWs& W, const cd* G, int n, int steps_far,
-                                  int steps_near, double refine_gap, const Apply& apply,
-                                  long long* tk = nullptr, bool single = false) {
+// (unit norm).  Every thread of the CTA calls; the CTA reduces G together, warp
+// 0 does the rest and holds the result.
+template <typename E>
+__device__ TriResult tri_smallest(const TriWs& W, const cd* G, int n) {
   const int lane = threadIdx.x & 31;
-  const bool lead = !BLOCK || threadIdx.x < 32;
   TriResult res = {};
-  double gs = 1.0, tnorm = 0.0;
-  int steps = 0;
-  bool pre = false;
-  if constexpr (BLOCK) {
-    // the CTA reduces G * 2^-ex together (ex from the largest diagonal entry)
-    double gmax = 0.0;
-    for (int i = lane; i < n; i += 32) gmax = fmax(gmax, G[(size_t)i * n + i].re);
-    gmax = warp_max(gmax);
-    if (gmax > 0.0) {
-      int ex;
-      frexp(gmax, &ex);
-      const double igs = ldexp(1.0, -ex);
-      E* A = (E*)W.A;
-      for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-        if constexpr (sizeof(E) == sizeof(double)) A[idx] = mk_e<E, double>(G[idx].re * igs, 0.0);
-        else A[idx] = mk_e<E, double>(G[idx].re * igs, G[idx].im * igs);
-      }
-      __syncthreads();
-      if (tk && threadIdx.x == 0) tk[0] = clock64();
-      tri_reduce_block<E>(A, (E*)W.tau, (E*)W.w, W.d, W.e, n, (E*)W.part);
-      if (tk && threadIdx.x == 0) tk[1] = clock64();
-      pre = true;
+  // the CTA reduces G 2^-ex, its largest diagonal entry in [1/2, 1)
+  double gmax = 0.0;
+  for (int i = lane; i < n; i += 32) gmax = fmax(gmax, G[(size_t)i * n + i].re);
+  gmax = warp_max(gmax);
+  const bool zero = !(gmax > 0.0);
+  int ex = 0;
+  if (!zero) {
+    frexp(gmax, &ex);
+    const double igs = ldexp(1.0, -ex);
+    E* A = (E*)W.A;
+    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+      if constexpr (sizeof(E) == sizeof(double)) A[idx] = mk_e<E, double>(G[idx].re * igs, 0.0);
+      else A[idx] = mk_e<E, double>(G[idx].re * igs, G[idx].im * igs);
     }
+    __syncthreads();
+    tri_reduce_block<E>(A, (E*)W.tau, (E*)W.w, W.d, W.e, n, (E*)W.part);
   }
-  if (lead) {
-    if (!BLOCK && single && n > 2 && tri_solve_lead_sp(W, G, n, res, gs, tnorm, tk))
-      steps = 0;
-    else
-      steps = tri_solve_lead<E>(W, G, n, steps_far, steps_near, refine_gap, res, gs, tnorm, tk, pre);
-  }
-  if constexpr (!BLOCK) {
-    for (int it = 0; it < steps; ++it) {
-      apply(W.x, W.r);
-      __syncwarp();
-      if (tk && lane == 0) tk[6] = clock64();   // end of the last step's apply
-      tri_olsen<E>(W, n, gs, tnorm);
-      __syncwarp();
-    }
-  }
-  if (tk && lead && lane == 0) tk[4] = clock64();
-  if (lead) {
-    // theta = x^H G x
-    cd th = mk(0.0, 0.0);
+  if (threadIdx.x >= 32) return res;
+  tri_solve_lead<E>(W, n, zero, ex, res);
+  // theta = x^H G x
+  cd th = mk(0.0, 0.0);
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const int i = lane + 32 * c;
-      if (i < n) {
-        cd gx = mk(0.0, 0.0);
-        for (int j = 0; j < n; ++j) cfmac(gx, G[(size_t)j * n + i], W.x[j]);   // (G x)_i
-        cfmac(th, W.x[i], gx);
-      }
+  for (int c = 0; c < 2; ++c) {
+    const int i = lane + 32 * c;
+    if (i < n) {
+      cd gx = mk(0.0, 0.0);
+      for (int j = 0; j < n; ++j) cfmac(gx, G[(size_t)j * n + i], W.x[j]);   // (G x)_i
+      cfmac(th, W.x[i], gx);
     }
-    res.theta = warp_sum(th.re);
   }
-  if (tk && lead && lane == 0) tk[5] = clock64();
+  res.theta = warp_sum(th.re);
   return res;
 }

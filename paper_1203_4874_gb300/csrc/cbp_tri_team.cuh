@@ -176,7 +176,7 @@ template <typename T> __device__ __forceinline__ T redot_(cpx<T> a, cpx<T> b) {
   return fma(a.re, b.re, a.im * b.im);
 }
 
-// Householder reduction by the team, results as tri_reduce's.  The lead warp
+// Householder reduction by the team, results as tri_reduce_block's.  The lead warp
 // carries the chain: a column's norm, its reflector, then -- from the others'
 // partial products -- w, and at once the next column, whose norm it starts
 // while the others (each on its own rows j, owner 1 + j mod 3) update the rest
@@ -575,7 +575,7 @@ __device__ void tri_solve_r(const R* u0, const R* u1, const R* u2, const R* lm, 
   __syncwarp();
 }
 
-// b <- Q b (back) or Q^H b by one warp, as tri_apply_q, b in registers and the
+// b <- Q b (back) or Q^H b by one warp, b in registers and the
 // reflector's product summed by one chain.
 __device__ __forceinline__ void mac_conj(cd& acc, cd v, cd b) { cfmac(acc, v, b); }
 __device__ __forceinline__ void mac_conj(double& acc, double v, double b) { acc = fma(v, b, acc); }
@@ -707,9 +707,16 @@ __device__ __forceinline__ void form_q(const cf* A, const cf* tau, int n, int i,
   }
 }
 
-// Single-precision solve and Newton steps against G by the team, as
-// tri_solve_lead_sp (same acceptance rules, same stopping rules); the result in
-// W.x; returns (uniformly) whether it was accepted.
+// The solve in single precision, then Newton steps in Olsen's form against G
+// itself, by the team: the residual G x - theta x in double precision, the
+// correction equation solved through the single-precision T (contraction
+// ~n u ||T|| / gap per step), until the correction stops shrinking or falls
+// below 1e-10.  For complex matrices whose two smallest eigenvalues single
+// precision separates by more than 3e-5 lambda_max (contraction <~ 0.1 per step,
+// at most 12 steps), or separates at all with a gap above 1e-5 lambda_max (at
+// most 24 steps, which must bring the correction below 1e-9); returns
+// (uniformly) false, having changed nothing but the work area, for the others
+// (they take tri_solve_team).  The result is in W.x.
 __device__ bool tri_solve_team_sp(const TriWs& W, TeamWs& S, const cd* G, int n, TriResult& res,
                                   long long* tk, const cfx* Gx) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
@@ -978,8 +985,7 @@ __device__ __forceinline__ void tri_bounds(const TriWs& W, int n, double eps, do
   team_bar();
 }
 
-// Steps 1-4 in double precision (E = cd or double) by the team, as
-// tri_solve_lead; FFR (real samples of the mixed path): from T on in float-float,
+// Steps 1-4 in double precision (E = cd or double) by the team; FFR (real samples of the mixed path): from T on in float-float,
 // the reflectors' copies overwriting the double ones in place.  Fills res, S.gs,
 // S.tnorm; returns the number of refinement steps to take.
 template <typename E, bool FFR>
@@ -1197,8 +1203,11 @@ __device__ void tri_olsen_team(const TriWs& W, TeamWs& S, int n) {
   team_bar();
 }
 
-// As tri_smallest<E, true>, by a CTA of at least four warps: warps 0..3 are the
+// The smallest eigenpair by a CTA of at least four warps: warps 0..3 are the
 // team, the others take part in apply() only.  The result is valid in warp 0.
+// apply(x, out): out = (exact operator) x; its Newton steps: `steps_far` when the
+// two smallest eigenvalues are more than refine_gap * lam_max apart, `steps_near`
+// otherwise.
 // single: complex matrices try the single-precision solve first; ffr: real
 // matrices go on in float-float after the double reduction (mixed path).
 template <typename E, class Apply>

@@ -1,9 +1,9 @@
 """The per-sample and scale solves where they change their arrangement: system
 widths n = t1 + t2 and 2 M on both sides of 32 (one or two matrix columns per
-lane) and at the smallest and largest supported, batches small enough for a
-CTA per sample and just too large for it.  Kernels against the oracle at the
-repository's bars: 1e-9 (FP64 path), 1e-3 (mixed path); pairs of a large batch
-against the same pairs alone within twice the FP64 bar."""
+lane) and at the smallest and largest supported, batches of few and of many
+samples to an SM.  Kernels against the oracle at the repository's bars: 1e-9
+(FP64 path), 1e-3 (mixed path); pairs of a large batch against the same pairs
+alone within twice the bar, and the same bits."""
 import numpy as np
 import pytest
 import torch
@@ -53,3 +53,19 @@ def test_batches_around_a_cta_per_sample(gpu_ctx, n, path):
         for g in range(f, n, 4):
             assert rel(stages["k1"][g].cpu().numpy(), k1[0].cpu().numpy()) <= tol
             assert rel(stages["k2"][g].cpu().numpy(), k2[0].cpu().numpy()) <= tol
+
+
+@pytest.mark.parametrize("path", ["fp64", "mixed"])
+@pytest.mark.parametrize("n", [7, 40])
+def test_a_pair_does_not_depend_on_its_batch(gpu_ctx, n, path):
+    """Bit for bit: the serving engine's batches give what each request gives alone."""
+    from paper_1203_4874_gb300 import cbp
+    pairs = [make_pair(7100 + f, 40, 45, 6, 5, c=3) for f in range(n)]
+    B1, B2 = (torch.from_numpy(np.stack([p[k] for p in pairs])).cuda() for k in (0, 1))
+    prm = cbp.params(6, 5, path=path, flags=cbp.CBP_FLAG_KERNELS_F64)
+    lat, k1, k2, _, _ = cbp.cbp_deblur_pair(gpu_ctx, B1, B2, prm)
+    torch.cuda.synchronize()
+    for f in range(0, n, 3):
+        a = cbp.cbp_deblur_pair(gpu_ctx, B1[f:f + 1], B2[f:f + 1], prm)
+        torch.cuda.synchronize()
+        assert torch.equal(a[0][0], lat[f]) and torch.equal(a[1][0], k1[f]) and torch.equal(a[2][0], k2[f])
