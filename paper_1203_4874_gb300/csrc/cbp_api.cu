@@ -208,8 +208,8 @@ cbp_status run_plan(const Plan& p, const cbp_frames* b1, const cbp_frames* b2,
       d2.tab = tabs->b2;
     }
   }
-  cudaMemsetAsync(wsp + p.off_bad, 0, (size_t)p.n * sizeof(int), st);
-  cudaMemsetAsync(wsp + p.off_err, 0, sizeof(int), st);
+  // the pairs' input flags and, next to them, the error word
+  cudaMemsetAsync(wsp + p.off_bad, 0, p.off_err + sizeof(int) - p.off_bad, st);
   if (kin) {
     if ((!k1d || !k2d) && !(tabs && tabs->k1 && tabs->k2)) return CBP_ERR_INVALID_ARG;
     begin(CBP_STAGE_SCALE_SOLVE);
@@ -230,7 +230,7 @@ cbp_status run_plan(const Plan& p, const cbp_frames* b1, const cbp_frames* b2,
     if (!tw_ready) {
       begin(CBP_STAGE_KERNEL_SPECTRA);   // FFT twiddle tables
       init_twiddles(p, wsp, st);
-      end(CBP_STAGE_KERNEL_SPECTRA, 4);
+      end(CBP_STAGE_KERNEL_SPECTRA, 1);
     }
     // one read of the frames: A1 folds and the A6 forward row FFTs together
     begin(CBP_STAGE_ROW_FFT);

@@ -155,31 +155,8 @@ __host__ __device__ inline bool plan_is(const FftPlan& pl) {
 #define CBP_ROW_PLAN 972, 9, 9, 4, 3
 
 template <typename T>
-__global__ void k_stage_twiddles(FftPlan pl, cpx<T>* out) {
-  for (int s = 0; s < pl.nst; ++s) {
-    const FftStage& st = pl.st[s];
-    const int cnt = st.Ns * (st.R - 1);
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < cnt; e += gridDim.x * blockDim.x) {
-      const int r = e / st.Ns + 1, k = e % st.Ns;
-      double sn, cs;
-      sincospi(-2.0 * (double)(k * r) / (double)(st.Ns * st.R), &sn, &cs);
-      out[st.tw + e] = mk<T>((T)cs, (T)sn);
-    }
-  }
-}
-
-template <typename T>
 __device__ __forceinline__ void load_twiddles(cpx<T>* dst, const cpx<T>* src, int n) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
-}
-
-template <typename T>
-__global__ void k_twiddles(cpx<T>* tw, int n) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    double s, c;
-    sincospi(-2.0 * (double)k / (double)n, &s, &c);
-    tw[k] = mk<T>((T)c, (T)s);
-  }
 }
 
 // Kernel spectra K^_k[u][v], u < Ph, v < Pw2, from the double kernels:
@@ -1822,34 +1799,79 @@ void run_row_ifft(const Plan& p, char* ws, void* latent, int out_f64, cudaStream
 
 }  // namespace
 
-// Transposed twiddle tables of a two-factor split N = A B:
-// out[b A + a] = w_N^(a b) and out[A B + a B + b] = w_N^(a b), a < A, b < B.
-__global__ void k_twiddles_2f(cf* out, int A, int B) {
-  const int N = A * B;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < N; e += gridDim.x * blockDim.x) {
-    const int b = e / A, a = e % A;
-    double sn, cs;
-    sincospi(-2.0 * (double)((a * b) % N) / (double)N, &sn, &cs);
-    const cf w = mk((float)cs, (float)sn);
-    out[b * A + a] = w;
-    out[N + a * B + b] = w;
+// All of a grid's twiddle tables in one launch, an entry a thread:
+//   tw_h[k] = w_Ph^k, tw_w[k] = w_Pw^k;
+//   the stage tables of the column and row plans;
+//   the transposed tables of the two-factor splits N = A B (972 = 36 x 27,
+//   1120 = 32 x 35): out[b A + a] = w_N^(a b) and out[A B + a B + b] = w_N^(a b).
+// A double sincospi is some 60 double instructions, so what counts is that the
+// few thousand entries spread over all SMs: as four to six launches, two of them
+// looping over the stages in a few blocks, they took 30-46 us before a small call's
+// first real kernel; this takes about 5.
+struct TableArgs {
+  FftPlan h, r;
+  int Ph, Pw;
+  void *tw_h, *tw_w, *stw_h, *stw_r;
+  cf *tw2r, *tw2c;      // or null
+};
+constexpr int kTableThreads = 64;
+template <typename T>
+__device__ __forceinline__ void root_to(cpx<T>* out, int k, int n) {
+  double sn, cs;
+  sincospi(-2.0 * (double)k / (double)n, &sn, &cs);
+  *out = mk<T>((T)cs, (T)sn);
+}
+template <typename T>
+__device__ __forceinline__ void stage_entry(const FftPlan& pl, cpx<T>* out, int e) {
+  for (int s = 0; s < pl.nst; ++s) {
+    const FftStage& st = pl.st[s];
+    const int i = e - st.tw;
+    if (i < 0 || i >= st.Ns * (st.R - 1)) continue;
+    const int r = i / st.Ns + 1, k = i % st.Ns;
+    root_to(out + e, k * r, st.Ns * st.R);
   }
 }
-
+__device__ __forceinline__ void split_entry(cf* out, int A, int B, int e) {
+  const int N = A * B, b = e / A, a = e % A;
+  cf w;
+  root_to(&w, (a * b) % N, N);
+  out[b * A + a] = w;
+  out[N + a * B + b] = w;
+}
 template <typename T>
-void run_twiddles(const Plan& p, char* ws, cudaStream_t st) {
-  if (p.off_tw2r) k_twiddles_2f<<<4, 256, 0, st>>>((cf*)(ws + p.off_tw2r), 36, 27);
-  if (p.off_tw2c) k_twiddles_2f<<<5, 256, 0, st>>>((cf*)(ws + p.off_tw2c), 32, 35);
-  k_twiddles<T><<<(p.Ph + 255) / 256, 256, 0, st>>>((cpx<T>*)(ws + p.off_tw_h), p.Ph);
-  k_twiddles<T><<<(p.Pw + 255) / 256, 256, 0, st>>>((cpx<T>*)(ws + p.off_tw_w), p.Pw);
-  const FftPlan& plw = p.pw_half ? p.fp_w2 : p.fp_w;
-  k_stage_twiddles<T><<<(p.Ph + 255) / 256, 256, 0, st>>>(p.fp_h, (cpx<T>*)(ws + p.off_stw_h));
-  k_stage_twiddles<T><<<(plw.n + 255) / 256, 256, 0, st>>>(plw, (cpx<T>*)(ws + p.off_stw_r));
+__global__ void __launch_bounds__(kTableThreads) k_tables(TableArgs t) {
+  int e = blockIdx.x * kTableThreads + threadIdx.x;
+  if (e < t.Ph) return root_to((cpx<T>*)t.tw_h + e, e, t.Ph);
+  e -= t.Ph;
+  if (e < t.Pw) return root_to((cpx<T>*)t.tw_w + e, e, t.Pw);
+  e -= t.Pw;
+  if (e < t.h.ntw) return stage_entry(t.h, (cpx<T>*)t.stw_h, e);
+  e -= t.h.ntw;
+  if (e < t.r.ntw) return stage_entry(t.r, (cpx<T>*)t.stw_r, e);
+  e -= t.r.ntw;
+  if (t.tw2r) {
+    if (e < 972) return split_entry(t.tw2r, 36, 27, e);
+    e -= 972;
+  }
+  if (t.tw2c && e < 1120) split_entry(t.tw2c, 32, 35, e);
 }
 
 void init_twiddles(const Plan& p, char* ws, cudaStream_t st) {
-  if (p.fft_f64) run_twiddles<double>(p, ws, st);
-  else run_twiddles<float>(p, ws, st);
+  TableArgs t;
+  t.h = p.fp_h;
+  t.r = p.pw_half ? p.fp_w2 : p.fp_w;
+  t.Ph = p.Ph;
+  t.Pw = p.Pw;
+  t.tw_h = ws + p.off_tw_h;
+  t.tw_w = ws + p.off_tw_w;
+  t.stw_h = ws + p.off_stw_h;
+  t.stw_r = ws + p.off_stw_r;
+  t.tw2r = p.off_tw2r ? (cf*)(ws + p.off_tw2r) : nullptr;
+  t.tw2c = p.off_tw2c ? (cf*)(ws + p.off_tw2c) : nullptr;
+  const int total = t.Ph + t.Pw + t.h.ntw + t.r.ntw + (t.tw2r ? 972 : 0) + (t.tw2c ? 1120 : 0);
+  const int blocks = (total + kTableThreads - 1) / kTableThreads;
+  if (p.fft_f64) k_tables<double><<<blocks, kTableThreads, 0, st>>>(t);
+  else k_tables<float><<<blocks, kTableThreads, 0, st>>>(t);
 }
 
 void launch_kernel_spectra(const Plan& p, char* ws, cudaStream_t st) {
