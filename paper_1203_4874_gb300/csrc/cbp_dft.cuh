@@ -103,7 +103,8 @@ __device__ __forceinline__ void dft_odd(cpx<T>* v, const T* C, const T* S) {
 
 template <typename T, bool Inv, int R>
 __device__ __forceinline__ void small_dft(cpx<T>* v) {
-  if constexpr (R == 2) {
+  if constexpr (R == 1) {
+  } else if constexpr (R == 2) {
     dft2<T, Inv>(v[0], v[1]);
   } else if constexpr (R == 3) {
     dft3<T, Inv>(v[0], v[1], v[2]);

@@ -440,6 +440,7 @@ __device__ __forceinline__ void first_stage_raw(const In* raw, const int* ph, in
                                                 cpx<T>* out, const FftPlan& pl, int nb) {
   const FftStage& st = pl.st[0];
   switch (st.R) {
+    case 1: stage_first_raw<T, 1, In>(raw, ph, rw, W, half, out, st, pl.n, nb); break;   // a grid of 1
     case 2: stage_first_raw<T, 2, In>(raw, ph, rw, W, half, out, st, pl.n, nb); break;
     case 3: stage_first_raw<T, 3, In>(raw, ph, rw, W, half, out, st, pl.n, nb); break;
     case 4: stage_first_raw<T, 4, In>(raw, ph, rw, W, half, out, st, pl.n, nb); break;
@@ -1360,6 +1361,7 @@ __device__ __forceinline__ void first_stage_spec(const cpx<T>* raw, int Pw2p, co
                                                  int nb) {
   const FftStage& st = pl.st[0];
   switch (st.R) {
+    case 1: stage_first_spec<T, 1>(raw, Pw2p, tw_w, half, Pw2, out, st, pl.n, nb); break;
     case 2: stage_first_spec<T, 2>(raw, Pw2p, tw_w, half, Pw2, out, st, pl.n, nb); break;
     case 3: stage_first_spec<T, 3>(raw, Pw2p, tw_w, half, Pw2, out, st, pl.n, nb); break;
     case 4: stage_first_spec<T, 4>(raw, Pw2p, tw_w, half, Pw2, out, st, pl.n, nb); break;

@@ -89,6 +89,11 @@ bool make_fft_plan(int n, FftPlan* p) {
     off += Ns * (R - 1);
     Ns *= R;
   }
+  if (n == 1) {   // no stage; the passes that fuse the first one copy by radix 1
+    p->st[0].R = p->st[0].Ns = p->st[0].Nr = 1;
+    p->st[0].mNs = p->st[0].mNr = 0;
+    p->st[0].tw = 0;
+  }
   p->ntw = off > 0 ? off : 1;
   return true;
 }
