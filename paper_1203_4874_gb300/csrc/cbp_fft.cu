@@ -39,7 +39,14 @@ static __device__ uint32_t cbp_tx_extra;
 
 namespace {
 
-constexpr int kFftThreads = 256;
+__device__ __forceinline__ cf ldg_cpx(const cf* p) {
+  const float2 v = __ldg((const float2*)p);
+  return mk(v.x, v.y);
+}
+__device__ __forceinline__ cd ldg_cpx(const cd* p) {
+  const double2 v = __ldg((const double2*)p);
+  return mk(v.x, v.y);
+}
 
 // One Stockham stage of radix R over nb transforms of length N (stride N),
 // in -> out; tw = this stage's twiddles (shared memory).
@@ -159,36 +166,45 @@ __device__ __forceinline__ void load_twiddles(cpx<T>* dst, const cpx<T>* src, in
   for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
 }
 
-// Kernel spectra K^_k[u][v], u < Ph, v < Pw2, from the double kernels:
-// Spectra of both kernels on the Ph x Pw grid (Pw/2 + 1 columns kept):
+// Spectra of both kernels on the Ph x Pw grid (Pw/2 + 1 columns kept), from the
+// double kernels:
 //   K^(u, v) = sum_p w_H^(u p) R_p(v),   R_p(v) = sum_q K[p][q] w_W^(q v).
-// A block takes 64 columns of one kernel: first the t row transforms R_p(v),
-// then every u with each lane on two columns (v, v + 32: coalesced 256-byte
-// row segments per warp store), kSpecRows rows at a time so that each R_p(v)
-// read serves kSpecRows outputs; the sum over p by Horner's rule in
-// z = w_H^u (one complex multiply-add per term, no twiddle indexing).
-constexpr int kSpecCols = 64;
-constexpr int kSpecRows = 8;
+// A block takes kSpecCols columns (a lane each) and a share of the rows of one
+// kernel: first the t row transforms R_p(v), then the rows u, u + Ph/S, ...,
+// u + (S-1) Ph/S together: with z = w_H^u the sums over p = r mod S,
+//   F_r = z^r sum_j R_{r + S j}(v) (z^S)^j    (Horner's rule in z^S),
+// serve all S of them, K^(u + m Ph/S, v) = sum_r w_S^(m r) F_r, an S-point DFT.
+// Bound by the double units on the FP64 path, by instruction issue on float
+// data: at S = 4 a 17-row kernel takes 20 multiply-adds a point (96 instructions
+// by Horner's rule row by row: S = 1).  Row shares keep every SM busy (a block's
+// own R_p are a tenth of its work at two shares).
+// Eight 480p colour pairs, 17 / 15 double kernels: 143 us (862 row by row on
+// 96 blocks); one 64 x 64 pair, 5 / 5: 6 us (43 on two).
+constexpr int kSpecCols = 32;
+constexpr int kSpecThreads = 128;
+template <typename T> constexpr int kSpecRows = sizeof(T) == 8 ? 2 : 4;   // rows u a thread and step
 
-template <typename T>
-__global__ void __launch_bounds__(kFftThreads)
-k_kernel_spectra(const double* kd, int t1, int t2, int Ph, int Pw, int Pw2, int Pw2p,
+template <typename T, int S>
+__global__ void __launch_bounds__(kSpecThreads)
+k_kernel_spectra(const double* kd, int t1, int t2, int Ph, int Pw, int Pw2, int Pw2p, int shares,
                  const cpx<T>* tw_h, const cpx<T>* tw_w, cpx<T>* khat) {
-  extern __shared__ __align__(16) char smem[];
-  cpx<T>* kv = (cpx<T>*)smem;                       // [t][kSpecCols]
-  cpx<T>* twh = kv + kMaxN * kSpecCols;             // [Ph]
-  const int k = blockIdx.y, f = blockIdx.z;
+  constexpr int R = kSpecRows<T>;
+  __shared__ cpx<T> kv[kMaxN * kSpecCols];          // [t][kSpecCols], t < kMaxN
+  const int k = blockIdx.y & 1, share = blockIdx.y >> 1, f = blockIdx.z;
   const int t = k ? t2 : t1;
   const double* K = kd + (int64_t)f * (t1 * t1 + t2 * t2) + (k ? t1 * t1 : 0);
   const int v0 = blockIdx.x * kSpecCols;
-  for (int i = threadIdx.x; i < Ph; i += blockDim.x) twh[i] = tw_h[i];
-  for (int idx = threadIdx.x; idx < t * kSpecCols; idx += blockDim.x) {
-    const int p = idx / kSpecCols, vl = idx % kSpecCols, v = v0 + vl;
+  for (int idx = threadIdx.x; idx < t * kSpecCols; idx += kSpecThreads) {
+    const int p = idx / kSpecCols, v = v0 + idx % kSpecCols;
     cpx<T> acc = mk<T>(0, 0);
     if (v < Pw2) {
       int e = 0;                              // (v q) mod Pw, incrementally
+#pragma unroll 4
       for (int q = 0; q < t; ++q) {
-        acc = acc + (T)K[p * t + q] * tw_w[e];
+        const T c = (T)K[p * t + q];
+        const cpx<T> w = ldg_cpx(tw_w + e);
+        acc.re = fma(c, w.re, acc.re);
+        acc.im = fma(c, w.im, acc.im);
         e += v;
         if (e >= Pw) e -= Pw;
       }
@@ -196,33 +212,60 @@ k_kernel_spectra(const double* kd, int t1, int t2, int Ph, int Pw, int Pw2, int 
     kv[idx] = acc;
   }
   __syncthreads();
-  cpx<T>* out = khat + ((int64_t)f * 2 + k) * Ph * Pw2p;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int va = v0 + lane, vb = v0 + 32 + lane;
-  // Horner's rule in z = w_H^u: K^(u, v) = (...(R_{t-1}(v) z + R_{t-2}(v)) z + ...) + R_0(v)
-  for (int u0 = warp * kSpecRows; u0 < Ph; u0 += nw * kSpecRows) {
-    cpx<T> acc[kSpecRows][2], z[kSpecRows];
-    const cpx<T> ra = kv[(t - 1) * kSpecCols + lane], rb = kv[(t - 1) * kSpecCols + 32 + lane];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int v = v0 + lane, Q = Ph / S;
+  const int jt = (t - 1) / S, rem = t - S * jt;      // the top row of terms holds rem of them
+  const cpx<T>* col = kv + lane;
+  cpx<T>* out = khat + ((int64_t)f * 2 + k) * Ph * Pw2p + v;
+  const int step = shares * (kSpecThreads / 32) * R;
+  for (int u0 = (share * (kSpecThreads / 32) + warp) * R; u0 < Q; u0 += step) {
+    cpx<T> acc[R][S], zs[R];
+    int u[R];
 #pragma unroll
-    for (int j = 0; j < kSpecRows; ++j) {
-      z[j] = twh[u0 + j < Ph ? u0 + j : 0];   // rows past Ph are computed as u = 0, not stored
-      acc[j][0] = ra;
-      acc[j][1] = rb;
+    for (int i = 0; i < R; ++i) {
+      u[i] = u0 + i < Q ? u0 + i : 0;         // rows past Q are computed as u = 0, not stored
+      zs[i] = ldg_cpx(tw_h + (S > 1 ? S * u[i] : u[i]));
     }
-    for (int p = t - 2; p >= 0; --p) {
-      const cpx<T> ca = kv[p * kSpecCols + lane], cb = kv[p * kSpecCols + 32 + lane];
+    if (jt == 0) {
 #pragma unroll
-      for (int j = 0; j < kSpecRows; ++j) {
-        acc[j][0] = acc[j][0] * z[j] + ca;
-        acc[j][1] = acc[j][1] * z[j] + cb;
+      for (int r = 0; r < S; ++r) {
+        const cpx<T> c = r < rem ? col[r * kSpecCols] : mk<T>(0, 0);
+#pragma unroll
+        for (int i = 0; i < R; ++i) acc[i][r] = c;
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < S; ++r) {
+        const cpx<T> c = col[((jt - 1) * S + r) * kSpecCols];
+#pragma unroll
+        for (int i = 0; i < R; ++i) acc[i][r] = c;
+        if (r < rem) {
+          const cpx<T> top = col[(jt * S + r) * kSpecCols];
+#pragma unroll
+          for (int i = 0; i < R; ++i) cfma(acc[i][r], top, zs[i]);
+        }
+      }
+      for (int j = jt - 2; j >= 0; --j) {
+#pragma unroll
+        for (int r = 0; r < S; ++r) {
+          const cpx<T> c = col[(j * S + r) * kSpecCols];
+#pragma unroll
+          for (int i = 0; i < R; ++i) {
+            cpx<T> a = c;
+            cfma(a, acc[i][r], zs[i]);
+            acc[i][r] = a;
+          }
+        }
       }
     }
 #pragma unroll
-    for (int j = 0; j < kSpecRows; ++j) {
-      if (u0 + j < Ph) {
-        cpx<T>* o = out + (int64_t)(u0 + j) * Pw2p;
-        if (va < Pw2) o[va] = acc[j][0];
-        if (vb < Pw2) o[vb] = acc[j][1];
+    for (int i = 0; i < R; ++i) {
+#pragma unroll
+      for (int r = 1; r < S; ++r) acc[i][r] = acc[i][r] * ldg_cpx(tw_h + r * u[i]);
+      if constexpr (S > 1) small_dft<T, false, S>(acc[i]);
+      if (u0 + i < Q && v < Pw2) {
+#pragma unroll
+        for (int m = 0; m < S; ++m) out[(int64_t)(u0 + i + m * Q) * Pw2p] = acc[i][m];
       }
     }
   }
@@ -288,14 +331,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int li
 }
 constexpr int kWaitLimit = 1 << 20;
 
-__device__ __forceinline__ cf ldg_cpx(const cf* p) {
-  const float2 v = __ldg((const float2*)p);
-  return mk(v.x, v.y);
-}
-__device__ __forceinline__ cd ldg_cpx(const cd* p) {
-  const double2 v = __ldg((const double2*)p);
-  return mk(v.x, v.y);
-}
 
 // ------------------------------------------ row pass (A1 folds + A6 rows) ---
 //
@@ -1598,16 +1633,23 @@ __global__ void __launch_bounds__(kIrThreads, 2) k_row_ifft_ir(IRowArgs a, const
   }
 }
 
+template <typename T, int S>
+void run_kernel_spectra_s(const Plan& p, char* ws, cudaStream_t st) {
+  const int tiles = (p.Pw2 + kSpecCols - 1) / kSpecCols;
+  constexpr int rows = kSpecThreads / 32 * kSpecRows<T>;      // of Ph / S, a block and step
+  // two blocks an SM, no share without rows
+  const int shares = std::max(1, std::min((p.Ph / S + rows - 1) / rows, 304 / (tiles * 2 * p.n) + 1));
+  dim3 g(tiles, 2 * shares, p.n);
+  k_kernel_spectra<T, S><<<g, kSpecThreads, 0, st>>>(
+      (const double*)(ws + p.off_kd), p.t1, p.t2, p.Ph, p.Pw, p.Pw2, p.Pw2p, shares,
+      (const cpx<T>*)(ws + p.off_tw_h), (const cpx<T>*)(ws + p.off_tw_w), (cpx<T>*)(ws + p.off_khat));
+}
 template <typename T>
 void run_kernel_spectra(const Plan& p, char* ws, cudaStream_t st) {
-  const cpx<T>* tw_h = (const cpx<T>*)(ws + p.off_tw_h);
-  const cpx<T>* tw_w = (const cpx<T>*)(ws + p.off_tw_w);
-  dim3 g((p.Pw2 + kSpecCols - 1) / kSpecCols, 2, p.n);
-  const size_t sm = sizeof(cpx<T>) * ((size_t)kMaxN * kSpecCols + p.Ph);
-  cudaFuncSetAttribute(k_kernel_spectra<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_kernel_spectra<T><<<g, kFftThreads, sm, st>>>((const double*)(ws + p.off_kd), p.t1, p.t2, p.Ph,
-                                                  p.Pw, p.Pw2, p.Pw2p, tw_h, tw_w,
-                                                  (cpx<T>*)(ws + p.off_khat));
+  if (p.Ph % 4 == 0) run_kernel_spectra_s<T, 4>(p, ws, st);
+  else if (p.Ph % 3 == 0) run_kernel_spectra_s<T, 3>(p, ws, st);
+  else if (p.Ph % 2 == 0) run_kernel_spectra_s<T, 2>(p, ws, st);
+  else run_kernel_spectra_s<T, 1>(p, ws, st);
 }
 
 // Shared-memory target of the row pass: two resident blocks per SM.
