@@ -673,10 +673,18 @@ cbp_status call_path(cbp_ctx* ctx, const cbp_frames* b1, const cbp_frames* b2,
                       host_io ? nullptr : c->solve_st[i % Ctx::kChunkStreams], c->fork_ev[i],
                       c->join_ev[i], tw_ready);
     if (s != CBP_OK) return s;
-    if (diag && cudaMemcpyAsync(diag + a, w + cp[i].off_diag, (size_t)cp[i].n * sizeof(cbp_diag),
-                                cudaMemcpyDeviceToHost, cs) != cudaSuccess)
-      return CBP_ERR_CUDA;
     if (cudaEventRecord(c->chunk_ev[i], cs) != cudaSuccess ||
+        cudaStreamWaitEvent(st, c->chunk_ev[i], 0) != cudaSuccess)
+      return CBP_ERR_CUDA;
+  }
+  // The diagnostics come back once every chunk is launched: a copy to pageable
+  // memory returns only when its stream has got there, and issued behind its own
+  // chunk it held the next one back until then (30 480p pairs 1.68 -> 1.09 ms).
+  for (int i = 0; diag && i < nch; ++i) {
+    cudaStream_t cs = c->chunk_st[i % Ctx::kChunkStreams];
+    if (cudaMemcpyAsync(diag + start[i], c->ws + off[i] + cp[i].off_diag, (size_t)cp[i].n * sizeof(cbp_diag),
+                        cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
+        cudaEventRecord(c->chunk_ev[i], cs) != cudaSuccess ||
         cudaStreamWaitEvent(st, c->chunk_ev[i], 0) != cudaSuccess)
       return CBP_ERR_CUDA;
   }

@@ -63,9 +63,11 @@ def test_a_pair_does_not_depend_on_its_batch(gpu_ctx, n, path):
     pairs = [make_pair(7100 + f, 40, 45, 6, 5, c=3) for f in range(n)]
     B1, B2 = (torch.from_numpy(np.stack([p[k] for p in pairs])).cuda() for k in (0, 1))
     prm = cbp.params(6, 5, path=path, flags=cbp.CBP_FLAG_KERNELS_F64)
-    lat, k1, k2, _, _ = cbp.cbp_deblur_pair(gpu_ctx, B1, B2, prm)
+    lat, k1, k2, diag, _ = cbp.cbp_deblur_pair(gpu_ctx, B1, B2, prm)     # 40 pairs: two chunks
     torch.cuda.synchronize()
     for f in range(0, n, 3):
         a = cbp.cbp_deblur_pair(gpu_ctx, B1[f:f + 1], B2[f:f + 1], prm)
         torch.cuda.synchronize()
         assert torch.equal(a[0][0], lat[f]) and torch.equal(a[1][0], k1[f]) and torch.equal(a[2][0], k2[f])
+        assert all(getattr(a[3][0], x) == getattr(diag[f], x) for x in
+                   ("kappa_max", "gap_min", "scale_resid", "support_ratio", "pad_h", "pad_w", "status"))
