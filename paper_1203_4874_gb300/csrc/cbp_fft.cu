@@ -359,6 +359,7 @@ struct RowPassArgs {
   int fft_frames;      // frames whose rows are transformed (1: single-kernel form)
   int Pw, Pw2, Pw2p, half, nbr, rw;
   int wl;              // width the shared-memory layout is sized for (max W_Bk)
+  uint32_t mK;         // half: ceil(2^32 / (pl.n / 2 + 1)), for the split's task indices
   FftPlan pl;          // plan of Pw/2 (half) or Pw
 };
 
@@ -538,7 +539,7 @@ __device__ __forceinline__ Edge<In> stage_rows_bulk(In* dst, int* rph, const In*
 }
 
 template <typename T, typename In, bool FOLD, bool FFT>
-__global__ void __launch_bounds__(kRowPassThreads)
+__global__ void __launch_bounds__(kRowPassThreads, sizeof(T) == 8 && FOLD && FFT ? 1 : 2)
 k_row_pass(RowPassArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
   using Acc = typename FoldAcc<In>::type;
   extern __shared__ __align__(16) char smem[];
@@ -694,21 +695,25 @@ k_row_pass(RowPassArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
       cpx<T>* Z = plan_is<CBP_ROW_PLAN>(a.pl) ? fft_rest_fixed<T, false, CBP_ROW_PLAN>(b0, b1, nr, tw)
                                               : fft_block<T, false>(b0, b1, a.pl, nr, tw, 1);
       RP_MARK(4);
-      // a thread keeps its output columns k (and their twiddle) over the rows
-      for (int k = threadIdx.x; k < a.Pw2; k += blockDim.x) {
-        if (a.half) {
-          const int ka = k < N ? k : 0, kb = k > 0 ? N - k : 0;
-          const cpx<T> w = tw_w[k];                 // X = e - i w d, w = exp(-2 pi i k / Pw)
-          for (int i = 0; i < nr; ++i) {
-            const cpx<T>* z = Z + i * N;
-            const cpx<T> zk = z[ka], zc = conj(z[kb]);
-            const cpx<T> e = (T)0.5 * (zk + zc), d = (T)0.5 * (zk - zc);
-            const cpx<T> wd = w * d;
-            spec[(int64_t)row_of(g, i) * a.Pw2p + k] = mk<T>(e.re + wd.im, e.im - wd.re);
-          }
-        } else {
-          for (int i = 0; i < nr; ++i) spec[(int64_t)row_of(g, i) * a.Pw2p + k] = Z[i * N + k];
+      if (a.half) {
+        // the real-FFT split, bins k and N - k together: with
+        // s, d = z[k] +- conj z[N - k] and q = w d / 2, w = exp(-2 pi i k / Pw),
+        // X[k] = s / 2 - i q and X[N - k] = conj(s / 2 + i q) -- six additions
+        // and multiplications a bin (14 one bin at a time)
+        const int K = N / 2 + 1;
+        for (int t = threadIdx.x; t < nr * K; t += kRowPassThreads) {
+          const int i = K > 1 ? (int)__umulhi((unsigned)t, a.mK) : t, k = t - i * K;
+          const cpx<T>* z = Z + i * N;
+          const cpx<T> zk = z[k], zc = conj(z[k ? N - k : 0]);
+          const cpx<T> w = ldg_cpx(tw_w + k);
+          const cpx<T> sm = zk + zc, q = mk<T>((T)0.5 * w.re, (T)0.5 * w.im) * (zk - zc);
+          cpx<T>* o = spec + (int64_t)row_of(g, i) * a.Pw2p;
+          o[k] = mk<T>(fma((T)0.5, sm.re, q.im), fma((T)0.5, sm.im, -q.re));
+          if (2 * k != N) o[N - k] = mk<T>(fma((T)0.5, sm.re, -q.im), -fma((T)0.5, sm.im, q.re));
         }
+      } else {
+        for (int k = threadIdx.x; k < a.Pw2; k += kRowPassThreads)
+          for (int i = 0; i < nr; ++i) spec[(int64_t)row_of(g, i) * a.Pw2p + k] = Z[i * N + k];
       }
     }
     RP_MARK(5);
@@ -1306,6 +1311,7 @@ k_col_deconv(ColArgs a) {
 }
 
 struct IRowArgs {
+  uint32_t mK;       // half: ceil(2^32 / (pl.n / 2 + 1)), for the split's task indices
   const cf* tw2;     // in-register inverse: w_N^(n1 k2) at [n1][k2]
   const void* ihat;  // cpx<T> [n][C][H][Pw2]
   void* latent;      // TO [n][C][H][W]
@@ -1412,7 +1418,7 @@ __device__ __forceinline__ void first_stage_spec(const cpx<T>* raw, int Pw2p, co
 // at a time, the next group's spectrum rows in flight (bulk copies on an
 // mbarrier per staging buffer) while the current group is transformed.
 template <typename T>
-__global__ void __launch_bounds__(kRowPassThreads)
+__global__ void __launch_bounds__(kRowPassThreads, 2)
 k_row_ifft(IRowArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
   extern __shared__ __align__(16) char smem[];
   const int N = a.pl.n, NB = a.nbr;
@@ -1446,7 +1452,14 @@ k_row_ifft(IRowArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
   if (ngroups > 0)
     stage_spec_rows_bulk<T>(raw0, [&](int i) { return src + (int64_t)row_of(0, i) * a.Pw2p; },
                             min(NB, nrows), a.Pw2p, &bars[0]);
-  const T sc = (T)a.scale;
+  // doubles: the Hermitian split ahead of the first stage, a pair of elements at
+  // a time, six additions and multiplications each (14 where the stage does it
+  // element by element); the double units bound the pass (24 480p planes 500 ->
+  // 447 us).  Floats are not: the stage does it (either way 29.5 us for 15 480p
+  // planes, 47 for nine 720p ones).
+  const bool pre = sizeof(T) == 8 && a.half;
+  // the exact halves and doubles of both splits gathered here
+  const T sc = (T)(a.half && !pre ? 2.0 * a.scale : a.scale);
   for (int g = 0; g < ngroups; ++g) {
     const int nr = min(NB, nrows - g * NB);
     if (g + 1 < ngroups) {
@@ -1465,11 +1478,25 @@ k_row_ifft(IRowArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
       return;
     }
     cpx<T>* const rw0 = (g & 1) ? raw1 : raw0;
+    if (pre) {
+      // elements m and N - m together, in place: with s, d = X[m] +- conj X[N - m]
+      // and o = conj(w) d, twice Z[m] is s + i o and twice Z[N - m] conj(s) + i conj(o)
+      const int K = N / 2 + 1;
+      for (int t = threadIdx.x; t < nr * K; t += kRowPassThreads) {
+        const int i = K > 1 ? (int)__umulhi((unsigned)t, a.mK) : t, m = t - i * K;
+        cpx<T>* X = rw0 + i * a.Pw2p;
+        const cpx<T> xk = X[m], xc = conj(X[N - m]);
+        const cpx<T> sm = xk + xc, o = conj(ldg_cpx(tw_w + m)) * (xk - xc);
+        X[m] = mk<T>(sm.re - o.im, sm.im + o.re);
+        if (m && 2 * m != N) X[N - m] = mk<T>(sm.re + o.im, o.re - sm.im);
+      }
+      __syncthreads();
+    }
     // first inverse stage straight from the staged spectrum rows into b0
     if (plan_is<CBP_ROW_PLAN>(a.pl))
-      stage_first_spec<T, 9, 972>(rw0, a.Pw2p, tw_w, a.half, a.Pw2, b0, a.pl.st[0], 972, nr);
+      stage_first_spec<T, 9, 972>(rw0, a.Pw2p, tw_w, a.half && !pre, a.Pw2, b0, a.pl.st[0], 972, nr);
     else
-      first_stage_spec<T>(rw0, a.Pw2p, tw_w, a.half, a.Pw2, b0, a.pl, nr);
+      first_stage_spec<T>(rw0, a.Pw2p, tw_w, a.half && !pre, a.Pw2, b0, a.pl, nr);
     __syncthreads();
     cpx<T>* b1 = L.b1_alias ? rw0 : (cpx<T>*)(smem + L.b1);
     cpx<T>* Z = plan_is<CBP_ROW_PLAN>(a.pl) ? fft_rest_fixed<T, true, CBP_ROW_PLAN>(b0, b1, nr, tw)
@@ -1477,20 +1504,18 @@ k_row_ifft(IRowArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
     for (int i = 0; i < nr; ++i) {
       const cpx<T>* z = Z + i * N;
       const int64_t ob = obase + (int64_t)row_of(g, i) * a.W;
+      // a half-length transform's element m holds columns 2 m and 2 m + 1
       if (a.half && !a.out_f64 && (((ob * 4 + (uintptr_t)outp) & 7) == 0)) {
         float2* o2 = (float2*)((float*)outp + ob);
         for (int m = threadIdx.x; m < (a.W >> 1); m += blockDim.x)
-          o2[m] = make_float2((float)((T)2 * sc * z[m].re), (float)((T)2 * sc * z[m].im));
+          o2[m] = make_float2((float)(sc * z[m].re), (float)(sc * z[m].im));
         if ((a.W & 1) && threadIdx.x == 0)
-          ((float*)outp)[ob + a.W - 1] = (float)((T)2 * sc * z[a.W >> 1].re);
+          ((float*)outp)[ob + a.W - 1] = (float)(sc * z[a.W >> 1].re);
       } else {
         for (int c = threadIdx.x; c < a.W; c += blockDim.x) {
-          T v;
-          if (a.half) v = (c & 1) ? (T)2 * z[c >> 1].im : (T)2 * z[c >> 1].re;
-          else v = z[c].re;
-          v *= sc;
-          if (a.out_f64) ((double*)outp)[ob + c] = (double)v;
-          else ((float*)outp)[ob + c] = (float)v;
+          const T x = a.half ? ((const T*)z)[c] : z[c].re;
+          if (a.out_f64) ((double*)outp)[ob + c] = (double)(sc * x);
+          else ((float*)outp)[ob + c] = (float)(sc * x);
         }
       }
     }
@@ -1655,6 +1680,25 @@ void run_kernel_spectra(const Plan& p, char* ws, cudaStream_t st) {
 // Shared-memory target of the row pass: two resident blocks per SM.
 constexpr size_t kRowPassSmemTarget = 112 * 1024;
 
+// Blocks for h independent rows of each of `planes` planes, groups of nbr rows
+// a step, two blocks per SM: the split whose slowest SM takes the fewest steps,
+// one more counted for a block's start.  Blocks of 32 rows left some calls a
+// last wave of a few blocks and small ones most SMs idle (with the passes over
+// doubles held to two blocks an SM: 24 480p planes of doubles 832 -> 679 us forward,
+// 447 -> 339 back; one 64 x 64 pair's inverse rows 35 -> 11; 15 480p planes of
+// floats 29.6 -> 23.5; 90 1080p planes 420 -> 408).
+int row_blocks(int h, int planes, int nbr) {
+  constexpr int kSlots = 304;
+  long best = 0;
+  int gx = 1;
+  for (int steps = 1; steps * nbr <= 64 || steps == 1; ++steps) {
+    const int x = (h + steps * nbr - 1) / (steps * nbr);
+    const long cost = (((long)x * planes + kSlots - 1) / kSlots) * (steps + 1);
+    if (steps == 1 || cost <= best) best = cost, gx = x;
+  }
+  return gx;
+}
+
 template <typename T, typename In, bool FOLD, bool FFT>
 void run_row_pass_t(const Plan& p, const RowPassArgs& a, int gx, int gz, char* ws,
                     cudaStream_t st) {
@@ -1700,6 +1744,7 @@ void run_row_pass(const Plan& p, const FrameDesc& b1, const FrameDesc& b2, char*
   a.Pw2p = p.Pw2p;
   a.half = p.pw_half;
   a.pl = p.pw_half ? p.fp_w2 : p.fp_w;
+  a.mK = magic_div(a.pl.n / 2 + 1);
   a.wl = p.W1 > p.W2 ? p.W1 : p.W2;
   constexpr int E = 16 / (int)sizeof(In);
   a.rw = ((a.wl + 2 * E + E - 1) / E) * E;
@@ -1714,16 +1759,17 @@ void run_row_pass(const Plan& p, const FrameDesc& b1, const FrameDesc& b2, char*
     }
   }
   const int hmax = p.H1 > p.H2 ? p.H1 : p.H2;
-  const int gx = fold ? p.M : (hmax + 31) / 32;
   const int gz = fold ? 2 : a.fft_frames;
+  const int gx = fold ? p.M : row_blocks(hmax, p.n * p.C * gz, a.nbr);
   if constexpr (sizeof(T) == 4 && sizeof(In) == 4) {
     if (row_pass_ir_ok(p, b1, b2, fft)) {
       a.rw = ((2 * a.pl.n + 4 + 3) / 4) * 4;       // transform length + the 16-byte phase
       const RowIrSmem L = row_ir_layout(a.rw);
       auto kern = fold ? k_row_pass_ir<36, 27, true> : k_row_pass_ir<36, 27, false>;
+      const int gi = fold ? p.M : row_blocks(hmax, p.n * p.C * gz, kIrRows);
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
       cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      kern<<<dim3(gx, p.n * p.C, gz), kIrThreads, L.total, st>>>(a, (const cf*)(ws + p.off_tw_w));
+      kern<<<dim3(gi, p.n * p.C, gz), kIrThreads, L.total, st>>>(a, (const cf*)(ws + p.off_tw_w));
       return;
     }
   }
@@ -1815,6 +1861,7 @@ void run_row_ifft(const Plan& p, char* ws, void* latent, int out_f64, cudaStream
   a.half = p.pw_half;
   a.scale = 1.0 / ((double)p.Ph * (double)p.Pw);
   a.pl = plw;
+  a.mK = magic_div(plw.n / 2 + 1);
   a.nbr = 1;
   for (int nb = 8; nb >= 1; nb >>= 1) {
     if (irow_layout(plw.n, plw.ntw, p.Pw2p, nb, sizeof(cpx<T>)).total <= kRowPassSmemTarget &&
@@ -1823,11 +1870,12 @@ void run_row_ifft(const Plan& p, char* ws, void* latent, int out_f64, cudaStream
       break;
     }
   }
-  dim3 g((p.H + 31) / 32, p.n * p.C);
+  dim3 g(row_blocks(p.H, p.n * p.C, a.nbr), p.n * p.C);
   if constexpr (sizeof(T) == 4) {
     // in-register transforms: float output rows on 8-byte boundaries, 972 = 36 x 27
     if (p.pw_half && plw.n == 972 && !out_f64 && !lat_tab && (p.W % 2) == 0 &&
         ((uintptr_t)latent & 7) == 0 && p.off_tw2r) {
+      g.x = row_blocks(p.H, p.n * p.C, kIrRows);
       const size_t smi = irow_ir_layout(p.Pw2p).total;
       cudaFuncSetAttribute(k_row_ifft_ir<36, 27>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smi);
       cudaFuncSetAttribute(k_row_ifft_ir<36, 27>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);

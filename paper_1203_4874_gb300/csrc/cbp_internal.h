@@ -125,6 +125,7 @@ const Roots& make_roots(int M);
 
 // ---- planning (cbp_plan.cpp) ----
 int next_7_smooth(int n);
+uint32_t magic_div(int d);   // ceil(2^32 / d): __umulhi(x, .) = x / d for x d < 2^32; 0 for d <= 1
 bool make_fft_plan(int n, FftPlan* p);
 cbp_status make_plan(const cbp_frames* b1, const cbp_frames* b2, const cbp_params* prm,
                      Plan* plan);

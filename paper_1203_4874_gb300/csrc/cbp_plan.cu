@@ -45,7 +45,7 @@ const Roots& make_roots(int M) {
   return table[m];
 }
 
-static uint32_t magic_div(int d) {
+uint32_t magic_div(int d) {
   return d <= 1 ? 0u : (uint32_t)(((uint64_t(1) << 32) + (uint64_t)d - 1) / (uint64_t)d);
 }
 
