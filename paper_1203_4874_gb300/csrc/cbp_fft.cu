@@ -357,6 +357,7 @@ struct RowPassArgs {
   int* err;            // set when a copy does not complete in time
   int M;
   int fft_frames;      // frames whose rows are transformed (1: single-kernel form)
+  int xf;              // > 0: folds and transforms in blocks of their own, xf of the latter a plane
   int Pw, Pw2, Pw2p, half, nbr, rw;
   int wl;              // width the shared-memory layout is sized for (max W_Bk)
   uint32_t mK;         // half: ceil(2^32 / (pl.n / 2 + 1)), for the split's task indices
@@ -538,14 +539,41 @@ __device__ __forceinline__ Edge<In> stage_rows_bulk(In* dst, int* rph, const In*
   return e;
 }
 
+// What a block of the row passes does.  One read of the frames serves the folds
+// and the transforms: block x of a plane (a frame's channel) takes the rows of
+// fold bin x and transforms them too.  That fixes the number of blocks (M a
+// plane), and a call of few planes leaves SMs idle, or a last wave with few
+// blocks; with a.xf > 0 the folds (M blocks a plane) and the transforms (a.xf
+// blocks a plane) have blocks of their own, and the rows are read twice, the
+// second time mostly from L2.  Rows are independent and a bin's rows stay in one
+// block, so both arrangements give the same bits.
+struct RowRole {
+  int frame, X;
+  bool fold, fft;
+};
+template <bool FOLD, bool FFT>
+__device__ __forceinline__ RowRole row_role(const RowPassArgs& a) {
+  const bool split = FOLD && FFT && a.xf > 0;
+  const int z = blockIdx.z, frame = split ? z & 1 : z;
+  RowRole r;
+  r.frame = frame;
+  r.fold = FOLD && (!split || z < 2);
+  r.fft = FFT && frame < a.fft_frames && (!split || z >= 2);
+  r.X = split ? (z < 2 ? a.M : a.xf) : (int)gridDim.x;
+  return r;
+}
+
 template <typename T, typename In, bool FOLD, bool FFT>
 __global__ void __launch_bounds__(kRowPassThreads, sizeof(T) == 8 && FOLD && FFT ? 1 : 2)
 k_row_pass(RowPassArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
   using Acc = typename FoldAcc<In>::type;
   extern __shared__ __align__(16) char smem[];
-  const FrameDesc& fr = a.fr[blockIdx.z];
+  const RowRole role = row_role<FOLD, FFT>(a);
+  const bool fold = role.fold, fft = role.fft;
+  const int fz = role.frame;
+  const FrameDesc& fr = a.fr[fz];
   const int N = a.pl.n, NB = a.nbr, W = fr.w, M = a.M;
-  const bool fft = FFT && (int)blockIdx.z < a.fft_frames;
+  if ((int)blockIdx.x >= role.X || !(fold || fft)) return;
   const RowPassSmem L = row_pass_layout(N, a.pl.ntw, a.wl, NB, a.rw, sizeof(cpx<T>), sizeof(In),
                                         FOLD, FFT);
   cpx<T>* tw = (cpx<T>*)(smem + L.tw);
@@ -565,10 +593,10 @@ k_row_pass(RowPassArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
   uint32_t par = 0u;   // bit b: phase parity of buffer b's next completion
   if (fft) load_twiddles(tw, stw, a.pl.ntw);
   Acc creg[kColRegs];
-  if (FOLD && L.col_smem)
+  if (fold && L.col_smem)
     for (int c = threadIdx.x; c < W; c += blockDim.x) colacc[c] = Acc();
   const int fc = blockIdx.y, f = fc / fr.c, ch = fc % fr.c;
-  const int x0 = blockIdx.x, X = gridDim.x;
+  const int x0 = blockIdx.x, X = role.X;
   const int nrows = x0 < fr.h ? (fr.h - x0 + X - 1) / X : 0;
   const int ngroups = (nrows + NB - 1) / NB;
   const In* fb = (const In*)frame_base(fr, f) + (int64_t)ch * fr.cs;
@@ -579,7 +607,7 @@ k_row_pass(RowPassArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
                                             min(NB, nrows), W, a.rw, &bars[0]);
     if (e0.at >= 0) raw0[e0.at] = e0.v;
   }
-  cpx<T>* spec = fft ? (cpx<T>*)a.spec[blockIdx.z] + (int64_t)fc * fr.h * a.Pw2p : nullptr;
+  cpx<T>* spec = fft ? (cpx<T>*)a.spec[fz] + (int64_t)fc * fr.h * a.Pw2p : nullptr;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #ifdef CBP_PHASE_TIMING
   long long rp_t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -608,7 +636,7 @@ k_row_pass(RowPassArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
     RP_MARK(1);
     In* const rw0 = (g & 1) ? raw1 : raw0;
     const int* ph = rph + (g & 1) * NB;
-    if (FOLD) {
+    if (fold) {
       // element c of staged row i is rw0[roff(i) + c]
       auto roff = [&](int i) { return i * a.rw + ph[i]; };
       // column folds: this block's bin, one thread per column (full groups
@@ -679,13 +707,13 @@ k_row_pass(RowPassArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
     }
     __syncthreads();
     RP_MARK(3);
-    if (FOLD) {
+    if (fold) {
       const int nseg = max(1, kRowPassThreads / (nr * M));
       for (int t = threadIdx.x; t < nr * M; t += blockDim.x) {
         const int i = t / M, m = t - i * M;
         Acc v = rb[(i * nseg) * M + m];
         for (int sg = 1; sg < nseg; ++sg) v.merge(rb[(i * nseg + sg) * M + m]);
-        v.store((char*)a.bins_r[blockIdx.z] + 8 * (((int64_t)fc * M + m) * fr.h + row_of(g, i)));
+        v.store((char*)a.bins_r[fz] + 8 * (((int64_t)fc * M + m) * fr.h + row_of(g, i)));
       }
     }
     if (fft) {
@@ -728,12 +756,12 @@ k_row_pass(RowPassArgs a, const cpx<T>* tw_w, const cpx<T>* stw) {
 #ifdef CBP_PHASE_TIMING
   if (threadIdx.x == 0 && blockIdx.x == 1 && blockIdx.y < 2)
     printf("row_pass fold=%d fft=%d z=%d groups=%d nb=%d | issue %lld wait %lld folds %lld convert+sync %lld "
-           "fft %lld post %lld endsync %lld loop %lld\n", (int)FOLD, (int)fft, (int)blockIdx.z,
+           "fft %lld post %lld endsync %lld loop %lld\n", (int)FOLD, (int)fft, fz,
            ngroups, NB, rp_t[0], rp_t[1], rp_t[2], rp_t[3], rp_t[4], rp_t[5], rp_t[6], rp_t[7]);
 #endif
-  if (FOLD) {
+  if (fold) {
     bool finite = true;
-    char* dst = (char*)a.bins_c[blockIdx.z] + 8 * (((int64_t)fc * M + x0) * W);
+    char* dst = (char*)a.bins_c[fz] + 8 * (((int64_t)fc * M + x0) * W);
     if (!L.col_smem) {
 #pragma unroll
       for (int j = 0; j < kColRegs; ++j) {
@@ -802,9 +830,12 @@ __global__ void __launch_bounds__(kIrThreads, 2)
 k_row_pass_ir(RowPassArgs a, const cf* tw_w) {
   constexpr int N = N1 * N2;
   extern __shared__ __align__(16) char smem[];
-  const FrameDesc& fr = a.fr[blockIdx.z];
+  const RowRole role = row_role<FOLD, true>(a);
+  const bool fold = role.fold, fft = role.fft;
+  const int fz = role.frame;
+  const FrameDesc& fr = a.fr[fz];
   const int W = fr.w, M = a.M, rw = a.rw;
-  const bool fft = (int)blockIdx.z < a.fft_frames;
+  if ((int)blockIdx.x >= role.X || !(fold || fft)) return;
   const RowIrSmem L = row_ir_layout(rw);
   float* const raw = (float*)(smem + L.raw);
   TwoSum* rb = (TwoSum*)(smem + L.rb);
@@ -825,17 +856,17 @@ k_row_pass_ir(RowPassArgs a, const cf* tw_w) {
   __syncthreads();
   uint32_t par = 0u;
   const int fc = blockIdx.y, f = fc / fr.c, ch = fc % fr.c;
-  const int x0 = blockIdx.x, X = gridDim.x;
+  const int x0 = blockIdx.x, X = role.X;
   const int nrows = x0 < fr.h ? (fr.h - x0 + X - 1) / X : 0;
   const int ngroups = (nrows + kIrRows - 1) / kIrRows;
   const float* fb = (const float*)frame_base(fr, f) + (int64_t)ch * fr.cs;
   auto row_of = [&](int g, int i) { return x0 + (g * kIrRows + i) * X; };
-  cf* spec = fft ? (cf*)a.spec[blockIdx.z] + (int64_t)fc * fr.h * a.Pw2p : nullptr;
+  cf* spec = fft ? (cf*)a.spec[fz] + (int64_t)fc * fr.h * a.Pw2p : nullptr;
   // column folds: this thread's column pairs (c, c + 1), c = 2 (tid + kIrThreads j),
   // accumulated in shared memory across the groups
   constexpr int kColPairs = 4;
   TwoSum* colacc = (TwoSum*)(smem + L.colacc);
-  if (FOLD)
+  if (fold)
     for (int c = tid; c < W; c += kIrThreads) colacc[c] = TwoSum();
   Edge<float> en{0.f, -1};
   if (ngroups > 0)
@@ -857,7 +888,7 @@ k_row_pass_ir(RowPassArgs a, const cf* tw_w) {
       if (CBP_CHECK(i < kIrRows && rph[i] + c < rw, 0)) raw[i * rw + rph[i] + c] = 0.f;
     }
     __syncthreads();
-    if (FOLD) {
+    if (fold) {
       // column folds (this block's bin), float pairs
 #pragma unroll
       for (int j = 0; j < kColPairs; ++j) {
@@ -902,14 +933,14 @@ k_row_pass_ir(RowPassArgs a, const cf* tw_w) {
       }
     }
     __syncthreads();
-    if (FOLD) {
+    if (fold) {
       const int nseg = max(1, kIrThreads / (nr * M));
       for (int t = tid; t < nr * M; t += kIrThreads) {
         const int i = t / M, m = t - i * M;
         TwoSum v = rb[(i * nseg) * M + m];
         for (int sg = 1; sg < nseg; ++sg) v.merge(rb[(i * nseg + sg) * M + m]);
         if (CBP_CHECK(row_of(g, i) < fr.h && (i * nseg + nseg) * M <= kIrThreads, 1))
-          v.store((char*)a.bins_r[blockIdx.z] + 8 * (((int64_t)fc * M + m) * fr.h + row_of(g, i)));
+          v.store((char*)a.bins_r[fz] + 8 * (((int64_t)fc * M + m) * fr.h + row_of(g, i)));
       }
     }
     if (fft) {
@@ -990,9 +1021,9 @@ k_row_pass_ir(RowPassArgs a, const cf* tw_w) {
                                   min(kIrRows, nrows - g1 * kIrRows), W, rw, bar);
     }
   }
-  if (FOLD) {
+  if (fold) {
     bool finite = true;
-    char* dst = (char*)a.bins_c[blockIdx.z] + 8 * (((int64_t)fc * M + x0) * W);
+    char* dst = (char*)a.bins_c[fz] + 8 * (((int64_t)fc * M + x0) * W);
     __syncthreads();
     for (int c = tid; c < W; c += kIrThreads) {
       finite = finite && colacc[c].finite();
@@ -1699,6 +1730,23 @@ int row_blocks(int h, int planes, int nbr) {
   return gx;
 }
 
+// Blocks a plane of the transforms' own when the folds and the transforms are
+// better apart (row_role), else 0: where the M blocks a plane fill up to 7/10 of
+// the slots (two an SM), or a first wave and up to 1/8 of a second.  Together
+// against apart, us: a 64 x 64 FP64 pair (10 blocks) 23.6 / 12.6, a 480p pair
+// (22) 39 / 22, four 1000 x 1300 pairs (72) 299 / 196, seven 1080p pairs (126)
+// 154 / 117, two 720p colour pairs (204) 86 / 79; three ragged 720p colour pairs
+// (234) 116 / 118; 15 480p pairs (330) 87 / 76; four 480p colour pairs (408)
+// 61 / 68, seven 720p ones (714) 212 / 241.
+int row_split(int h, int M, int planes, int fft_planes) {
+  constexpr int kSlots = 304;
+  const int blocks = M * planes;
+  if (blocks > kSlots + kSlots / 8 || (blocks > kSlots * 7 / 10 && blocks <= kSlots)) return 0;
+  // about as many rows a block as an even share, 8 to 32
+  const int r = std::max(8, std::min(32, (int)((double)h * fft_planes / kSlots)));
+  return (h + r - 1) / r;
+}
+
 template <typename T, typename In, bool FOLD, bool FFT>
 void run_row_pass_t(const Plan& p, const RowPassArgs& a, int gx, int gz, char* ws,
                     cudaStream_t st) {
@@ -1759,14 +1807,20 @@ void run_row_pass(const Plan& p, const FrameDesc& b1, const FrameDesc& b2, char*
     }
   }
   const int hmax = p.H1 > p.H2 ? p.H1 : p.H2;
-  const int gz = fold ? 2 : a.fft_frames;
-  const int gx = fold ? p.M : row_blocks(hmax, p.n * p.C * gz, a.nbr);
+  int gz = fold ? 2 : a.fft_frames;
+  const int planes = p.n * p.C * gz;
+  int gx = fold ? p.M : row_blocks(hmax, planes, a.nbr);
+  a.xf = fold && fft ? row_split(hmax, p.M, planes, p.n * p.C * a.fft_frames) : 0;
+  if (a.xf) {
+    gx = std::max(p.M, a.xf);
+    gz = 4;
+  }
   if constexpr (sizeof(T) == 4 && sizeof(In) == 4) {
     if (row_pass_ir_ok(p, b1, b2, fft)) {
       a.rw = ((2 * a.pl.n + 4 + 3) / 4) * 4;       // transform length + the 16-byte phase
       const RowIrSmem L = row_ir_layout(a.rw);
       auto kern = fold ? k_row_pass_ir<36, 27, true> : k_row_pass_ir<36, 27, false>;
-      const int gi = fold ? p.M : row_blocks(hmax, p.n * p.C * gz, kIrRows);
+      const int gi = fold ? gx : row_blocks(hmax, planes, kIrRows);
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
       cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
       kern<<<dim3(gi, p.n * p.C, gz), kIrThreads, L.total, st>>>(a, (const cf*)(ws + p.off_tw_w));

@@ -40,3 +40,24 @@ def test_given_kernels(gpu_ctx, n, c, h, w, t1, t2, dt, path, bar):
     for i in range(n):
         want = oracle.deconvolve_dual(b1[i].astype(np.float64), b2[i].astype(np.float64), k1[i], k2[i], h, w, eps)
         assert rel(out[i].cpu().numpy(), want) <= bar
+
+
+@pytest.mark.parametrize("h,w,c,t1,t2,dt,path", [(50, 61, 1, 6, 5, torch.float32, "mixed"),
+                                                 (33, 48, 2, 5, 5, torch.float64, "fp64"),
+                                                 (24, 1920, 1, 17, 15, torch.float32, "mixed"),
+                                                 (24, 1919, 1, 9, 11, torch.float32, "fp64")])
+def test_folds_and_transforms_apart_and_together(gpu_ctx, h, w, c, t1, t2, dt, path):
+    """A pair alone has blocks of their own for the folds and the transforms, one of
+    a batch that fills the GPU shares them: the same bits."""
+    from paper_1203_4874_gb300 import cbp
+    n = 30
+    g = torch.Generator().manual_seed(h + w)
+    b1 = torch.rand((n, c, h + t1 - 1, w + t1 - 1), generator=g, dtype=dt).cuda()
+    b2 = torch.rand((n, c, h + t2 - 1, w + t2 - 1), generator=g, dtype=dt).cuda()
+    for n_ in (8, 15, n):                  # 15 pairs: one chunk
+        prm = cbp.params(t1, t2, path=path, eps=1e-3, flags=cbp.CBP_FLAG_KERNELS_F64)
+        lat, k1, k2, _, _ = cbp.cbp_deblur_pair(gpu_ctx, b1[:n_], b2[:n_], prm)
+        for f in (0, n_ // 2, n_ - 1):
+            a = cbp.cbp_deblur_pair(gpu_ctx, b1[f:f + 1], b2[f:f + 1], prm)
+            torch.cuda.synchronize()
+            assert torch.equal(a[0][0], lat[f]) and torch.equal(a[1][0], k1[f]) and torch.equal(a[2][0], k2[f])
