@@ -288,6 +288,9 @@ __device__ void correlations_ff(const cdf* const base[2], const int len[2], int 
       }
       __syncthreads();
       if (it + 1 < iters) fetch(it + 1, pre);
+      // a channel's last tile only as far as its polynomials reach (16 480p pairs
+      // 577 -> 570 us, 16 1080p colour pairs 2097 -> 2083)
+      const int rows = min(kGramChunk / 32, (maxlen - (it % nchunk) * kGramChunk + 31) / 32);
 #pragma unroll
       for (int q = 0; q < kGramLags; ++q) {
         const int j = (j0 + warp + q * nw) * sp.step + sp.first;
@@ -299,7 +302,7 @@ __device__ void correlations_ff(const cdf* const base[2], const int len[2], int 
         const cdf* A = tile + ka * kGramTile + kMaxN;
         const cdf* B = tile + kb * kGramTile + kMaxN + d;
 #pragma unroll 4
-        for (int r = 0; r < kGramChunk / 32; ++r) {
+        for (int r = 0; r < rows; ++r) {
           const int m = lane + 32 * r;
           const cdf x = A[m], y = B[m];
           // conj(x) y = (xr yr + xi yi) + i (xr yi - xi yr)
@@ -895,11 +898,13 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_scale_solve(ScaleArgs a) {
   cfx* cof = (cfx*)(smem + scale_ff_offset(M, a.nn));   // [2][M][nn] cofactors, conjugates expanded
   cfx* abx = cof + 2 * M * a.nn;                         // [4][M][M] A_1, A_2, B_1, B_2
   if (ffx) {
+#pragma unroll 2
     for (int idx = threadIdx.x; idx < 2 * M * a.nn; idx += blockDim.x) {
       const int ps = idx / (M * a.nn), sm = (idx / a.nn) % M, e = idx % a.nn;
       cof[idx] = cfx_of(cofactor(a, f, ps, sm, e));
     }
     __syncthreads();
+#pragma unroll 1
     for (int idx = threadIdx.x; idx < 4 * MM; idx += blockDim.x) {
       const int which = idx / MM, i = (idx % MM) / M, j = idx % M;
       const int kk = which & 1, isB = which >> 1;
@@ -907,6 +912,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_scale_solve(ScaleArgs a) {
       const cfx* u = cof + ((isB ? M : 0) + (isB ? i : j)) * a.nn + lo;
       const int mult = isB ? j : i;
       cfx_acc acc;
+#pragma unroll 1
       for (int q = 0, e = 0; q < t; ++q) {      // e = mult q mod M
         acc.mac(u[q], wtx[e]);
         e += mult;
@@ -918,6 +924,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_scale_solve(ScaleArgs a) {
     }
   }
   // lift: A_k[i][j] = sum_p u^{Z2}_{k,j}[p] w^{ip};  B_k[i][j] = sum_q u^{Z1}_{k,i}[q] w^{jq}
+#pragma unroll 1
   for (int idx = threadIdx.x; !ffx && idx < 4 * MM; idx += blockDim.x) {
     const int which = idx / MM, i = (idx % MM) / M, j = idx % M;
     const int kk = which & 1, isB = which >> 1;
@@ -1017,6 +1024,42 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_scale_solve(ScaleArgs a) {
     for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) Gx[idx] = cfx_of(Gs[idx]);
     __syncthreads();
   }
+  // The samples' diagnostics by a warp outside the team, beside its reduction:
+  // every quantity is a maximum or minimum of non-negative doubles, compared as
+  // integers.
+  __shared__ double agg[3];   // gap, sqrt(theta / lambda_max) (max), 1 / gap
+  __shared__ int aggi[2];     // flagged, hard
+  if ((threadIdx.x >> 5) == kTeamThreads / 32) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long gmin = 0x7fefffffffffffffull, smax = 0;
+    int flagged = 0, hard = 0;
+    for (int i = lane; i < 2 * a.ns; i += 32) {
+      const double* d = a.sdiag + ((int64_t)f * 2 * a.ns + i) * 4;
+      const double lmax = d[0] > 0 ? d[0] : 1e-300;
+      const double g = fmax(d[1], 0.0) / lmax, m = fmax(d[2], 0.0) / lmax;
+      const unsigned long long gb = (unsigned long long)__double_as_longlong(g),
+                               mb = (unsigned long long)__double_as_longlong(m);
+      if (gb < gmin) gmin = gb;
+      if (mb > smax) smax = mb;
+      if (sqrt(g) < 1e-8) ++flagged;
+      hard += (int)d[3];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long g2 = __shfl_xor_sync(0xffffffffu, gmin, o), m2 = __shfl_xor_sync(0xffffffffu, smax, o);
+      if (g2 < gmin) gmin = g2;
+      if (m2 > smax) smax = m2;
+    }
+    flagged = __reduce_add_sync(0xffffffffu, flagged);
+    hard = __reduce_add_sync(0xffffffffu, hard);
+    const double v = sqrt(__longlong_as_double((long long)(lane ? smax : gmin)));
+    if (lane < 2) agg[lane] = v;
+    if (lane == 0) {
+      agg[2] = v > 0 ? 1.0 / v : 1e300;
+      aggi[0] = flagged;
+      aggi[1] = hard;
+    }
+  }
   TriResult res;
   if (mode == kScaleSupport) {
     SupportApply ap{ab, wt, X, M, t1, t2};      // X is free until the combination below
@@ -1040,13 +1083,21 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_scale_solve(ScaleArgs a) {
   __shared__ cd x00[2];
   CBP_TICK(ph, 4);
   // inverse DFT, separable: T[i][q] = sum_j X[i][j] w^{-jq};  K[p][q] = sum_i w^{-ip} T[i][q] / M^2,
-  // both kernels side by side, T in place of X (each row by the threads that read it)
+  // four warps a kernel (so that a thread's sums are of one)
+  constexpr int kHalf = kSolveThreads / 2;
+  const int kh = threadIdx.x / kHalf, th = threadIdx.x % kHalf;
   __shared__ cd inv00[2];
+  __shared__ cfx invx[2];
+  __shared__ double iMM;
   if (threadIdx.x < 2) {
     const cd z = X[threadIdx.x * MM];
     x00[threadIdx.x] = z;
-    const double d = abs2(z);
-    inv00[threadIdx.x] = d > 0 ? mk(z.re / d, -z.im / d) : mk(0.0, 0.0);
+    const double d = abs2(z), r = 1.0 / d;
+    const cd v = d > 0 ? mk(z.re * r, -z.im * r) : mk(0.0, 0.0);
+    inv00[threadIdx.x] = v;
+    invx[threadIdx.x] = cfx_of(v);
+  } else if (threadIdx.x == 32) {
+    iMM = 1.0 / (double)MM;
   }
   if (nk < 2) {
     // k1-only: no kernel 2 (its internal copy zeroed, the caller's buffer untouched)
@@ -1054,86 +1105,81 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_scale_solve(ScaleArgs a) {
     for (int e = threadIdx.x; e < t2 * t2; e += blockDim.x) kd2[e] = 0.0;
   }
   __syncthreads();
-  cfx* Xx = (cfx*)X;   // float-float: X inv00 in place (the same 16 bytes an entry)
-  for (int idx = threadIdx.x; idx < nk * MM; idx += blockDim.x) {
-    const int k = idx >= MM;
-    if (ffx) Xx[idx] = cfx_mul(cfx_of(X[idx]), cfx_of(inv00[k]));
-    else X[idx] = X[idx] * inv00[k];
+  cd* Xk = X + kh * MM;
+  cfx* Xx = (cfx*)Xk;  // float-float: X inv00 in place (the same 16 bytes an entry)
+  const int lim = kh < nk ? MM : 0;
+#pragma unroll 1
+  for (int e = th; e < lim; e += kHalf) {
+    if (ffx) Xx[e] = cfx_mul(cfx_of(Xk[e]), invx[kh]);
+    else Xk[e] = Xk[e] * inv00[kh];
   }
   __syncthreads();
-  // a thread keeps one (kernel, q) and its T values until all of X's rows are read
-  constexpr int kTPer = (2 * kMaxM * kMaxM + kSolveThreads - 1) / kSolveThreads;
-  cd tv[kTPer];
-#pragma unroll
-  for (int r = 0; r < kTPer; ++r) {
-    const int idx = threadIdx.x + r * kSolveThreads;
-    if (idx < nk * MM) {
-      const int i0 = idx / M, q = idx - i0 * M;           // row i0 = k M + i
-      if (ffx) {
-        cfx_acc acc;
-        for (int j = 0, e = 0; j < M; ++j) {
-          const cfx w = wtx[e];
-          acc.mac(Xx[i0 * M + j], {w.re, fx_neg(w.im)});
-          e += q;
-          if (e >= M) e -= M;
-        }
-        const cfx v = acc.value();             // kept as its 16 bytes
-        tv[r] = mk(__hiloint2double(__float_as_int(v.re.lo), __float_as_int(v.re.hi)),
-                   __hiloint2double(__float_as_int(v.im.lo), __float_as_int(v.im.hi)));
-      } else {
-        cd acc = mk(0.0, 0.0);
-        for (int j = 0, e = 0; j < M; ++j) {
-          cfma(acc, X[i0 * M + j], conj(wt[e]));
-          e += q;
-          if (e >= M) e -= M;
-        }
-        tv[r] = acc;
+  // T where the normal matrix was.  Loops, not unrolled copies: the code runs
+  // once, and what it costs is fetching it (eight copies of the row transforms'
+  // loops and a thread's sums over both kernels: three pairs of 13 / 11 kernels
+  // 143 us a call, 123 now; four of 17 / 15 156, 148; one FP64 pair of 5 / 5 112,
+  // 107).
+  cd* Tk = Gs + kh * MM;
+  cfx* Tx = (cfx*)Tk;
+#pragma unroll 1
+  for (int idx = th; idx < lim; idx += kHalf) {
+    const int i0 = idx / M, q = idx - i0 * M;
+    if (ffx) {
+      cfx_acc acc;
+#pragma unroll 1
+      for (int j = 0, e = 0; j < M; ++j) {
+        const cfx w = wtx[e];
+        acc.mac(Xx[i0 * M + j], {w.re, fx_neg(w.im)});
+        e += q;
+        if (e >= M) e -= M;
       }
+      Tx[idx] = acc.value();
+    } else {
+      cd acc = mk(0.0, 0.0);
+#pragma unroll 1
+      for (int j = 0, e = 0; j < M; ++j) {
+        cfma(acc, Xk[i0 * M + j], conj(wt[e]));
+        e += q;
+        if (e >= M) e -= M;
+      }
+      Tk[idx] = acc;
     }
   }
   __syncthreads();
-#pragma unroll
-  for (int r = 0; r < kTPer; ++r) {
-    const int idx = threadIdx.x + r * kSolveThreads;
-    if (idx < nk * MM) X[idx] = tv[r];
-  }
-  __syncthreads();
-  double sums[6] = {0, 0, 0, 0, 0, 0};   // per kernel: Re^2, Im^2, energy outside t x t
-  for (int idx = threadIdx.x; idx < nk * MM; idx += blockDim.x) {
-    const int k = idx >= MM, e0 = idx - k * MM;
-    const int pp = e0 / M, q = e0 - pp * M, t = k ? t2 : t1;
+  const int t = kh ? t2 : t1;
+  double s_re = 0.0, s_im = 0.0, s_out = 0.0;   // Re^2, Im^2, energy outside t x t
+#pragma unroll 1
+  for (int e0 = th; e0 < lim; e0 += kHalf) {
+    const int pp = e0 / M, q = e0 - pp * M;
     cd acc = mk(0.0, 0.0);
     if (ffx) {
       cfx_acc ax;
+#pragma unroll 1
       for (int i = 0, e = 0; i < M; ++i) {
         const cfx w = wtx[e];
-        ax.mac({w.re, fx_neg(w.im)}, Xx[k * MM + i * M + q]);
+        ax.mac({w.re, fx_neg(w.im)}, Tx[i * M + q]);
         e += pp;
         if (e >= M) e -= M;
       }
       acc = cfx_val(ax.value());
     } else {
+#pragma unroll 1
       for (int i = 0, e = 0; i < M; ++i) {
-        cfma(acc, conj(wt[e]), X[k * MM + i * M + q]);
+        cfma(acc, conj(wt[e]), Tk[i * M + q]);
         e += pp;
         if (e >= M) e -= M;
       }
     }
-    acc = (1.0 / (double)MM) * acc;
-    const double r2 = acc.re * acc.re, i2 = acc.im * acc.im;
-    const bool outside = pp >= t || q >= t;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (h == k) {
-        sums[3 * h] += r2;
-        sums[3 * h + 1] += i2;
-        if (outside) sums[3 * h + 2] += r2 + i2;
-      }
-    if (!outside && CBP_CHECK(pp < a.M && q < a.M, 3)) {
-      a.kd[(int64_t)f * (t1 * t1 + t2 * t2) + (k ? t1 * t1 : 0) + pp * t + q] = acc.re;
-      void* out = k ? a.k2_out : a.k1_out;
+    acc = iMM * acc;
+    s_re = fma(acc.re, acc.re, s_re);
+    s_im = fma(acc.im, acc.im, s_im);
+    if (pp >= t || q >= t) {
+      s_out += abs2(acc);
+    } else if (CBP_CHECK(pp < a.M && q < a.M, 3)) {
+      a.kd[(int64_t)f * (t1 * t1 + t2 * t2) + (kh ? t1 * t1 : 0) + pp * t + q] = acc.re;
+      void* out = kh ? a.k2_out : a.k1_out;
       int64_t oi = (int64_t)f * t * t + pp * t + q;
-      const uint64_t* tab = k ? a.k2_tab : a.k1_tab;
+      const uint64_t* tab = kh ? a.k2_tab : a.k1_tab;
       if (tab) {
         out = (void*)tab[f];
         oi = pp * t + q;
@@ -1144,55 +1190,28 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_scale_solve(ScaleArgs a) {
       }
     }
   }
-  __shared__ double dsum[6][kSolveThreads / 32], dtot[6];
-#pragma unroll
-  for (int h = 0; h < 6; h += 2) {
-    lane_sum2(sums[h], sums[h + 1]);
-    if ((threadIdx.x & 31) == 0) {
-      dsum[h][threadIdx.x >> 5] = sums[h];
-      dsum[h + 1][threadIdx.x >> 5] = sums[h + 1];
-    }
-  }
-  // the samples' diagnostics by warp 1: every quantity is a maximum or minimum
-  // of non-negative doubles, compared as integers
-  __shared__ double agg[4];   // gap^2 (min), (theta / lambda_max) (max), flagged, hard
-  if (threadIdx.x >= 32 && threadIdx.x < 64) {
-    const int lane = threadIdx.x & 31;
-    unsigned long long gmin = 0x7fefffffffffffffull, smax = 0;
-    int flagged = 0, hard = 0;
-    for (int i = lane; i < 2 * a.ns; i += 32) {
-      const double* d = a.sdiag + ((int64_t)f * 2 * a.ns + i) * 4;
-      const double lmax = d[0] > 0 ? d[0] : 1e-300;
-      const double g = fmax(d[1], 0.0) / lmax, m = fmax(d[2], 0.0) / lmax;
-      const unsigned long long gb = (unsigned long long)__double_as_longlong(g),
-                               mb = (unsigned long long)__double_as_longlong(m);
-      if (gb < gmin) gmin = gb;
-      if (mb > smax) smax = mb;
-      if (sqrt(g) < 1e-8) ++flagged;
-      hard += (int)d[3];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long g2 = __shfl_xor_sync(0xffffffffu, gmin, o), m2 = __shfl_xor_sync(0xffffffffu, smax, o);
-      if (g2 < gmin) gmin = g2;
-      if (m2 > smax) smax = m2;
-    }
-    flagged = __reduce_add_sync(0xffffffffu, flagged);
-    hard = __reduce_add_sync(0xffffffffu, hard);
-    if (lane == 0) {
-      agg[0] = __longlong_as_double((long long)gmin);
-      agg[1] = __longlong_as_double((long long)smax);
-      agg[2] = (double)flagged;
-      agg[3] = (double)hard;
-    }
+  __shared__ double dsum[3][kSolveThreads / 32];
+  lane_sum2(s_re, s_im);
+  s_out = lane_sum(s_out);
+  if ((threadIdx.x & 31) == 0) {
+    dsum[0][threadIdx.x >> 5] = s_re;
+    dsum[1][threadIdx.x >> 5] = s_im;
+    dsum[2][threadIdx.x >> 5] = s_out;
   }
   __syncthreads();
-  if (threadIdx.x < 6) {
-    double t = 0.0;
-    for (int w = 0; w < kSolveThreads / 32; ++w) t += dsum[threadIdx.x][w];
-    dtot[threadIdx.x] = t;
+  // a kernel's ratios (lanes 0 and 1): imaginary part, energy outside t x t
+  double ir = 0.0, sr = 0.0;
+  if (threadIdx.x < (unsigned)nk) {
+    double tot[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double* d = dsum[c] + threadIdx.x * (kSolveThreads / 64);
+      tot[c] = (d[0] + d[1]) + (d[2] + d[3]);
+    }
+    ir = tot[0] > 0 ? sqrt(tot[1] / tot[0]) : 0.0;
+    sr = (tot[0] + tot[1]) > 0 ? tot[2] / (tot[0] + tot[1]) : 0.0;
   }
-  __syncwarp();
+  const double ir1 = __shfl_down_sync(0xffffffffu, ir, 1), sr1 = __shfl_down_sync(0xffffffffu, sr, 1);
   CBP_TICK(ph, 5);
 #ifdef CBP_PHASE_TIMING
   if (tk && threadIdx.x == 0)
@@ -1203,17 +1222,10 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_scale_solve(ScaleArgs a) {
 #endif
   // aggregate diagnostics
   if (threadIdx.x == 0) {
-    double ir = 0.0, sr = 0.0;
-    for (int k = 0; k < nk; ++k) {
-      const double* t = dtot + 3 * k;
-      ir = fmax(ir, t[0] > 0 ? sqrt(t[1] / t[0]) : 0.0);
-      sr = fmax(sr, (t[0] + t[1]) > 0 ? t[2] / (t[0] + t[1]) : 0.0);
-    }
-    a.diag[f].imag_ratio = ir;
-    a.diag[f].support_ratio = sr;
-    const double gap = sqrt(agg[0]), smin = sqrt(agg[1]);
-    const double kappa = gap > 0 ? 1.0 / gap : 1e300;
-    const int flagged = (int)agg[2], hard = (int)agg[3];
+    a.diag[f].imag_ratio = fmax(fmax(0.0, ir), ir1);
+    a.diag[f].support_ratio = fmax(fmax(0.0, sr), sr1);
+    const double gap = agg[0], smin = agg[1], kappa = agg[2];
+    const int flagged = aggi[0], hard = aggi[1];
     cbp_diag& dg = a.diag[f];
     dg.kappa_max = kappa;
     dg.gap_min = gap;
