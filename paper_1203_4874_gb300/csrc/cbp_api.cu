@@ -627,6 +627,21 @@ cbp_status call_path(cbp_ctx* ctx, const cbp_frames* b1, const cbp_frames* b2,
   if (host_io && !overlap &&
       cudaStreamWaitEvent(c->io_st, c->chunk_ev[c->kMaxChunks], 0) != cudaSuccess)
     return CBP_ERR_CUDA;
+  // A copy to pageable memory returns only when its stream has got there: behind
+  // its own chunk it would hold the next one back until then, so such diagnostics
+  // come back once every chunk is launched (30 480p pairs 1.68 -> 1.09 ms).
+  // Copies to pinned memory go behind their chunk.
+  bool late = false;
+  if (diag) {
+    cudaPointerAttributes at = {};
+    const bool known = cudaPointerGetAttributes(&at, diag) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    late = !known || at.type == cudaMemoryTypeUnregistered;
+  }
+  auto diag_back = [&](int i, cudaStream_t cs) {
+    return cudaMemcpyAsync(diag + start[i], c->ws + off[i] + cp[i].off_diag, (size_t)cp[i].n * sizeof(cbp_diag),
+                           cudaMemcpyDeviceToHost, cs) == cudaSuccess;
+  };
   for (int i = 0; i < nch; ++i) {
     cudaStream_t cs = c->chunk_st[i % Ctx::kChunkStreams];
     if (!overlap && cudaStreamWaitEvent(cs, c->chunk_ev[c->kMaxChunks], 0) != cudaSuccess)
@@ -673,18 +688,14 @@ cbp_status call_path(cbp_ctx* ctx, const cbp_frames* b1, const cbp_frames* b2,
                       host_io ? nullptr : c->solve_st[i % Ctx::kChunkStreams], c->fork_ev[i],
                       c->join_ev[i], tw_ready);
     if (s != CBP_OK) return s;
+    if (diag && !late && !diag_back(i, cs)) return CBP_ERR_CUDA;
     if (cudaEventRecord(c->chunk_ev[i], cs) != cudaSuccess ||
         cudaStreamWaitEvent(st, c->chunk_ev[i], 0) != cudaSuccess)
       return CBP_ERR_CUDA;
   }
-  // The diagnostics come back once every chunk is launched: a copy to pageable
-  // memory returns only when its stream has got there, and issued behind its own
-  // chunk it held the next one back until then (30 480p pairs 1.68 -> 1.09 ms).
-  for (int i = 0; diag && i < nch; ++i) {
+  for (int i = 0; late && i < nch; ++i) {
     cudaStream_t cs = c->chunk_st[i % Ctx::kChunkStreams];
-    if (cudaMemcpyAsync(diag + start[i], c->ws + off[i] + cp[i].off_diag, (size_t)cp[i].n * sizeof(cbp_diag),
-                        cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
-        cudaEventRecord(c->chunk_ev[i], cs) != cudaSuccess ||
+    if (!diag_back(i, cs) || cudaEventRecord(c->chunk_ev[i], cs) != cudaSuccess ||
         cudaStreamWaitEvent(st, c->chunk_ev[i], 0) != cudaSuccess)
       return CBP_ERR_CUDA;
   }

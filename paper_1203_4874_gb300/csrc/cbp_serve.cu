@@ -34,9 +34,9 @@ namespace cbp {
 namespace serve {
 
 constexpr int kSlots = 8;          // concurrent batches, one stream each (as many as the process's
-                                   // hardware queues let run: with four of them 2.31 ms for 16
-                                   // cameras' requests, with eight 1.60, against 2.53 and 2.5 with
-                                   // four slots)
+                                   // hardware queues let run: with four of them 2.31 ms (1.94 with
+                                   // today's row passes) for 16 cameras' requests, with eight 1.60,
+                                   // against 2.53 and 2.5 with four slots)
 constexpr int kMaxBatch = 16;      // requests per batch
 // Captured batches kept, whatever the streams.  (A cache of eight per stream
 // captured a batch again, ~0.35 ms of the scheduler's time, whenever the stream
