@@ -1953,7 +1953,7 @@ void run_row_ifft(const Plan& p, char* ws, void* latent, int out_f64, cudaStream
 // A double sincospi is some 60 double instructions, so what counts is that the
 // few thousand entries spread over all SMs: as four to six launches, two of them
 // looping over the stages in a few blocks, they took 30-46 us before a small call's
-// first real kernel; this takes about 5.
+// first real kernel; this takes 7.
 struct TableArgs {
   FftPlan h, r;
   int Ph, Pw;
