@@ -123,6 +123,11 @@ struct Roots {
 };
 const Roots& make_roots(int M);
 
+// Dynamic shared memory a block of `kernel` can have on the current device: the
+// device's limit less the kernel's own static arrays (kept per device and
+// kernel; 0 where it cannot be found out).
+size_t smem_room(const void* kernel);
+
 // ---- planning (cbp_plan.cpp) ----
 int next_7_smooth(int n);
 uint32_t magic_div(int d);   // ceil(2^32 / d): __umulhi(x, .) = x / d for x d < 2^32; 0 for d <= 1

@@ -2,7 +2,9 @@
 // the per-call device workspace.
 #include <algorithm>
 #include <cmath>
+#include <map>
 #include <mutex>
+#include <utility>
 #include "cbp_common.cuh"
 #include "cbp_internal.h"
 
@@ -43,6 +45,23 @@ const Roots& make_roots(int M) {
   const int m = M < 1 ? 1 : M > kMaxM ? kMaxM : M;
   std::call_once(once[m], [m] { table[m] = compute_roots(m); });
   return table[m];
+}
+
+size_t smem_room(const void* kernel) {
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, size_t> room;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> g(mu);
+  const auto key = std::make_pair(dev, kernel);
+  const auto it = room.find(key);
+  if (it != room.end()) return it->second;
+  int limit = 0;
+  cudaFuncAttributes at = {};
+  if (cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaFuncGetAttributes(&at, kernel) != cudaSuccess || at.sharedSizeBytes >= (size_t)limit)
+    return 0;
+  return room[key] = (size_t)limit - at.sharedSizeBytes;
 }
 
 uint32_t magic_div(int d) {

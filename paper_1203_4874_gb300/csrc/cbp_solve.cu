@@ -1723,12 +1723,11 @@ void launch_scale_solve(const Plan& p, char* ws, void* k1_out, void* k2_out, int
   a.rho = p.learned ? (const double*)(ws + p.off_rho) : nullptr;
   a.mode = p.scale_mode;
   a.w = make_roots(p.M);
-  // the mixed path's float-float stage where its shared memory fits
+  // the mixed path's float-float stage where its shared memory fits beside the
+  // kernel's static arrays (M = 28 with t1 + t2 = 42 or 43, M = 29 with 27 and
+  // M = 30 with 11 or 12 fit the device's limit only without them)
   const size_t ff_end = scale_ff_offset(p.M, p.nn) + scale_ff_bytes(p.M, p.nn);
-  int dev = 0, smem_max = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  a.ffx = p.mixed && p.scale_mode != kScaleSupport && ff_end <= (size_t)smem_max;
+  a.ffx = p.mixed && p.scale_mode != kScaleSupport && ff_end <= smem_room((const void*)k_scale_solve);
   const size_t sm = a.ffx ? ff_end : scale_solve_smem(p.M, p.nn);
   cudaFuncSetAttribute(k_scale_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   k_scale_solve<<<p.n, kSolveThreads, sm, st>>>(a);
