@@ -627,6 +627,16 @@ __global__ void __launch_bounds__(kSolveThreads) k_sample_gram(SampleArgs a) {
 // 6.48), takes twice as long for one, and on the FP64 path, where the double
 // units bound either form, loses throughout (40 pairs of 25 / 20 kernels, 520
 // samples a chunk: 5.19 ms against 4.44).
+//
+// Mixed path, real samples: up to kFloatFloatN unknowns T and what follows it in
+// float-float, above in double.  Float-float leaves ~n 2^-48 lambda_max / gap in
+// x before the refinement step, which contracts by as much, and the gap between
+// the two smallest eigenvalues closes with the width: to 1e-10 lambda_max at 50
+// unknowns with noise of 1e-3, to 1e-14 without.  Largest error of the kernels
+// against 64-bit singular vectors over 12 noise-free pairs, float-float /
+// double: 20 and 20 1.1e-1 / 7.8e-5, 24 and 20 8.4e-3 / 2.1e-5, 25 and 25 5.7e-4
+// / 8.6e-5.  At 39 the vectors of the same samples agree.
+constexpr int kFloatFloatN = 39;
 __global__ void __launch_bounds__(kTeamThreads, 3) k_sample_solve(SampleArgs a, int nreal) {
   extern __shared__ __align__(16) char smem[];
 #ifdef CBP_SCHED_TRACE
@@ -694,7 +704,7 @@ __global__ void __launch_bounds__(kTeamThreads, 3) k_sample_solve(SampleArgs a, 
       ap.ys = reinterpret_cast<float2*>(smem + per);
       ap.ys_cap = (int)((dsm - per) / sizeof(float2));
     }
-    res = tri_smallest_team<double>(W, G, n, far, 1, gap, ap, tk, false, nullptr, a.mixed != 0);
+    res = tri_smallest_team<double>(W, G, n, far, 1, gap, ap, tk, false, nullptr, a.mixed && n <= kFloatFloatN);
   } else {
     res = tri_smallest_team<cd>(W, G, n, far, 1, gap, ap, tk, a.mixed != 0);
   }
