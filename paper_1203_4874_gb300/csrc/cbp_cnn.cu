@@ -463,7 +463,7 @@ void run_conv_tc(const bf16* x, const uint8_t* img, const float* prm, TO* y, int
   const Layer L = cnn_layer(li);
   const int npos = L.hout * L.hout;
   auto kfn = k_conv_tc<CIN, KS, N, TO>;
-  cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
+  allow_smem((const void*)kfn);
   kfn<<<dim3((npos + kTcM - 1) / kTcM, n), kTcThreads, C::kSmem, st>>>(x, img + tc_img_offset(li), prm, y, L, err);
 }
 
@@ -891,7 +891,7 @@ void run_bwd_w_tc(const float* dy, const bf16* x, float* part, float* grad, int 
   const Layer L = cnn_layer(li);
   const WChunks wc = tc_wchunks((int64_t)n * L.hout * L.hout, W::kPos);
   auto kfn = k_conv_bwd_w_tc<CIN, KS, N>;
-  cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, W::kSmem);
+  allow_smem((const void*)kfn);
   kfn<<<wc.count, W::kThreads, W::kSmem, st>>>(dy, x, part, L, n, wc.chunk, err);
   k_conv_bwd_w_sum<CIN, KS, N><<<((W::kW + 1) * L.cout + kWSumOut - 1) / kWSumOut, kWSumOut * kWSumRuns, 0, st>>>(
       part, grad, L, wc.count);
@@ -903,7 +903,7 @@ void run_bwd_data_tc(const float* dy, const uint8_t* wt, const bf16* xact, float
   using C = ConvTcT<CIN, KS, COUT>;
   const Layer L = cnn_layer(li);
   auto kfn = k_conv_bwd_data_tc<CIN, KS, COUT>;
-  cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
+  allow_smem((const void*)kfn);
   kfn<<<dim3((L.hin * L.hin + kTcM - 1) / kTcM, n), kTcThreads, C::kSmem, st>>>(
       dy, wt + tct_img_offset(li), xact, dx, L, err);
 }

@@ -426,7 +426,7 @@ void run_fused(const Plan& p, char* ws, cudaStream_t st) {
       p.t2, p.Pw, p.Pw2, p.Pw2p);
   const size_t sm = FcSmem<N1, N2>::kBytes;
   auto kern = k_col_deconv_fused<N1, N2, RESID>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)kern);
   cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   kern<<<dim3(fused_strips(p), p.n * p.C), kFcThreads, sm, st>>>(a);
 }

@@ -1752,8 +1752,7 @@ void run_row_pass_t(const Plan& p, const RowPassArgs& a, int gx, int gz, char* w
                     cudaStream_t st) {
   const RowPassSmem L = row_pass_layout(a.pl.n, a.pl.ntw, a.wl, a.nbr, a.rw, sizeof(cpx<T>),
                                         sizeof(In), FOLD, FFT);
-  cudaFuncSetAttribute(k_row_pass<T, In, FOLD, FFT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)L.total);
+  allow_smem((const void*)k_row_pass<T, In, FOLD, FFT>);
   k_row_pass<T, In, FOLD, FFT><<<dim3(gx, p.n * p.C, gz), kRowPassThreads, L.total, st>>>(
       a, (const cpx<T>*)(ws + p.off_tw_w), (const cpx<T>*)(ws + p.off_stw_r));
 }
@@ -1821,7 +1820,7 @@ void run_row_pass(const Plan& p, const FrameDesc& b1, const FrameDesc& b2, char*
       const RowIrSmem L = row_ir_layout(a.rw);
       auto kern = fold ? k_row_pass_ir<36, 27, true> : k_row_pass_ir<36, 27, false>;
       const int gi = fold ? gx : row_blocks(hmax, planes, kIrRows);
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+      allow_smem((const void*)kern);
       cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
       kern<<<dim3(gi, p.n * p.C, gz), kIrThreads, L.total, st>>>(a, (const cf*)(ws + p.off_tw_w));
       return;
@@ -1855,8 +1854,7 @@ void run_col_deconv(const Plan& p, char* ws, cudaStream_t st) {
   constexpr int CW = sizeof(T) == 4 ? 4 : 2;
   dim3 g((p.Pw2 + CW - 1) / CW, p.n * p.C);
   const size_t sm = sizeof(cpx<T>) * 3 * (size_t)CW * p.Ph;
-  cudaFuncSetAttribute(k_col_deconv<T, CW, RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sm);
+  allow_smem((const void*)k_col_deconv<T, CW, RESID>);
   k_col_deconv<T, CW, RESID><<<g, kColThreads, sm, st>>>(a);
 }
 
@@ -1931,14 +1929,14 @@ void run_row_ifft(const Plan& p, char* ws, void* latent, int out_f64, cudaStream
         ((uintptr_t)latent & 7) == 0 && p.off_tw2r) {
       g.x = row_blocks(p.H, p.n * p.C, kIrRows);
       const size_t smi = irow_ir_layout(p.Pw2p).total;
-      cudaFuncSetAttribute(k_row_ifft_ir<36, 27>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smi);
+      allow_smem((const void*)k_row_ifft_ir<36, 27>);
       cudaFuncSetAttribute(k_row_ifft_ir<36, 27>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
       k_row_ifft_ir<36, 27><<<g, kIrThreads, smi, st>>>(a, (const cf*)(ws + p.off_tw_w));
       return;
     }
   }
   const size_t sm = irow_layout(plw.n, plw.ntw, p.Pw2p, a.nbr, sizeof(cpx<T>)).total;
-  cudaFuncSetAttribute(k_row_ifft<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)k_row_ifft<T>);
   k_row_ifft<T><<<g, kRowPassThreads, sm, st>>>(a, (const cpx<T>*)(ws + p.off_tw_w),
                                                 (const cpx<T>*)(ws + p.off_stw_r));
 }

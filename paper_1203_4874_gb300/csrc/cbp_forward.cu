@@ -203,7 +203,7 @@ void launch_blur_rows(const float* lat, int n, int c, int h, int w, const double
   constexpr int tr = kBlurWarps * R;
   dim3 g((wb + kBlurTileC - 1) / kBlurTileC, (hb + tr - 1) / tr, n * c);
   constexpr size_t sm = sizeof(float2) * (size_t)T * ((T + 1) & ~1) + sizeof(float) * (size_t)(tr + T - 1) * kBlurPitch;
-  cudaFuncSetAttribute(k_forward_blur_rb<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)k_forward_blur_rb<T, R>);
   k_forward_blur_rb<T, R><<<g, 32 * kBlurWarps, sm, st>>>(lat, c, h, w, kern, sigma, seed, out);
 }
 template <int T>
@@ -412,7 +412,7 @@ void launch_forward_blur(const void* latent, int n, int c, int h, int w, int f64
   const int th = kTile + t - 1;
   const size_t sm = ((t * t * sizeof(double) + 15) & ~size_t(15)) + (size_t)th * th * (f64 ? 8 : 4);
   if (f64) {
-    cudaFuncSetAttribute(k_forward_blur<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem((const void*)k_forward_blur<double>);
     k_forward_blur<double><<<g, kTile * 8, sm, st>>>((const double*)latent, c, h, w, kernel, t,
                                                       sigma, seed, (double*)out);
   } else if (t <= 17) {
@@ -428,7 +428,7 @@ void launch_forward_blur(const void* latent, int n, int c, int h, int w, int f64
 #undef CBP_BLUR_CASE
     }
   } else {
-    cudaFuncSetAttribute(k_forward_blur<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem((const void*)k_forward_blur<float>);
     k_forward_blur<float><<<g, kTile * 8, sm, st>>>((const float*)latent, c, h, w, kernel, t,
                                                      sigma, seed, (float*)out);
   }

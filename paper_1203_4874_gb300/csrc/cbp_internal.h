@@ -123,10 +123,13 @@ struct Roots {
 };
 const Roots& make_roots(int M);
 
-// Dynamic shared memory a block of `kernel` can have on the current device: the
-// device's limit less the kernel's own static arrays (kept per device and
-// kernel; 0 where it cannot be found out).
-size_t smem_room(const void* kernel);
+// Lets `kernel` have all the dynamic shared memory a block can on the current
+// device beside the kernel's own static arrays, and returns that size (0 where it
+// cannot be found out).  The limit is state of the process: with each call's own
+// size in it, a call or a captured batch of another thread could lower it between
+// the setting and the launch, which then fails.  Set on every call all the same: it
+// goes with a device reset.
+size_t allow_smem(const void* kernel);
 
 // ---- planning (cbp_plan.cpp) ----
 int next_7_smooth(int n);

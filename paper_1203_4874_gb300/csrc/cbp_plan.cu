@@ -47,21 +47,26 @@ const Roots& make_roots(int M) {
   return table[m];
 }
 
-size_t smem_room(const void* kernel) {
+size_t allow_smem(const void* kernel) {
   static std::mutex mu;
-  static std::map<std::pair<int, const void*>, size_t> room;
+  static std::map<std::pair<int, const void*>, size_t> room;   // per device and kernel
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  std::lock_guard<std::mutex> g(mu);
-  const auto key = std::make_pair(dev, kernel);
-  const auto it = room.find(key);
-  if (it != room.end()) return it->second;
-  int limit = 0;
-  cudaFuncAttributes at = {};
-  if (cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-      cudaFuncGetAttributes(&at, kernel) != cudaSuccess || at.sharedSizeBytes >= (size_t)limit)
-    return 0;
-  return room[key] = (size_t)limit - at.sharedSizeBytes;
+  size_t bytes = 0;
+  {
+    std::lock_guard<std::mutex> g(mu);
+    size_t& r = room[std::make_pair(dev, kernel)];
+    if (r == 0) {
+      int limit = 0;
+      cudaFuncAttributes at = {};
+      if (cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+          cudaFuncGetAttributes(&at, kernel) != cudaSuccess || at.sharedSizeBytes >= (size_t)limit)
+        return 0;
+      r = (size_t)limit - at.sharedSizeBytes;
+    }
+    bytes = r;
+  }
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess ? bytes : 0;
 }
 
 uint32_t magic_div(int d) {

@@ -1702,7 +1702,7 @@ void launch_sample_solve(const Plan& p, char* ws, cudaStream_t st) {
     const size_t need = per + sizeof(float2) * (size_t)std::max(lz1, lz2);
     if (need <= (110u << 10)) sm = need;
   }
-  cudaFuncSetAttribute(k_sample_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)k_sample_solve);
   k_sample_solve<<<nreal + ncomplex, kTeamThreads, sm, st>>>(a, nreal);
 }
 
@@ -1737,9 +1737,8 @@ void launch_scale_solve(const Plan& p, char* ws, void* k1_out, void* k2_out, int
   // kernel's static arrays (M = 28 with t1 + t2 = 42 or 43, M = 29 with 27 and
   // M = 30 with 11 or 12 fit the device's limit only without them)
   const size_t ff_end = scale_ff_offset(p.M, p.nn) + scale_ff_bytes(p.M, p.nn);
-  a.ffx = p.mixed && p.scale_mode != kScaleSupport && ff_end <= smem_room((const void*)k_scale_solve);
+  a.ffx = p.mixed && p.scale_mode != kScaleSupport && ff_end <= allow_smem((const void*)k_scale_solve);
   const size_t sm = a.ffx ? ff_end : scale_solve_smem(p.M, p.nn);
-  cudaFuncSetAttribute(k_scale_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   k_scale_solve<<<p.n, kSolveThreads, sm, st>>>(a);
 }
 
@@ -1791,7 +1790,7 @@ void launch_size_scan(const SizePlan& sp, const FrameDesc& b1, const FrameDesc& 
   constexpr int kLagWarps = kSolveThreads / 32;
   k_size_lags<<<dim3((2 * (a.ta + a.tb) - 1 + kLagWarps - 1) / kLagWarps, 2, sp.n), kSolveThreads, 0, st>>>(a);
   const size_t sm = size_scan_smem();
-  cudaFuncSetAttribute(k_size_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)k_size_scan);
   k_size_scan<<<dim3(sp.ncand, 2, sp.n), kSolveThreads, sm, st>>>(a);
   k_size_pick<<<(sp.n + 127) / 128, 128, 0, st>>>(a.ratio, sp.n, sp.ncand, sp.t_min, sp.d, sp.tol,
                                                  (int*)(ws + sp.off_t), (double*)(ws + sp.off_rmax));
@@ -1819,7 +1818,7 @@ void launch_coprime_round(const double* ka, const double* kb, int n, int ta, int
   a.pass = pass;
   a.w = make_roots(M);
   const size_t sm = coprime_test_smem();
-  cudaFuncSetAttribute(k_coprime_test, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)k_coprime_test);
   k_coprime_test<<<dim3(a.ns, 2, n), kSolveThreads, sm, st>>>(a);
   k_coprime_pick<<<(n + 127) / 128, 128, 0, st>>>(n, a.ns, pass, active, attempt, max_attempts, any);
 }
