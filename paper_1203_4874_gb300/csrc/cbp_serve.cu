@@ -33,15 +33,15 @@
 namespace cbp {
 namespace serve {
 
-constexpr int kSlots = 8;          // concurrent batches, one stream each (as many as the process's
-                                   // hardware queues let run: with four of them 2.31 ms (1.94 with
-                                   // today's row passes) for 16 cameras' requests, with eight 1.60,
-                                   // against 2.53 and 2.5 with four slots)
+constexpr int kSlots = 8;          // concurrent batches, one stream each (16 cameras' requests:
+                                   // 2.31 ms, with four streams 2.53)
 constexpr int kMaxBatch = 16;      // requests per batch
 // Captured batches kept, whatever the streams.  (A cache of eight per stream
 // captured a batch again, ~0.35 ms of the scheduler's time, whenever the stream
 // that was free had not run it before: with sixteen cameras, on every pass.)
-constexpr int kCache = 64;
+// A workspace each, held until another takes its place: as many as the cache per
+// stream held on four streams.
+constexpr int kCache = 32;
 constexpr int kTables = 5;         // b1, b2, k1, k2, latent addresses
 using Clock = std::chrono::steady_clock;
 

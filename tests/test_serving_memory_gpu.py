@@ -1,0 +1,69 @@
+"""Device memory the serving engine holds, as the allocator counts it (the
+process's default pool, which nothing else here allocates from)."""
+import ctypes
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+USED_NOW, USED_HIGH = 7, 8          # cudaMemPoolAttrUsedMemCurrent, -High
+
+
+class Pool:
+    """The default memory pool of device 0."""
+
+    def __init__(self):
+        self.rt = ctypes.CDLL("libcudart.so.13")
+        self.h = ctypes.c_void_p()
+        assert self.rt.cudaDeviceGetDefaultMemPool(ctypes.byref(self.h), 0) == 0
+
+    def used(self, attr=USED_NOW):
+        v = ctypes.c_uint64()
+        assert self.rt.cudaMemPoolGetAttribute(self.h, attr, ctypes.byref(v)) == 0
+        return v.value
+
+    def reset_high(self):
+        assert self.rt.cudaMemPoolSetAttribute(self.h, USED_HIGH, ctypes.byref(ctypes.c_uint64(0))) == 0
+
+
+@pytest.fixture
+def pool(built_lib):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.synchronize()
+    return Pool()
+
+
+def request(h, w, t1=7, t2=8, c=1):
+    from paper_1203_4874_gb300 import cbp
+    b1, b2 = (torch.rand((1, c, h + t - 1, w + t - 1), device="cuda") for t in (t1, t2))
+    out = (torch.empty((1, t1, t1), device="cuda"), torch.empty((1, t2, t2), device="cuda"),
+           torch.empty((1, c, h, w), device="cuda"))
+    return b1, b2, cbp.params(t1, t2, path="mixed", eps=1e-4), out
+
+
+def submit(ctx, r):
+    from paper_1203_4874_gb300 import cbp
+    return cbp.cbp_stream_submit(ctx, *r[:3], *r[3])
+
+
+def wait(ctx, t):
+    from paper_1203_4874_gb300 import cbp
+    s, _ = cbp.cbp_stream_poll(ctx, t, -1)
+    return s
+
+
+def test_kept_batches_are_bounded(pool):
+    """48 request shapes one after the other: 32 workspaces stay."""
+    from paper_1203_4874_gb300 import cbp
+    ctx = cbp.cbp_create(0)
+    before, one = pool.used(), 0
+    for i in range(48):
+        assert wait(ctx, submit(ctx, request(120 + 2 * i, 160))) >= 0
+        one = max(one, cbp.cbp_workspace_size(*request(120 + 2 * i, 160)[:3]) + (1 << 12))
+    held = pool.used() - before
+    cbp.cbp_destroy(ctx)
+    assert held <= 32 * one
+    torch.cuda.synchronize()
+    assert pool.used() == before
