@@ -106,7 +106,6 @@ struct Entry {
   uint64_t* tab = nullptr;    // device [kTables][B]
   cudaGraphExec_t exec = nullptr;
   uint64_t last_use = 0;
-  cudaStream_t st = nullptr;  // the stream its memory was allocated on
   bool busy = false;          // its batch is on the GPU
 };
 
@@ -154,35 +153,37 @@ struct ServeState {
   }
 
   // An idle entry: its last batch's completion has been seen on the host, so
-  // the order of streams does not matter.
-  void free_entry(Entry* e) {
+  // any stream may free it.  `st` is the idle one that allocates next, or that the
+  // memory came from just now: on a stream with a batch on it the memory would stay
+  // in use until that batch ends, although its bytes are released here.
+  void free_entry(Entry* e, cudaStream_t st) {
     if (e->exec) cudaGraphExecDestroy(e->exec);
-    if (e->mem) cudaFreeAsync(e->mem, e->st);
+    if (e->mem) cudaFreeAsync(e->mem, st);
     ctx->release(e->bytes);
     delete e;
   }
 
-  // Free the idle cached batch used least recently; false if none is idle.
-  bool evict_one() {
+  // Free the idle cached batch used least recently on `st`; false if none is idle.
+  bool evict_one(cudaStream_t st) {
     auto it = cache.end();
     for (auto i = cache.begin(); i != cache.end(); ++i)
       if (!(*i)->busy && (it == cache.end() || (*i)->last_use < (*it)->last_use)) it = i;
     if (it == cache.end()) return false;
     Entry* e = *it;
     cache.erase(it);
-    free_entry(e);
+    free_entry(e, st);
     return true;
   }
 
   // Free idle cached batches, least recently used first, until `bytes` more
   // would fit the budget (or nothing idle is left).
-  void evict_for(size_t bytes) {
+  void evict_for(size_t bytes, cudaStream_t st) {
     for (;;) {
       {
         std::lock_guard<std::mutex> g(ctx->mem_mu);
         if (ctx->used + bytes <= ctx->budget) return;
       }
-      if (!evict_one()) return;
+      if (!evict_one(st)) return;
     }
   }
 
@@ -201,7 +202,7 @@ struct ServeState {
     }
     const size_t bytes = align256(p.total) + align256((size_t)kTables * B * sizeof(uint64_t));
     if (!ctx->reserve(bytes)) {
-      evict_for(bytes);
+      evict_for(bytes, s.st);
       if (!ctx->reserve(bytes)) return nullptr;
     }
     Entry* e = new Entry();
@@ -209,7 +210,6 @@ struct ServeState {
     e->B = B;
     e->plan = p;
     e->bytes = bytes;
-    e->st = s.st;
     if (cudaMallocAsync((void**)&e->mem, bytes, s.st) != cudaSuccess) {
       cudaGetLastError();
       e->mem = nullptr;
@@ -241,11 +241,11 @@ struct ServeState {
     if (rs != CBP_OK) {
       cudaGetLastError();
       e->exec = nullptr;
-      free_entry(e);
+      free_entry(e, s.st);
       *st = rs;
       return nullptr;
     }
-    while ((int)cache.size() >= kCache && evict_one()) {
+    while ((int)cache.size() >= kCache && evict_one(s.st)) {
     }
     cache.push_back(e);
     return e;
@@ -402,7 +402,7 @@ struct ServeState {
         else wake.wait(lk, [&] { return stop || !pending.empty(); });
       }
     }
-    for (Entry* e : cache) free_entry(e);
+    for (Entry* e : cache) free_entry(e, slots[0].st);
     cache.clear();
     for (Slot& s : slots) {
       if (s.st) cudaStreamSynchronize(s.st);

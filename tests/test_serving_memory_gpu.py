@@ -7,7 +7,7 @@ import torch
 
 pytestmark = pytest.mark.gpu
 
-USED_NOW, USED_HIGH = 7, 8          # cudaMemPoolAttrUsedMemCurrent, -High
+RESERVED_NOW, RESERVED_HIGH, USED_NOW = 5, 6, 7      # cudaMemPoolAttrReservedMemCurrent, -High, UsedMemCurrent
 
 
 class Pool:
@@ -24,7 +24,7 @@ class Pool:
         return v.value
 
     def reset_high(self):
-        assert self.rt.cudaMemPoolSetAttribute(self.h, USED_HIGH, ctypes.byref(ctypes.c_uint64(0))) == 0
+        assert self.rt.cudaMemPoolSetAttribute(self.h, RESERVED_HIGH, ctypes.byref(ctypes.c_uint64(0))) == 0
 
 
 @pytest.fixture
@@ -67,3 +67,27 @@ def test_kept_batches_are_bounded(pool):
     assert held <= 32 * one
     torch.cuda.synchronize()
     assert pool.used() == before
+
+
+def test_room_for_a_new_shape_while_another_batch_runs(pool):
+    """A kept batch gives its workspace to a new shape while the stream it was
+    captured on runs something else: the pool takes no more memory from the device."""
+    from paper_1203_4874_gb300 import cbp
+    kept, long, new = request(720, 1280), request(480, 640, 25, 24), request(700, 1270)
+    sizes = [cbp.cbp_workspace_size(*r[:3]) for r in (kept, long, new)]
+    assert sizes[2] <= sizes[0]
+    for _ in range(3):
+        base = pool.used()                       # other contexts' workspaces
+        ctx = cbp.cbp_create(0, sizes[0] + sizes[1] + (1 << 16))     # tables and alignment
+        for r in (long, kept):                   # both captured on the first stream
+            assert wait(ctx, submit(ctx, r)) >= 0
+        torch.cuda.synchronize()
+        before = pool.used(RESERVED_NOW)
+        pool.reset_high()
+        tickets = [submit(ctx, long), submit(ctx, new)]
+        assert all(wait(ctx, t) >= 0 for t in tickets)
+        high = pool.used(RESERVED_HIGH)
+        cbp.cbp_destroy(ctx)
+        torch.cuda.synchronize()
+        assert high <= before
+        assert pool.used() == base
