@@ -9,9 +9,9 @@
 //   - groups pending requests by shape bucket (everything but the data
 //     addresses agrees), oldest request first, up to kMaxBatch per batch;
 //   - admits a batch when its workspace fits the context's HBM budget,
-//     evicting idle cached batches first and halving the batch if it still
-//     does not fit; a request that cannot fit even alone fails with
-//     CBP_ERR_BUDGET;
+//     evicting idle cached batches first (also where the device itself is out
+//     of memory) and halving the batch if it still does not fit; a request that
+//     cannot fit even alone fails with CBP_ERR_BUDGET;
 //   - runs each batch on one of kSlots streams as a CUDA graph captured once
 //     per (bucket, batch size) running at a time: the graph owns a fixed
 //     workspace, reads the per-pair addresses from device tables that are
@@ -210,9 +210,12 @@ struct ServeState {
     e->B = B;
     e->plan = p;
     e->bytes = bytes;
-    if (cudaMallocAsync((void**)&e->mem, bytes, s.st) != cudaSuccess) {
+    // The device may be short of memory within the budget (the program's own
+    // tensors): kept batches give theirs back before the request is refused.
+    while (cudaMallocAsync((void**)&e->mem, bytes, s.st) != cudaSuccess) {
       cudaGetLastError();
       e->mem = nullptr;
+      if (evict_one(s.st)) continue;
       ctx->release(bytes);
       delete e;
       return nullptr;

@@ -1,11 +1,17 @@
 """Device memory the serving engine holds, as the allocator counts it (the
 process's default pool, which nothing else here allocates from)."""
 import ctypes
+import os
+import subprocess
+import sys
+from pathlib import Path
 
 import pytest
 import torch
 
 pytestmark = pytest.mark.gpu
+
+ROOT = Path(__file__).resolve().parents[1]
 
 RESERVED_NOW, RESERVED_HIGH, USED_NOW = 5, 6, 7      # cudaMemPoolAttrReservedMemCurrent, -High, UsedMemCurrent
 
@@ -91,3 +97,51 @@ def test_room_for_a_new_shape_while_another_batch_runs(pool):
         torch.cuda.synchronize()
         assert high <= before
         assert pool.used() == base
+
+
+# cudaMallocAsync that fails as often as it is told to, then passes through
+SHIM = """
+#define _GNU_SOURCE
+#include <dlfcn.h>
+#include <stddef.h>
+static int left;
+void fail_next(int n) { left = n; }
+int cudaMallocAsync(void** p, size_t bytes, void* stream) {
+  if (left > 0) { --left; return 2; }   /* cudaErrorMemoryAllocation */
+  int (*real)(void**, size_t, void*) = 0;
+  void* h = dlopen("libcudart.so.13", RTLD_LAZY | RTLD_NOLOAD);
+  *(void**)&real = dlsym(h, "cudaMallocAsync");
+  return real(p, bytes, stream);
+}
+"""
+CHILD = """
+import ctypes, sys
+from tests.test_serving_memory_gpu import request, submit, wait
+from paper_1203_4874_gb300 import cbp
+shim = ctypes.CDLL(sys.argv[1])
+ctx = cbp.cbp_create(0)
+for h in (100, 120, 140):
+    assert wait(ctx, submit(ctx, request(h, 160))) >= 0
+out = []
+for fails in (1, 2, 50, 0):
+    shim.fail_next(fails)
+    out.append(wait(ctx, submit(ctx, request(180 + fails, 160))))
+    shim.fail_next(0)
+cbp.cbp_destroy(ctx)
+print(*out)
+"""
+
+
+def test_device_out_of_memory(built_lib, tmp_path):
+    """Allocations that fail within the budget: kept batches are given up until
+    one succeeds; with none left the request is refused, and the next one runs."""
+    from paper_1203_4874_gb300 import cbp
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    src, lib = tmp_path / "shim.c", tmp_path / "shim.so"
+    src.write_text(SHIM)
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(lib), str(src), "-ldl"], check=True)
+    r = subprocess.run([sys.executable, "-c", CHILD, str(lib)], cwd=ROOT, capture_output=True, text=True,
+                       timeout=300, env=dict(os.environ, LD_PRELOAD=str(lib)))
+    assert r.returncode == 0, r.stderr[-3000:]
+    assert [int(x) for x in r.stdout.split()] == [0, 0, cbp.CBP_ERR_BUDGET, 0]
