@@ -1737,7 +1737,8 @@ void launch_scale_solve(const Plan& p, char* ws, void* k1_out, void* k2_out, int
   // kernel's static arrays (M = 28 with t1 + t2 = 42 or 43, M = 29 with 27 and
   // M = 30 with 11 or 12 fit the device's limit only without them)
   const size_t ff_end = scale_ff_offset(p.M, p.nn) + scale_ff_bytes(p.M, p.nn);
-  a.ffx = p.mixed && p.scale_mode != kScaleSupport && ff_end <= allow_smem((const void*)k_scale_solve);
+  const size_t room = allow_smem((const void*)k_scale_solve);
+  a.ffx = p.mixed && p.scale_mode != kScaleSupport && ff_end <= room;
   const size_t sm = a.ffx ? ff_end : scale_solve_smem(p.M, p.nn);
   k_scale_solve<<<p.n, kSolveThreads, sm, st>>>(a);
 }
