@@ -33,9 +33,6 @@ template <typename T> __host__ __device__ __forceinline__ void cfmac(cpx<T>& acc
   acc.re = fma(a.re, b.re, fma(a.im, b.im, acc.re));
   acc.im = fma(a.re, b.im, fma(-a.im, b.re, acc.im));
 }
-template <typename D, typename S> __host__ __device__ __forceinline__ cpx<D> cvt(cpx<S> a) {
-  return {(D)a.re, (D)a.im};
-}
 
 // A complex double held as two float-float numbers (hi + lo each), for
 // extended-precision arithmetic on the single-precision units.
@@ -82,10 +79,6 @@ template <typename T> __device__ __forceinline__ T warp_max(T v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
-}
-
-template <typename T> __device__ __forceinline__ T ld_elem(const void* p, int64_t i) {
-  return (T)(((const T*)p)[i]);
 }
 
 // Base address of frame f of a batch: from the table if present, else strided.

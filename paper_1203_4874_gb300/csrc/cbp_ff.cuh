@@ -75,8 +75,6 @@ __device__ __forceinline__ fx fx_div(fx a, fx b) {
   const float r = (((a.hi - p) - pe) + a.lo) - q1 * b.lo;   // a - q1 b
   return fx_norm(q1, __fdividef(r, b.hi));
 }
-__device__ __forceinline__ fx fx_ldexp(fx a, int e) { return {ldexpf(a.hi, e), ldexpf(a.lo, e)}; }
-__device__ __forceinline__ float fx_abs_hi(fx a) { return fabsf(a.hi); }
 __device__ __forceinline__ bool fx_neg_sign(fx a) { return a.hi < 0.f || (a.hi == 0.f && a.lo < 0.f); }
 __device__ __forceinline__ bool fx_is_zero(fx a) { return a.hi == 0.f && a.lo == 0.f; }
 

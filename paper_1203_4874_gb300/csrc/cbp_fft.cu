@@ -277,11 +277,6 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc, int
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gsrc), "r"(src_bytes)
                : "memory");
 }
-template <int B>
-__device__ __forceinline__ void cp_async_small(void* smem_dst, const void* gsrc) {   // B = 4 or 8
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(s), "l"(gsrc), "n"(B) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {

@@ -30,20 +30,17 @@ template <typename T> __device__ __forceinline__ T im_(cpx<T> x) { return x.im; 
 template <typename E, typename R> __device__ __forceinline__ E mk_e(R re, R im);
 template <> __device__ __forceinline__ double mk_e<double, double>(double re, double) { return re; }
 template <> __device__ __forceinline__ cd mk_e<cd, double>(double re, double im) { return mk(re, im); }
-template <> __device__ __forceinline__ cf mk_e<cf, float>(float re, float im) { return mk(re, im); }
 __device__ __forceinline__ double mul_(double a, double b) { return a * b; }
 template <typename T> __device__ __forceinline__ cpx<T> mul_(cpx<T> a, cpx<T> b) { return a * b; }
 __device__ __forceinline__ double sc_(double s, double a) { return s * a; }
 template <typename T> __device__ __forceinline__ cpx<T> sc_(T s, cpx<T> a) { return s * a; }
 __device__ __forceinline__ void fma_(cf& acc, cf a, cf b) { cfma(acc, a, b); }
-__device__ __forceinline__ cf warp_sum_e(cf v) { return mk(warp_sum(v.re), warp_sum(v.im)); }
 // real scalar type of an element type
 template <typename E> struct RealOf { using type = E; };
 template <typename T> struct RealOf<cpx<T>> { using type = T; };
 // reflector element -> vector element
 __device__ __forceinline__ cd to_v(double x, cd) { return mk(x, 0.0); }
 __device__ __forceinline__ cd to_v(cd x, cd) { return x; }
-__device__ __forceinline__ cf to_v(cf x, cf) { return x; }
 
 // Per-warp work area.
 struct TriWs {
@@ -61,7 +58,6 @@ struct TriWs {
   int* piv;       // [n] 1 where rows k and k + 1 were interchanged
   float* df;      // [n] d in single precision
   float* e2f;     // [n] e^2 in single precision
-  int* iv;        // [4] values broadcast to the CTA
   void* part;     // [8][n] complex: per-warp partial sums of the CTA's reduction
   cd* x;          // [n] the eigenvector of G
   cd* r;          // [n] residual
@@ -73,7 +69,7 @@ struct TriWs {
 // (placed back to back) and each of its 16-byte-aligned parts stay aligned.
 __host__ __device__ inline size_t tri_ws_bytes(int n) {
   const size_t b = (size_t)16 * ((size_t)n * n + 3 * n) + (size_t)8 * 7 * n + (size_t)4 * 3 * n +
-                   16 + (size_t)16 * 4 * n + (size_t)16 * 8 * n + 16 * 19;   // + alignment of the 19 parts
+                   (size_t)16 * 4 * n + (size_t)16 * 8 * n + 16 * 20;   // + alignment of the parts
   return (b + 127) & ~size_t(127);
 }
 
@@ -101,7 +97,6 @@ __device__ inline TriWs carve_tri(char* p, int n) {
   W.piv = (int*)take((size_t)4 * n);
   W.df = (float*)take((size_t)4 * n);
   W.e2f = (float*)take((size_t)4 * n);
-  W.iv = (int*)take(16);
   W.part = take((size_t)16 * 8 * n);
   return W;
 }
@@ -330,7 +325,6 @@ __device__ __forceinline__ double rsqrt_safe(double x) {
 __device__ __forceinline__ double clamp_pivot(double x, double tiny) {
   return fabs(x) >= tiny ? x : (dneg(x) ? -tiny : tiny);
 }
-__device__ __forceinline__ float rcp_safe(float x) { return 1.0f / x; }
 __device__ __forceinline__ float clamp_pivot(float x, float tiny) {
   return fabsf(x) >= tiny ? x : (x < 0.f ? -tiny : tiny);
 }
