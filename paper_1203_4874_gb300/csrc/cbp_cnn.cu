@@ -7,13 +7,14 @@
 //   softmax over each output channel's 15 x 15 logits -> K1, K2.
 // Activations are stored as bfloat16, a position's channels side by side
 // ([pair][position][channel]; the gradients of the hidden layers likewise in
-// float32), and weights kept as float32 master copies.  The forward convolutions run on the tensor cores (tcgen05, BF16
-// operands with the weights rounded to BF16, FP32 accumulation in tensor
-// memory) as implicit GEMMs over 128 output positions per CTA; the backward
-// pass (training only) stays on the FP32 units with the float32 weights, a
-// thread per output and weight gradients reduced in a fixed order
-// (deterministic).  Training minimises the mean squared error of both
-// kernels with AdamW (decoupled weight decay).
+// float32), and weights kept as float32 master copies.  The convolutions, and in
+// training the gradients of their inputs and weights, run on the tensor cores
+// (tcgen05, BF16 operands, FP32 accumulation in tensor memory) as implicit GEMMs:
+// forward and input gradients 128 positions per CTA with the weights rounded to
+// BF16, weight gradients a chunk of positions per CTA, reduced in a fixed order
+// (deterministic).  Bias gradients are FP32 sums of the unrounded gradients.
+// Training minimises the mean squared error of both kernels with AdamW (decoupled
+// weight decay) on the master copies.
 #include <cuda_bf16.h>
 #include <cstdio>
 #include <cstring>

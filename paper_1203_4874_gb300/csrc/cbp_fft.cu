@@ -1730,9 +1730,14 @@ int row_blocks(int h, int planes, int nbr) {
 // the slots (two an SM), or a first wave and up to 1/8 of a second.  Together
 // against apart, us: a 64 x 64 FP64 pair (10 blocks) 23.6 / 12.6, a 480p pair
 // (22) 39 / 22, four 1000 x 1300 pairs (72) 299 / 196, seven 1080p pairs (126)
-// 154 / 117, two 720p colour pairs (204) 86 / 79; three ragged 720p colour pairs
-// (234) 116 / 118; 15 480p pairs (330) 87 / 76; four 480p colour pairs (408)
-// 61 / 68, seven 720p ones (714) 212 / 241.
+// 154 / 117, two 720p colour pairs (204) 86 / 79; then seven 1080p pairs (238)
+// 119 / 131, eight 720p pairs (272) 90 / 110.  Past the first wave: 14 480p pairs
+// (308) 90 / 73, four 720p colour pairs (312) 175 / 141, 17 1080p pairs (306)
+// 338 / 265, ten 1000 x 1300 pairs (340) 353 / 310; 240 x 320 pairs break even (36.8
+// / 37.1 at 312, 47.2 / 47.3 at 342).  The gain fades from there: (374) 17 480p pairs
+// 90 / 93, 11 1080p pairs 199 / 185, 13 1080p pairs (442) 201 / 218.  Past the second
+// wave it stays below a tenth and is lost on the smaller frames: 28 480p pairs
+// (616) 136 / 130, 29 (638) 137 / 141, 26 1080p pairs (676, 13 / 11 kernels) 379 / 408.
 int row_split(int h, int M, int planes, int fft_planes) {
   constexpr int kSlots = 304;
   const int blocks = M * planes;

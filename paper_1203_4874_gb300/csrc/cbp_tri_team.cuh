@@ -1,7 +1,6 @@
 // Smallest eigenpair of a Hermitian (or real symmetric) n x n matrix, n <= 64,
-// by a team of four warps -- one per scheduler of the SM -- for the solves that
-// have a CTA to themselves: the real samples, the scale system of every pair,
-// and the complex samples of small batches.  The method is cbp_tri.cuh's
+// by a team of four warps -- one per scheduler of the SM: every sample's null
+// vector and every pair's scale system.  The method is cbp_tri.cuh's
 // (tridiagonal T, Sturm counts, inverse iteration, Newton steps in Olsen's
 // form); this file arranges it for latency.
 //
@@ -985,8 +984,9 @@ __device__ __forceinline__ void tri_bounds(const TriWs& W, int n, double eps, do
   team_bar();
 }
 
-// Steps 1-4 in double precision (E = cd or double) by the team; FFR (real samples of the mixed path): from T on in float-float,
-// the reflectors' copies overwriting the double ones in place.  Fills res, S.gs,
+// Steps 1-4 in double precision (E = cd or double) by the team; FFR (real samples
+// of the mixed path, up to kFloatFloatN unknowns): from T on in float-float, the
+// reflectors' copies overwriting the double ones in place.  Fills res, S.gs,
 // S.tnorm; returns the number of refinement steps to take.
 template <typename E, bool FFR>
 __device__ int tri_solve_team(const TriWs& W, TeamWs& S, const cd* G, int n, int steps_far,
