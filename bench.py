@@ -96,8 +96,8 @@ def fp32_peak_tflops(sm_mhz: float) -> float:
 # headers its kernels' code comes from).
 _COMMON = ["cbp_common.cuh", "cbp_internal.h"]
 STAGE_FILES = {"eval": ["cbp_eval.cu"] + _COMMON,
-               "sample_solve": ["cbp_solve.cu", "cbp_tri.cuh", "cbp_ff.cuh"] + _COMMON,
-               "scale_solve": ["cbp_solve.cu", "cbp_tri.cuh", "cbp_ff.cuh"] + _COMMON,
+               "sample_solve": ["cbp_solve.cu", "cbp_tri.cuh", "cbp_tri_team.cuh", "cbp_ff.cuh"] + _COMMON,
+               "scale_solve": ["cbp_solve.cu", "cbp_tri.cuh", "cbp_tri_team.cuh", "cbp_ff.cuh"] + _COMMON,
                "kernel_spectra": ["cbp_fft.cu", "cbp_dft.cuh"] + _COMMON,
                "row_fft": ["cbp_fft.cu", "cbp_dft.cuh"] + _COMMON,
                "col_deconv": ["cbp_colpass.cu", "cbp_dft.cuh"] + _COMMON,

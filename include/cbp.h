@@ -52,16 +52,17 @@ typedef enum cbp_status {
 typedef enum cbp_dtype { CBP_F32 = 0, CBP_F64 = 1 } cbp_dtype;
 
 /* Arithmetic of the kernel-estimation path.
- *   FP64:  evaluation, Gram and per-sample solves in double precision (the
- *          per-sample eigen-solve runs in single precision and is refined to
- *          double precision against the double-precision Gram and two
- *          exact-residual steps).  Deconvolution in the frames' dtype.
- *   MIXED: evaluation with single-precision arithmetic (float frames are
- *          folded with an exact hi + lo float accumulation, samples kept in
- *          double); Gram of the samples other than z = 1 in single precision;
- *          eigen-solves in single precision refined in double precision (one
- *          exact-residual step); scale fix in double precision;
- *          deconvolution in single precision.
+ *   FP64:  evaluation, Gram and eigen-solves in double precision, one
+ *          exact-residual step a sample.  Deconvolution in the frames' dtype.
+ *   MIXED: evaluation on the single-precision units (float frames are folded
+ *          with an exact hi + lo float accumulation, samples kept as float-float
+ *          pairs of ~48 bits); Gram of the complex samples in float-float, of the
+ *          real ones (z = 1, z = -1) in double; complex samples' eigen-solves in
+ *          single precision refined against the double Gram, in double where
+ *          single precision does not separate the two smallest eigenvalues; real
+ *          samples' in double up to the tridiagonal form, then in float-float
+ *          (t1 + t2 < 40) or double, with one exact-residual step; scale fix in
+ *          float-float or double; deconvolution in single precision.
  *   LEARNED: a network proposal checked by the consistency residual, falling
  *          back to MIXED (see cbp_learned_*). */
 typedef enum cbp_path { CBP_PATH_FP64 = 0, CBP_PATH_MIXED = 1, CBP_PATH_LEARNED = 2 } cbp_path;
